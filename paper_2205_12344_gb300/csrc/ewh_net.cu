@@ -1,121 +1,24 @@
 // Layers of the learned warm start (a small convolutional encoder-decoder that
 // maps medium, forcing and frequency to an initial guess for the CG solve of
-// M (I - S) v = M Pi 0): 3x3 convolutions as implicit GEMMs on the BF16 tensor
-// cores with FP32 accumulation, their data and weight gradients, and the small
-// element-wise layers.  Activations are NHWC with channel counts that are
+// M (I - S) v = M Pi 0): the entry points of the 3x3 convolutions and their
+// gradients (kernels in ewh_conv.cu) and the small element-wise layers.  Activations are NHWC with channel counts that are
 // multiples of 16; weights are [Co][3][3][Ci].  The paper has no learned part:
 // these kernels serve the precision/warm-start forms of the solver.
+#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
 #include <string>
 
 #include "../../include/ewh.h"
+#include "ewh_conv.cuh"
 #include "ewh_internal.cuh"
 
 namespace {
 
 using bf16 = __nv_bfloat16;
 
-// D (16x8 f32) += A (16x16 bf16, row) * B (16x8 bf16, col)
-__device__ __forceinline__ void mma_bf16_16816(float* d, const unsigned* a, const unsigned* b) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
-      "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
-__device__ __forceinline__ unsigned ld32(const bf16* p) { return *reinterpret_cast<const unsigned*>(p); }
-
 constexpr float LEAK = 0.1f;
-
-// ---------------------------------------------------------------------------
-// Forward 3x3 convolution, zero padding, stride 1.
-// CTA: 64 pixels (one image row segment) x 64 output channels, 4 warps; warp w
-// owns pixels 16w..16w+15 and all 64 channels (8 mma tiles of n = 8).  The K
-// loop walks (ky, kx, 16-channel chunk); each step stages a 64x16 A tile (the
-// im2col gather) and a 16x64 B tile in shared memory.
-// ---------------------------------------------------------------------------
-constexpr int CF_PIX = 64, CF_CO = 64, CF_KS = 16, CF_LD = 24;  // LD: padded row length (bf16)
-
-__global__ void __launch_bounds__(128) conv3x3_fwd_kernel(const bf16* __restrict__ x, const bf16* __restrict__ w,
-                                                          const float* __restrict__ bias, float* __restrict__ y_pre,
-                                                          bf16* __restrict__ y_act, int act, int N, int H, int W,
-                                                          int Ci, int Co) {
-  __shared__ __align__(16) bf16 sA[CF_PIX][CF_LD];
-  __shared__ __align__(16) bf16 sB[CF_CO][CF_LD];
-  const int wx_tiles = (W + CF_PIX - 1) / CF_PIX;
-  const int tile = blockIdx.x;
-  const int n = tile / (H * wx_tiles);
-  const int rem = tile - n * H * wx_tiles;
-  const int yrow = rem / wx_tiles;
-  const int x0 = (rem - yrow * wx_tiles) * CF_PIX;
-  const int co0 = blockIdx.y * CF_CO;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int gid = lane >> 2, tig = lane & 3;
-  float acc[8][4];
-#pragma unroll
-  for (int j = 0; j < 8; ++j)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[j][q] = 0.f;
-  const int nck = Ci / CF_KS;
-  for (int ky = 0; ky < 3; ++ky) {
-    const int yy = yrow + ky - 1;
-    for (int kx = 0; kx < 3; ++kx) {
-      for (int ck = 0; ck < nck; ++ck) {
-        const int ci0 = ck * CF_KS;
-        // A: 64 pixels x 16 channels, two 16-byte pieces per pixel
-        for (int i = tid; i < CF_PIX * 2; i += 128) {
-          const int p = i >> 1, half = i & 1;
-          const int xx = x0 + p + kx - 1;
-          uint4 v = make_uint4(0, 0, 0, 0);
-          if (yy >= 0 && yy < H && xx >= 0 && xx < W && x0 + p < W)
-            v = *reinterpret_cast<const uint4*>(x + (((long long)n * H + yy) * W + xx) * Ci + ci0 + half * 8);
-          *reinterpret_cast<uint4*>(&sA[p][half * 8]) = v;
-        }
-        // B: 64 output channels x 16 input channels
-        for (int i = tid; i < CF_CO * 2; i += 128) {
-          const int c = i >> 1, half = i & 1;
-          uint4 v = make_uint4(0, 0, 0, 0);
-          if (co0 + c < Co)
-            v = *reinterpret_cast<const uint4*>(w + (((long long)(co0 + c) * 3 + ky) * 3 + kx) * Ci + ci0 + half * 8);
-          *reinterpret_cast<uint4*>(&sB[c][half * 8]) = v;
-        }
-        __syncthreads();
-        unsigned a[4];
-        const int r0 = warp * 16 + gid;
-        a[0] = ld32(&sA[r0][tig * 2]);
-        a[1] = ld32(&sA[r0 + 8][tig * 2]);
-        a[2] = ld32(&sA[r0][tig * 2 + 8]);
-        a[3] = ld32(&sA[r0 + 8][tig * 2 + 8]);
-#pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          unsigned b[2];
-          b[0] = ld32(&sB[j * 8 + gid][tig * 2]);
-          b[1] = ld32(&sB[j * 8 + gid][tig * 2 + 8]);
-          mma_bf16_16816(acc[j], a, b);
-        }
-        __syncthreads();
-      }
-    }
-  }
-  // epilogue: bias, optional leaky ReLU; c0,c1 at row gid, c2,c3 at row gid+8
-#pragma unroll
-  for (int j = 0; j < 8; ++j) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int p = warp * 16 + gid + (q >= 2 ? 8 : 0);
-      const int c = co0 + j * 8 + tig * 2 + (q & 1);
-      const int xx = x0 + p;
-      if (xx >= W || c >= Co) continue;
-      float v = acc[j][q] + (bias ? bias[c] : 0.f);
-      const long long o = (((long long)n * H + yrow) * W + xx) * Co + c;
-      if (y_pre) y_pre[o] = v;
-      if (y_act) y_act[o] = __float2bfloat16(act == 1 ? (v > 0.f ? v : LEAK * v) : v);
-    }
-  }
-}
 
 // weights [Co][3][3][Ci] -> flipped/transposed [Ci][3][3][Co] (for the data gradient)
 __global__ void flip_transpose_kernel(const bf16* __restrict__ w, bf16* __restrict__ wt, int Ci, int Co) {
@@ -130,99 +33,77 @@ __global__ void flip_transpose_kernel(const bf16* __restrict__ w, bf16* __restri
 }
 
 // ---------------------------------------------------------------------------
-// Weight gradient: dw[co][ky][kx][ci] = sum_p dy[p][co] x[p shifted][ci].
-// CTA: 64 co x 64 ci for one (ky, kx) and one chunk of pixels (split K);
-// partial sums are added into the FP32 result with atomics.  A = dy^T (co x
-// pixels), B = shifted x (pixels x ci), K step = 16 pixels.
-// ---------------------------------------------------------------------------
-constexpr int WG_PIX_CHUNK = 1024;
-
-__global__ void __launch_bounds__(128) conv3x3_wgrad_kernel(const bf16* __restrict__ x, const bf16* __restrict__ dy,
-                                                            float* __restrict__ dw, int N, int H, int W, int Ci,
-                                                            int Co) {
-  __shared__ __align__(16) bf16 sA[64][CF_LD];  // [co][pixel]
-  __shared__ __align__(16) bf16 sB[64][CF_LD];  // [ci][pixel]
-  const int k9 = blockIdx.x % 9;
-  const int ky = k9 / 3, kx = k9 % 3;
-  const int ci_tiles = (Ci + 63) / 64;
-  const int co0 = (blockIdx.x / 9 / ci_tiles) * 64;
-  const int ci0 = ((blockIdx.x / 9) % ci_tiles) * 64;
-  const long long P = (long long)N * H * W;
-  const long long p_begin = (long long)blockIdx.y * WG_PIX_CHUNK;
-  const long long p_end = p_begin + WG_PIX_CHUNK < P ? p_begin + WG_PIX_CHUNK : P;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int gid = lane >> 2, tig = lane & 3;
-  // warp tile: 16 co (rows) x 64 ci (8 n-tiles)
-  float acc[8][4];
-#pragma unroll
-  for (int j = 0; j < 8; ++j)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) acc[j][q] = 0.f;
-  for (long long pb = p_begin; pb < p_end; pb += 16) {
-    // stage dy[p][co0..co0+63] transposed into sA[co][p], and the shifted x
-    for (int i = tid; i < 16 * 64; i += 128) {
-      const int pl = i / 64, c = i % 64;
-      const long long p = pb + pl;
-      bf16 vdy = __float2bfloat16(0.f), vx = __float2bfloat16(0.f);
-      if (p < p_end) {
-        if (co0 + c < Co) vdy = dy[p * Co + co0 + c];
-        const int n = (int)(p / ((long long)H * W));
-        const int r = (int)(p - (long long)n * H * W);
-        const int yy = r / W + ky - 1, xx = r % W + kx - 1;
-        if (ci0 + c < Ci && yy >= 0 && yy < H && xx >= 0 && xx < W)
-          vx = x[(((long long)n * H + yy) * W + xx) * Ci + ci0 + c];
-      }
-      sA[c][pl] = vdy;
-      sB[c][pl] = vx;
-    }
-    __syncthreads();
-    unsigned a[4];
-    const int r0 = warp * 16 + gid;
-    a[0] = ld32(&sA[r0][tig * 2]);
-    a[1] = ld32(&sA[r0 + 8][tig * 2]);
-    a[2] = ld32(&sA[r0][tig * 2 + 8]);
-    a[3] = ld32(&sA[r0 + 8][tig * 2 + 8]);
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      unsigned b[2];
-      b[0] = ld32(&sB[j * 8 + gid][tig * 2]);
-      b[1] = ld32(&sB[j * 8 + gid][tig * 2 + 8]);
-      mma_bf16_16816(acc[j], a, b);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int j = 0; j < 8; ++j)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int co = co0 + warp * 16 + gid + (q >= 2 ? 8 : 0);
-      const int ci = ci0 + j * 8 + tig * 2 + (q & 1);
-      if (co < Co && ci < Ci) atomicAdd(&dw[(((long long)co * 3 + ky) * 3 + kx) * Ci + ci], acc[j][q]);
-    }
-}
-
-// ---------------------------------------------------------------------------
 // Element-wise layers
 // ---------------------------------------------------------------------------
-__global__ void bias_grad_kernel(const float* __restrict__ dy, float* __restrict__ db, long long P, int C) {
-  // one block per channel; fixed-order block reduction
-  __shared__ float part[256];
-  const int c = blockIdx.x;
+// db[c] = sum over pixels of dy[p][c].  A cluster of CTAs takes 8 channels (one
+// 32-byte sector of every pixel), each CTA every gridDim.y-th run of 128 pixels;
+// its first CTA adds the others' sums from their shared memory, in rank order,
+// so the result does not depend on timing.  Bound by memory: one block per channel
+// read each sector 8 times on 32 SMs (267 us for 524288 x 32; this one 20 us).
+constexpr int BG_THREADS = 1024, BG_CH = 8, BG_PIX = BG_THREADS / BG_CH;
+constexpr int BG_CLUSTER = 16;           // CTAs per cluster for long sums
+constexpr long long BG_LONG = 16384;     // pixels from which the cluster pays
+__global__ void __launch_bounds__(BG_THREADS) bias_grad_kernel(const float* __restrict__ dy, float* __restrict__ db,
+                                                               long long P, int C) {
+  __shared__ float warp_part[BG_THREADS / 32][BG_CH];
+  __shared__ float cta_part[BG_CH];
+  const int c0 = blockIdx.x * BG_CH, c = c0 + (int)(threadIdx.x % BG_CH);
   float s = 0.f;
-  for (long long p = threadIdx.x; p < P; p += 256) s += dy[p * C + c];
-  part[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = 128; o > 0; o >>= 1) {
-    if (threadIdx.x < o) part[threadIdx.x] += part[threadIdx.x + o];
-    __syncthreads();
+  if (c < C) {
+    const long long step = (long long)gridDim.y * BG_PIX;
+    long long p = (long long)blockIdx.y * BG_PIX + threadIdx.x / BG_CH;
+    const float* q = dy + p * C + c;
+    for (; p + 7 * step < P; p += 8 * step, q += 8 * step * C) {  // eight loads in flight
+      float v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = __ldg(q + k * step * C);
+      s += ((v[0] + v[1]) + (v[2] + v[3])) + ((v[4] + v[5]) + (v[6] + v[7]));
+    }
+    for (; p < P; p += step, q += step * C) s += __ldg(q);
   }
-  if (threadIdx.x == 0) db[c] = part[0];
+  s += __shfl_xor_sync(0xffffffffu, s, 16);
+  s += __shfl_xor_sync(0xffffffffu, s, 8);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane < BG_CH) warp_part[warp][lane] = s;
+  __syncthreads();
+  if (threadIdx.x < BG_CH) {
+    float t = 0.f;
+    for (int w = 0; w < BG_THREADS / 32; ++w) t += warp_part[w][threadIdx.x];
+    cta_part[threadIdx.x] = t;
+  }
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  if (cl.block_rank() == 0 && threadIdx.x < BG_CH && c0 + (int)threadIdx.x < C) {
+    float t = 0.f;
+    for (unsigned r = 0; r < cl.num_blocks(); ++r) t += cl.map_shared_rank(cta_part, r)[threadIdx.x];
+    db[c0 + threadIdx.x] = t;
+  }
+  cl.sync();  // the other CTAs' shared memory stays until it is read
 }
 
+__device__ __forceinline__ float leaky_grad(float pre, float dy) { return pre > 0.f ? dy : LEAK * dy; }
+
+// vec: every pointer 16-byte (8-byte for the BF16 one) aligned; four values a
+// thread and pass then (bound by memory: 14 bytes a value)
 __global__ void leaky_bwd_kernel(const float* __restrict__ pre, const float* __restrict__ dy, float* __restrict__ dx,
-                                 bf16* __restrict__ dx_bf, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const float g = pre[i] > 0.f ? dy[i] : LEAK * dy[i];
+                                 bf16* __restrict__ dx_bf, long long n, int vec) {
+  const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x, nt = (long long)gridDim.x * blockDim.x;
+  const long long n4 = vec ? n / 4 : 0;
+  for (long long i = t; i < n4; i += nt) {
+    const float4 a = __ldcs(reinterpret_cast<const float4*>(pre) + i), d = __ldcs(reinterpret_cast<const float4*>(dy) + i);
+    const float4 g = make_float4(leaky_grad(a.x, d.x), leaky_grad(a.y, d.y), leaky_grad(a.z, d.z), leaky_grad(a.w, d.w));
+    if (dx) reinterpret_cast<float4*>(dx)[i] = g;
+    if (dx_bf) {
+      const __nv_bfloat162 lo = __floats2bfloat162_rn(g.x, g.y), hi = __floats2bfloat162_rn(g.z, g.w);
+      uint2 u;
+      u.x = *reinterpret_cast<const unsigned*>(&lo);
+      u.y = *reinterpret_cast<const unsigned*>(&hi);
+      reinterpret_cast<uint2*>(dx_bf)[i] = u;
+    }
+  }
+  for (long long i = 4 * n4 + t; i < n; i += nt) {
+    const float g = leaky_grad(pre[i], dy[i]);
     if (dx) dx[i] = g;
     if (dx_bf) dx_bf[i] = __float2bfloat16(g);
   }
@@ -356,8 +237,9 @@ ewh_status nfail(const char* msg) {
   return EWH_EINVAL;
 }
 
-ewh_status launched() {
-  const cudaError_t e = cudaGetLastError();
+ewh_status launched(cudaError_t e = cudaSuccess) {
+  const cudaError_t pending = cudaGetLastError();
+  if (e == cudaSuccess) e = pending;
   if (e != cudaSuccess) {
     ewh::set_global_error(std::string("warm-start kernel launch failed: ") + cudaGetErrorString(e));
     return EWH_ECUDA;
@@ -373,11 +255,7 @@ ewh_status ewh_conv3x3_fwd(const void* x, const void* w, const float* bias, floa
                            int H, int W, int Ci, int Co, void* stream) {
   if (!x || !w || (!y_pre && !y_act) || N < 1 || H < 1 || W < 1 || Ci < 16 || Ci % 16 || Co < 8 || Co % 8)
     return nfail("ewh_conv3x3_fwd: bad arguments (Ci multiple of 16, Co multiple of 8)");
-  const int wx = (W + CF_PIX - 1) / CF_PIX;
-  dim3 grid((unsigned)(N * H * wx), (unsigned)((Co + CF_CO - 1) / CF_CO));
-  conv3x3_fwd_kernel<<<grid, 128, 0, (cudaStream_t)stream>>>((const bf16*)x, (const bf16*)w, bias, y_pre,
-                                                             (bf16*)y_act, act, N, H, W, Ci, Co);
-  return launched();
+  return launched(ewh::launch_conv3x3(x, w, bias, y_pre, y_act, act, N, H, W, Ci, Co, (cudaStream_t)stream));
 }
 
 ewh_status ewh_conv3x3_dgrad(const void* dy, const void* w, void* w_scratch, float* dx, int N, int H, int W, int Ci,
@@ -386,11 +264,7 @@ ewh_status ewh_conv3x3_dgrad(const void* dy, const void* w, void* w_scratch, flo
     return nfail("ewh_conv3x3_dgrad: bad arguments (Ci, Co multiples of 16)");
   cudaStream_t st = (cudaStream_t)stream;
   flip_transpose_kernel<<<egrid(9LL * Ci * Co), 256, 0, st>>>((const bf16*)w, (bf16*)w_scratch, Ci, Co);
-  const int wx = (W + CF_PIX - 1) / CF_PIX;
-  dim3 grid((unsigned)(N * H * wx), (unsigned)((Ci + CF_CO - 1) / CF_CO));
-  conv3x3_fwd_kernel<<<grid, 128, 0, st>>>((const bf16*)dy, (const bf16*)w_scratch, nullptr, dx, nullptr, 0, N, H, W,
-                                           Co, Ci);
-  return launched();
+  return launched(ewh::launch_conv3x3(dy, w_scratch, nullptr, dx, nullptr, 0, N, H, W, Co, Ci, st));
 }
 
 ewh_status ewh_conv3x3_wgrad(const void* x, const void* dy, float* dw, int N, int H, int W, int Ci, int Co,
@@ -399,22 +273,32 @@ ewh_status ewh_conv3x3_wgrad(const void* x, const void* dy, float* dw, int N, in
     return nfail("ewh_conv3x3_wgrad: bad arguments (Ci, Co multiples of 16)");
   cudaStream_t st = (cudaStream_t)stream;
   cudaMemsetAsync(dw, 0, sizeof(float) * 9LL * Ci * Co, st);
-  const long long P = (long long)N * H * W;
-  const int ci_t = (Ci + 63) / 64, co_t = (Co + 63) / 64;
-  dim3 grid((unsigned)(9 * ci_t * co_t), (unsigned)((P + WG_PIX_CHUNK - 1) / WG_PIX_CHUNK));
-  conv3x3_wgrad_kernel<<<grid, 128, 0, st>>>((const bf16*)x, (const bf16*)dy, dw, N, H, W, Ci, Co);
-  return launched();
+  return launched(ewh::launch_conv3x3_wgrad(x, dy, dw, N, H, W, Ci, Co, st));
 }
 
 ewh_status ewh_bias_grad(const float* dy, float* db, long long P, int C, void* stream) {
   if (!dy || !db || P < 1 || C < 1) return nfail("ewh_bias_grad: bad arguments");
-  bias_grad_kernel<<<C, 256, 0, (cudaStream_t)stream>>>(dy, db, P, C);
-  return launched();
+  const int cs = P >= BG_LONG ? BG_CLUSTER : 1;
+  cudaError_t e = cudaFuncSetAttribute(bias_grad_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  if (e != cudaSuccess) return launched(e);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)((C + BG_CH - 1) / BG_CH), (unsigned)cs);
+  cfg.blockDim = dim3(BG_THREADS);
+  cfg.stream = (cudaStream_t)stream;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = 1;
+  attr[0].val.clusterDim.y = cs;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return launched(cudaLaunchKernelEx(&cfg, bias_grad_kernel, dy, db, P, C));
 }
 
 ewh_status ewh_leaky_relu_bwd(const float* pre, const float* dy, float* dx, void* dx_bf16, long long n, void* stream) {
   if (!pre || !dy || (!dx && !dx_bf16) || n < 0) return nfail("ewh_leaky_relu_bwd: bad arguments");
-  leaky_bwd_kernel<<<egrid(n), 256, 0, (cudaStream_t)stream>>>(pre, dy, dx, (bf16*)dx_bf16, n);
+  const int vec = ((uintptr_t)pre | (uintptr_t)dy | (uintptr_t)dx) % 16 == 0 && (uintptr_t)dx_bf16 % 8 == 0;
+  leaky_bwd_kernel<<<egrid(vec ? n / 4 : n), 256, 0, (cudaStream_t)stream>>>(pre, dy, dx, (bf16*)dx_bf16, n, vec);
   return launched();
 }
 
