@@ -755,8 +755,9 @@ static cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, cud
 
 // 2D order-4 kernel variants (Geom::variant, chosen per context by the
 // autotuner): 0..3 = stress + divergence launches with 32x8, 32x16, 64x8 or
-// 64x4 blocks, 4 = single fused launch, YM_VARIANT = the FP32 y-march
-// (ewh_ymarch.cu).  EWH_STEP2D_O4=fused|split|ym overrides it (read whenever
+// 64x4 blocks (FP64: 0 = 32x8, FX_VARIANT + shape = the block-fixed-point step,
+// ewh_fx2d.cu), 4 = single fused launch, YM_VARIANT = the FP32 y-march
+// (ewh_ymarch.cu).  EWH_STEP2D_O4=fused|split|ym|fx overrides it (read whenever
 // launches are enqueued; a context captures its step graph once, on first use).
 // Mapped 2D grids: 0 = fused curv_step2d with 32x8 outputs per block, 1 =
 // curv_stress2d + curv_div2d, 2 = fused with 32x16 outputs (FP32; FP64 runs 32x8).  Geom::variant
@@ -770,7 +771,7 @@ static int curv_variant(const Geom& g) {
 
 static int step2d_o4_variant(const Geom& g) {
   const char* e = getenv("EWH_STEP2D_O4");
-  if (e && e[0] == 'f') return 1;
+  if (e && e[0] == 'f' && e[1] != 'x') return 1;
   if (e && e[0] == 's') return 0;
   return g.variant == 4 ? 1 : 0;
 }
@@ -1159,6 +1160,18 @@ static cudaError_t launch_mode(const Geom& g, int order, const WaveFields<T>& f,
       return cudaGetLastError();
     }
   }
+  if constexpr (sizeof(T) == 8 && MODE != 3) {
+    // fused block-fixed-point step: autotuner variants FX_VARIANT + shape; EWH_STEP2D_O4=fx|fx1 forces one
+    const char* ev = getenv("EWH_STEP2D_O4");
+    int shape = g.variant - FX_VARIANT;
+    if (ev) shape = (ev[0] == 'f' && ev[1] == 'x') ? (ev[2] == '1' ? 1 : 0) : -1;
+    if (g.dim == 2 && !g.contrast && shape >= 0 && shape < FX_SHAPES) {
+      cudaError_t e = launch_fx2d(g, shape, f, (StepMode)MODE, s, st);
+      if (e != cudaSuccess) return e;
+      if (nl) *nl += 1;
+      return cudaGetLastError();
+    }
+  }
   if (g.dim == 2 && step2d_o4_variant(g) == 1) {
     constexpr int TY = o4_tile_y<T>();
     dim3 blk(32, TY), grd((g.n[0] + 31) / 32, (g.n[1] + TY - 1) / TY, g.nrhs);
@@ -1170,11 +1183,16 @@ static cudaError_t launch_mode(const Geom& g, int order, const WaveFields<T>& f,
   dim3 blk(32, 8);
   dim3 grd((g.n[0] + 31) / 32, (g.n[1] + 7) / 8, g.dim == 2 ? g.nrhs : g.n[2] * g.nrhs);
   if (g.dim == 2) {
-    const int tv = step2d_o4_tile(g);
-    cudaError_t e = tv == 1   ? launch_split_o4<T, MODE, FORCED, 32, 16>(g, f, s, st)
-                    : tv == 2 ? launch_split_o4<T, MODE, FORCED, 64, 8>(g, f, s, st)
-                    : tv == 3 ? launch_split_o4<T, MODE, FORCED, 64, 4>(g, f, s, st)
-                              : launch_split_o4<T, MODE, FORCED, 32, 8>(g, f, s, st);
+    cudaError_t e;
+    if constexpr (sizeof(T) == 8) {
+      e = launch_split_o4<T, MODE, FORCED, 32, 8>(g, f, s, st);
+    } else {
+      const int tv = step2d_o4_tile(g);
+      e = tv == 1   ? launch_split_o4<T, MODE, FORCED, 32, 16>(g, f, s, st)
+          : tv == 2 ? launch_split_o4<T, MODE, FORCED, 64, 8>(g, f, s, st)
+          : tv == 3 ? launch_split_o4<T, MODE, FORCED, 64, 4>(g, f, s, st)
+                    : launch_split_o4<T, MODE, FORCED, 32, 8>(g, f, s, st);
+    }
     if (e != cudaSuccess) return e;
   } else {
     if constexpr (sizeof(T) == 4 && MODE != 3) {
