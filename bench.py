@@ -463,8 +463,8 @@ ALG_BYTES_3D = {"fp32": 72.0, "fp64": 144.0}      # read u, u_prev, acc + write 
 
 
 KERNELS_3D = {0: "sbp_stress + sbp_divergence_step (3D, per level)",
-              1: "step3d_o4_zm<16> (fused z-march, 32x16 tiles, per level)",
-              2: "step3d_o4_zm<8> (fused z-march, 32x8 tiles, per level)",
+              1: "step3d_o4_zm<64, 8> (fused z-march, 64x8 tiles, per level)",
+              2: "step3d_o4_zm<32, 8> (fused z-march, 32x8 tiles, per level)",
               "fp64": "sbp_stress + sbp_divergence_step (3D, per level; FP64 has no fused z-march)"}
 
 

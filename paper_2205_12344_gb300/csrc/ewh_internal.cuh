@@ -51,7 +51,7 @@ constexpr double SBP_CLOSURE[4][6] = {{-24.0 / 17, 59.0 / 34, -4.0 / 17, -3.0 / 
 inline int step_variant_count(int dim, int order) {
   if (dim == 2 && order == 4) return 5;  // split with 4 block shapes (FP64: one, and 2 fixed-point tiles), fused
   if (dim == 2 && order == 2) return 3;  // tile heights 8, 4, 16
-  if (dim == 3 && order == 4) return 3;  // stress + divergence pair, fused z-march 32x16 and 32x8 (FP32)
+  if (dim == 3 && order == 4) return 3;  // stress + divergence pair, fused z-march 64x8 and 32x8 (FP32)
   return 1;
 }
 
@@ -87,7 +87,7 @@ enum StepMode { STEP_FIRST = 0, STEP_MID = 1, STEP_LAST = 2 };
 // Plan of the fused marching FP32 order-4 steps: bulk-tensor maps of both u
 // buffers, the persistent grid and the control words (wait limit in ns at
 // [2..3] as a u64, give-up count at [4]).
-// 3D z-march (ewh_zmarch.cu), shapes k = 0 tiles of 32 x 16 nodes (one CTA
+// 3D z-march (ewh_zmarch.cu), shapes k = 0 tiles of 64 x 8 nodes (one CTA
 // per SM), k = 1 tiles of 32 x 8 (two CTAs per SM); 2D y-march
 // (ewh_ymarch.cu), slot 0: strips of 60 columns, one warp per CTA.
 constexpr int ZM_MAP_BYTES = 128;

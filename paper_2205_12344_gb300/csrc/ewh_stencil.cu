@@ -1196,8 +1196,8 @@ static cudaError_t launch_mode(const Geom& g, int order, const WaveFields<T>& f,
     if (e != cudaSuccess) return e;
   } else {
     if constexpr (sizeof(T) == 4 && MODE != 3) {
-      // fused z-march: autotuner variants 1 (32 x 16 tiles) and 2 (32 x 8);
-      // EWH_STEP3D_O4=pair|zm16|zm8 (zm: 32 x 8) overrides it
+      // fused z-march: autotuner variants 1 (64 x 8 tiles) and 2 (32 x 8);
+      // EWH_STEP3D_O4=pair|zm16|zm8 (zm16: 64 x 8, else 32 x 8) overrides it
       const char* ev = getenv("EWH_STEP3D_O4");
       int zk = g.variant == 1 ? 0 : (g.variant == 2 ? 1 : -1);
       if (ev) zk = ev[0] != 'z' ? -1 : (strcmp(ev, "zm16") == 0 ? 0 : 1);

@@ -6,28 +6,35 @@
 // (pointwise energy density with fourth-order diagonal-norm SBP first
 // derivatives D; the stresses sigma = lambda div u I + mu (grad u + grad u^T)).
 //
-// Each CTA owns tiles of 32 x TY unknown columns and walks them plane by
-// plane.  Per plane it
-//   - receives u^n (3 components) on the tile +- 4 nodes in x and y through a
-//     bulk-tensor (TMA) load issued two planes ahead into a ring of 8 plane
-//     buffers in shared memory, completed on one mbarrier per buffer;
-//   - forms the stresses, scaled by 12 (12 D from unscaled central
-//     differences or 12x closure rows), on the tile +- 2 nodes: the in-plane
-//     components (xx, yy, xy, xz, yz) into a plane buffer, (xz, yz, zz) of
-//     the own nodes into a ring of 8 planes;
-//   - forms the in-plane part of -D sigma + H^{-1} B sigma of the own nodes
-//     into a ring of 6 pending planes;
-//   - and, for every output plane whose z stencil is complete, adds the z
-//     part and applies the leapfrog/filter update (8-byte loads and stores of
-//     node pairs; the operands of the next output plane are requested one
-//     plane ahead).
+// Each CTA owns tiles of TX x 8 unknown columns (TX = 64: one CTA of 12 warps per
+// SM, TX = 32: two of 6) and walks them plane by plane.  A thread holds a pair of
+// nodes adjacent along x, computed with packed FP32 instructions.  Per plane s it
+//   - waits for the u planes that the stresses of plane s read: bulk-tensor (TMA)
+//     loads of the tile +- 4 nodes in x and y into a ring of 8 plane buffers, one
+//     mbarrier each;
+//   - forms the stresses, scaled by 12 (12 D from unscaled central differences or
+//     12x closure rows), on the tile +- 2 nodes: the own rows by the own warps,
+//     the rows above and below by the halo warps, the pairs to the left and right
+//     by a second pass of the first of these; xx, yy, xy, xz, yz go into one of two
+//     plane buffers, so that one barrier per plane is enough;
+//   - after it forms the in-plane part of -D sigma + H^{-1} B sigma of the own
+//     nodes and adds the plane's z stresses, still in registers, to the pending
+//     sums of the outputs s - 2 .. s + 2 (the central difference along z, by
+//     column instead of by row: four packed instructions per component and no
+//     ring of stress planes);
+//   - completes output plane s - 2 with the leapfrog/filter update (8-byte loads
+//     and stores; the operands are requested ahead of the barrier).
 // Only u^n, delta, acc, lambda, mu, 1/(rho h^2) (and f/rho) are read and only
-// delta, u^{n+1} and acc written: the stresses never leave the chip.  Near
-// the z sides the SBP closure rows reach up to 3 planes, so each stress plane
-// is formed as soon as every u plane it reads has arrived and each output
-// plane as soon as every stress plane it reads exists (the exact reach of
-// each row of D); the ring depths hold for every z range of grids with at
-// least 10 planes.
+// delta, u^{n+1} and acc written: the stresses never leave the chip, except for
+// the six planes next to each z side, which the outputs on z closure rows (the
+// first and last four) read back: every thread keeps its own column of them in
+// the stress scratch field.
+//
+// 256^3: 571 us per level (0.31 of the copy rate in the 72-byte count), against
+// 790 us with rings of z stresses and in-plane sums in shared memory.  Bound by
+// latency: 12 warps of 168 registers per SM issue 0.33 instructions per clock and
+// scheduler; 96 registers and 18 warps spill (815 us), and with the shared memory
+// taken a spill goes to L2.
 //
 // The grid is persistent: the (rhs, tile, plane) work is split into equal
 // contiguous shares, one per CTA, each a few (tile, z range) segments.
@@ -49,40 +56,34 @@ namespace ewh {
 
 namespace {
 
-constexpr int ZM_TX = 32;    // own nodes per tile along x
-constexpr int ZM_UX = 40;    // u tile row: x from X0 - 4 (the bulk-tensor box width)
-constexpr int ZM_SX = 36;    // stress tile row: x from X0 - 2
-constexpr int ZM_RU = 8;     // u plane ring
-constexpr int ZM_RS = 8;     // (xz, yz, zz) stress ring of the own nodes
-constexpr int ZM_RP = 6;     // pending in-plane divergence ring
-constexpr int ZM_PREF = 2;   // u planes requested ahead of the march
+constexpr int ZM_RU = 8;  // u plane ring: planes s - 3 .. s + 3 of the current stress plane s, and one in flight
+static_assert((ZM_RU & (ZM_RU - 1)) == 0, "ring index by mask");
 
-
-
-template <int TY>
+template <int TX, int TY>
 struct ZmLayout {
-  static constexpr int NT = 18 * (TY + 4);   // one stress-tile pair per thread
-  static constexpr int UY = TY + 8;
-  static constexpr int SY = TY + 4;
-  static constexpr int UPLANE = UY * ZM_UX;   // one component of one u plane (floats)
+  static constexpr int PW = TX / 2;                  // pairs per row
+  static constexpr int RPW = 32 / PW;                // rows per warp
+  static constexpr int NWO = TY / RPW;               // warps of the own rows,
+  static constexpr int NWY = 4 / RPW;                // of the 2 + 2 halo rows,
+  static_assert(2 * TY <= 32, "the left and right halo pairs are one more pass of the first halo warp");
+  static constexpr int NT = 32 * (NWO + NWY);
+  static constexpr int UX = TX + 8, UY = TY + 8;     // u tile: x from X0 - 4 (the bulk-tensor box), y from Y0 - 4
+  static constexpr int SX = TX + 4, SY = TY + 4;     // stress tile: from X0 - 2, Y0 - 2
+  static constexpr int UPLANE = UX * UY;             // one component of one u plane (floats)
   static constexpr int USLOT = 3 * UPLANE;
-  static constexpr int OWN = TY * ZM_TX;
-  static constexpr int SPLANE = SY * ZM_SX;   // one in-plane stress component
-  static constexpr int OFF_SZ = ZM_RU * USLOT;
-  static constexpr int OFF_PD = OFF_SZ + ZM_RS * 3 * OWN;
-  static constexpr int OFF_SIP = OFF_PD + ZM_RP * 3 * OWN;
-  static constexpr int OFF_TAB = OFF_SIP + 5 * SPLANE;
-  static constexpr int OFF_CLS = OFF_TAB + 24;              // tap offsets (int) then weights, per class
+  static constexpr int SPLANE = SX * SY;             // one in-plane stress component
+  static constexpr int SBUF = 5 * SPLANE;            // xx, yy, xy, xz, yz; two buffers
+  static constexpr int OFF_SIP = ZM_RU * USLOT;
+  static constexpr int OFF_CLS = OFF_SIP + 2 * SBUF;        // tap offsets (int) then weights, per class
   static constexpr int FLOATS = OFF_CLS + 8 * ZM_CLASSES;   // even: the mbarriers follow, 8-byte aligned
   static constexpr size_t BYTES = 128 + sizeof(float) * FLOATS + sizeof(uint64_t) * ZM_RU;
   static constexpr unsigned TX_BYTES = sizeof(float) * USLOT;  // one bulk-tensor box
   static_assert(USLOT % 32 == 0, "u ring slots stay 128-byte aligned");
-  static_assert(FLOATS % 2 == 0, "mbarrier alignment");
+  static_assert(FLOATS % 2 == 0 && SBUF % 2 == 0 && UPLANE % 2 == 0, "8-byte pairs and mbarriers");
   static_assert(OFF_CLS % 4 == 0, "16-byte table rows");
 };
 
 struct ZmScalars {
-  float tab12[24];  // 12 x SBP_CLOSURE
   float kt144;      // c dt^2 / 144
   float w0, wnew;   // trapezoid weights of level 0 (first level only) and of the new level
   float fcos144;    // 144 cos(w t_n)
@@ -95,22 +96,42 @@ struct ZmScalars {
   float tcf[4 * ZM_CLASSES];
 };
 
-// Stresses (scaled by 12) at one node from its nine scaled derivatives
-// d[c][a] = 12 D_a u_c; out: xx, yy, zz, xy, xz, yz.
-__device__ __forceinline__ void zm_sigma(const float d[3][3], float l, float m, float s[6]) {
-  const float div = d[0][0] + d[1][1] + d[2][2];
-  const float m2 = 2.0f * m;
-  s[0] = l * div + m2 * d[0][0];
-  s[1] = l * div + m2 * d[1][1];
-  s[2] = l * div + m2 * d[2][2];
-  s[3] = m * (d[0][1] + d[1][0]);
-  s[4] = m * (d[0][2] + d[2][0]);
-  s[5] = m * (d[1][2] + d[2][1]);
+// ---- pairs: two FP32 values per instruction ----------------------------------
+__device__ __forceinline__ uint64_t p2(float2 v) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(v.x), "f"(v.y));
+  return r;
 }
-
-struct ZmOperands {  // update operands of one own node pair at one output plane
-  float2 d[3], a[3], f[3], irh;
-};
+__device__ __forceinline__ float2 f2(uint64_t v) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+  return r;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(p2(a)), "l"(p2(b)));
+  return f2(r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(p2(a)), "l"(p2(b)));
+  return f2(r);
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(p2(a)), "l"(p2(b)), "l"(p2(c)));
+  return f2(r);
+}
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, both(-1.0f), a); }
+// 12 D of a pair across rows or planes: (m2 - p2) + 8 (p1 - m1)
+__device__ __forceinline__ float2 c4p(float2 m2, float2 m1, float2 p1, float2 q2) {
+  return fma2(both(8.0f), sub2(p1, m1), sub2(m2, q2));
+}
+// 12 D of the pair b along x, from the pairs before and after it
+__device__ __forceinline__ float2 c4x(float2 a, float2 b, float2 e) {
+  return fma2(both(8.0f), make_float2(b.y - a.y, e.x - b.x), sub2(a, e));
+}
 
 // Offset of node (x, y) of plane 0 in one padded component (32 bits: a
 // component holds fewer than 2^31 nodes); plane z adds z * Geom::plane.
@@ -118,91 +139,215 @@ __device__ __forceinline__ int zm_off(const Geom& g, int x, int y) {
   return g.pz * (int)g.plane + (y + PAD) * g.np[0] + x + g.padx;
 }
 
-// Update operands of the own pair at component offset o (node pair o, o + 1;
-// v0, v1: which of them are unknowns); D, A, R: delta, acc and f/rho of this
+struct ZmOperands {  // update operands of one own node pair at one output plane
+  float2 d[3], a[3], f[3], irh;
+};
+
+// Element access at a 32-bit byte offset from a base that is the same for the
+// whole warp: one instruction, no 64-bit address arithmetic (a component is
+// below 4 GB: plan_zmarch).
+template <class V>
+__device__ __forceinline__ V* zm_at(const float* base, unsigned bytes) {
+  return reinterpret_cast<V*>(reinterpret_cast<char*>(const_cast<float*>(base)) + bytes);
+}
+
+// Update operands of the own pair at byte offset o of a component (full: both
+// nodes are unknowns; else v0, v1); D, A, R: delta, acc and f/rho of this
 // right-hand side, F the component stride.
-template <bool FORCED>
-__device__ __forceinline__ void zm_load_ops(const float* D, const float* A, const float* R, const float* irh2, int o,
-                                            int F, bool v0, bool v1, ZmOperands& op) {
-  if (v0 && v1) {  // 8-byte aligned: x - off[0] and the padded row start are even
+template <int MODE, bool FORCED>
+__device__ __forceinline__ void zm_load_ops(const float* D, const float* A, const float* R, const float* irh2,
+                                            unsigned o, long long F, bool full, bool v0, bool v1, ZmOperands& op) {
+  if (full) {  // 8-byte aligned: x - off[0] and the padded row start are even
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      op.d[c] = __ldcs(reinterpret_cast<const float2*>(D + o + c * F));
-      op.a[c] = __ldcs(reinterpret_cast<const float2*>(A + o + c * F));
-      if (FORCED) op.f[c] = __ldg(reinterpret_cast<const float2*>(R + o + c * F));
+      if (MODE != STEP_FIRST) {
+        op.d[c] = __ldcs(zm_at<const float2>(D + c * F, o));
+        op.a[c] = __ldcs(zm_at<const float2>(A + c * F, o));
+      }
+      if (FORCED) op.f[c] = __ldg(zm_at<const float2>(R + c * F, o));
     }
-    op.irh = __ldg(reinterpret_cast<const float2*>(irh2 + o));
+    op.irh = __ldg(zm_at<const float2>(irh2, o));
   } else {
+    auto ld = [&](const float* b) {
+      return make_float2(v0 ? *zm_at<const float>(b, o) : 0.f, v1 ? *zm_at<const float>(b, o + 4) : 0.f);
+    };
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      op.d[c] = make_float2(v0 ? D[o + c * F] : 0.f, v1 ? D[o + c * F + 1] : 0.f);
-      op.a[c] = make_float2(v0 ? A[o + c * F] : 0.f, v1 ? A[o + c * F + 1] : 0.f);
-      if (FORCED) op.f[c] = make_float2(v0 ? R[o + c * F] : 0.f, v1 ? R[o + c * F + 1] : 0.f);
+      if (MODE != STEP_FIRST) op.d[c] = ld(D + c * F), op.a[c] = ld(A + c * F);
+      if (FORCED) op.f[c] = ld(R + c * F);
     }
-    op.irh = make_float2(v0 ? irh2[o] : 0.f, v1 ? irh2[o + 1] : 0.f);
+    op.irh = ld(irh2);
   }
 }
 
-// lambda, mu at the stress pair at component offset o (zero outside the grid;
-// g0, g1: which nodes lie in it)
-__device__ __forceinline__ void zm_load_lm(const float* lam, const float* mu, int o, bool g0, bool g1, float2& l,
-                                           float2& m) {
-  if (g0 && g1) {  // padded x even: 8-byte aligned
-    l = __ldg(reinterpret_cast<const float2*>(lam + o));
-    m = __ldg(reinterpret_cast<const float2*>(mu + o));
+// lambda, mu at the stress pair at byte offset o (zero outside the grid; full:
+// both nodes lie in it, else g0, g1)
+__device__ __forceinline__ void zm_load_lm(const float* lam, const float* mu, unsigned o, bool full, bool g0, bool g1,
+                                           float2& l, float2& m) {
+  if (full) {  // padded x even: 8-byte aligned
+    l = __ldg(zm_at<const float2>(lam, o));
+    m = __ldg(zm_at<const float2>(mu, o));
     return;
   }
   l = m = make_float2(0.f, 0.f);
-  if (g0) l.x = __ldg(lam + o), m.x = __ldg(mu + o);
-  if (g1) l.y = __ldg(lam + o + 1), m.y = __ldg(mu + o + 1);
+  if (g0) l.x = __ldg(zm_at<const float>(lam, o)), m.x = __ldg(zm_at<const float>(mu, o));
+  if (g1) l.y = __ldg(zm_at<const float>(lam, o + 4)), m.y = __ldg(zm_at<const float>(mu, o + 4));
+}
+
+// Leapfrog / filter update (increment form) of the own pair at byte offset p
+// of a component from k = 144 h^2 rho M^{-1} K u; u of the pair at Us
+// (component stride us).
+template <int MODE, bool FORCED>
+__device__ __forceinline__ void zm_update(const ZmScalars& sc, const ZmOperands& op, const float2 k[3], const float* Us,
+                                          int us, float* D, float* A, float* U, unsigned p, long long F, bool full,
+                                          bool v0, bool v1) {
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const float2 u = ld2(Us + c * us);
+    float2 a = mul2(k[c], op.irh);
+    if (FORCED) a = fma2(op.f[c], both(sc.fcos144), a);
+    float2 d, ac;
+    if (MODE == STEP_FIRST) d = mul2(both(-0.5f * sc.kt144), a);
+    else d = fma2(both(-sc.kt144), a, op.d[c]);
+    const float2 un = add2(u, d);
+    if (MODE == STEP_FIRST) ac = fma2(both(sc.w0), u, mul2(both(sc.wnew), un));
+    else ac = fma2(both(sc.wnew), un, op.a[c]);
+    auto st = [&](float* b, float2 v) {
+      if (full) {
+        __stcs(zm_at<float2>(b, p), v);
+      } else {
+        if (v0) *zm_at<float>(b, p) = v.x;
+        if (v1) *zm_at<float>(b, p + 4) = v.y;
+      }
+    };
+    if (MODE != STEP_LAST) st(D + c * F, d), st(U + c * F, un);
+    st(A + c * F, ac);
+  }
+}
+
+// 12 D along x of the pair at v (8-byte aligned), class taps per node
+__device__ __forceinline__ float2 zm_tap_pair_x(const float* v, int c0, int c1, const int* toff, const float* tcf) {
+  return make_float2(zm_d12t(v, 1, c0, toff, tcf), zm_d12t(v + 1, 1, c1, toff, tcf));
+}
+__device__ __forceinline__ float2 zm_tap_pair_y(const float* v, int stride, int c, const int* toff, const float* tcf) {
+  return make_float2(zm_d12t(v, stride, c, toff, tcf), zm_d12t(v + 1, stride, c, toff, tcf));
 }
 
 __device__ __forceinline__ bool zm_unknown_x(const Geom& g, int x) { return x >= g.off[0] && x < g.off[0] + g.nu[0]; }
 __device__ __forceinline__ bool zm_unknown_y(const Geom& g, int y) { return y >= g.off[1] && y < g.off[1] + g.nu[1]; }
 
-// Every thread owns one pair of the stress tile (18 pairs x TY + 4 rows);
-// the threads whose pair lies in the own tile also update those two nodes.
-template <int TY>
-constexpr int zm_threads() { return 18 * (TY + 4); }
+// A pair of stress nodes (x, x + 1) of row y: which lie in the grid, and the
+// SBP classes along x and y.
+struct ZmPair {
+  bool g0, g1;
+  int c0, c1, cy;
+  __device__ __forceinline__ ZmPair(const Geom& g, int x, int y) {
+    const bool in = y >= 0 && y < g.n[1];
+    g0 = in && x >= 0 && x < g.n[0];
+    g1 = in && x + 1 >= 0 && x + 1 < g.n[0];
+    c0 = zm_class(x, g.n[0]);
+    c1 = zm_class(x + 1, g.n[0]);
+    cy = zm_class(y, g.n[1]);
+  }
+};
 
-template <int TY, int MODE, bool FORCED>
-__global__ void __launch_bounds__(zm_threads<TY>(), TY <= 8 ? 2 : 1)
+// 12 sigma at a pair of plane s (u ring at sm, pair at offset uo of a plane)
+// into the in-plane buffer at offset ps; returns (xz, yz, zz).  lambda = mu = 0
+// outside the grid.
+template <class L>
+__device__ __forceinline__ void zm_stress(const float* sm, float* sip, int uo, int ps, int s, bool zin, int n2,
+                                          const ZmPair& p, bool wx, bool wy, float2 l, float2 m, const int* toff,
+                                          const float* tcf, float2 out_z[3]) {
+  const float* const U0 = sm + (s & (ZM_RU - 1)) * L::USLOT + uo;
+  float2 dx[3], dy[3], dz[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const float* Uc = U0 + c * L::UPLANE;
+    dx[c] = wx ? zm_tap_pair_x(Uc, p.c0, p.c1, toff, tcf) : c4x(ld2(Uc - 2), ld2(Uc), ld2(Uc + 2));
+    dy[c] = wy ? zm_tap_pair_y(Uc, L::UX, p.cy, toff, tcf)
+               : c4p(ld2(Uc - 2 * L::UX), ld2(Uc - L::UX), ld2(Uc + L::UX), ld2(Uc + 2 * L::UX));
+  }
+  if (zin) {  // uniform per plane
+    const float* const M2 = sm + ((s - 2) & (ZM_RU - 1)) * L::USLOT + uo;
+    const float* const M1 = sm + ((s - 1) & (ZM_RU - 1)) * L::USLOT + uo;
+    const float* const P1 = sm + ((s + 1) & (ZM_RU - 1)) * L::USLOT + uo;
+    const float* const P2 = sm + ((s + 2) & (ZM_RU - 1)) * L::USLOT + uo;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const int o = c * L::UPLANE;
+      dz[c] = c4p(ld2(M2 + o), ld2(M1 + o), ld2(P1 + o), ld2(P2 + o));
+    }
+  } else {
+    const int cz = zm_class(s, n2);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) dz[c] = make_float2(0.f, 0.f);
+    for (int q = 0; q < 4; ++q) {
+      const float* const P = sm + ((s + toff[4 * cz + q]) & (ZM_RU - 1)) * L::USLOT + uo;
+      const float2 wq = both(tcf[4 * cz + q]);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) dz[c] = fma2(wq, ld2(P + c * L::UPLANE), dz[c]);
+    }
+  }
+  const float2 ld = mul2(l, add2(add2(dx[0], dy[1]), dz[2])), m2 = add2(m, m);
+  const float2 sxx = fma2(m2, dx[0], ld), syy = fma2(m2, dy[1], ld), sxy = mul2(m, add2(dy[0], dx[1]));
+  out_z[0] = mul2(m, add2(dz[0], dx[2]));
+  out_z[1] = mul2(m, add2(dz[1], dy[2]));
+  out_z[2] = fma2(m2, dz[2], ld);
+  float* const S = sip + ps;
+  st2(S, sxx.x, sxx.y);
+  st2(S + L::SPLANE, syy.x, syy.y);
+  st2(S + 2 * L::SPLANE, sxy.x, sxy.y);
+  st2(S + 3 * L::SPLANE, out_z[0].x, out_z[0].y);
+  st2(S + 4 * L::SPLANE, out_z[1].x, out_z[1].y);
+}
+
+template <int TX, int TY>
+constexpr int zm_ctas() { return TX * TY <= 256 ? 2 : 1; }
+
+template <int TX, int TY, int MODE, bool FORCED>
+__global__ void __launch_bounds__(ZmLayout<TX, TY>::NT, zm_ctas<TX, TY>())
     step3d_o4_zm(Geom g, WaveFields<float> f, ZmScalars sc, unsigned* ctl, const __grid_constant__ CUtensorMap tmu) {
-  using L = ZmLayout<TY>;
+  using L = ZmLayout<TX, TY>;
   extern __shared__ unsigned char zm_raw[];
   // 128-byte aligned base; offsetting the shared array itself (rather than an
   // integer round trip) keeps every access below in the shared address space
   float* const sm = reinterpret_cast<float*>(zm_raw + ((128u - (smem_u32(zm_raw) & 127u)) & 127u));
   uint64_t* const bar = reinterpret_cast<uint64_t*>(sm + L::FLOATS);
-  float* const tab = sm + L::OFF_TAB;
-  float* const sip = sm + L::OFF_SIP;
-  const int t = threadIdx.x;
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
   int* const toff = reinterpret_cast<int*>(sm + L::OFF_CLS);
   float* const tcf = sm + L::OFF_CLS + 4 * ZM_CLASSES;
   if (t == 0) {  // static indices: the parameter arrays stay in the constant bank
-#pragma unroll
-    for (int k = 0; k < 24; ++k) tab[k] = sc.tab12[k];
 #pragma unroll
     for (int k = 0; k < 4 * ZM_CLASSES; ++k) toff[k] = sc.toff[k], tcf[k] = sc.tcf[k];
     for (int k = 0; k < ZM_RU; ++k) mbar_init(bar + k, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  // this thread's stress pair: nodes (X0 + 2 pi, + 1), row Y0 + ri
+  const bool own = warp < L::NWO;
+  int pi = lane % L::PW, ri;
+  if (own) {
+    ri = warp * L::RPW + lane / L::PW;
+  } else {
+    const int k = (warp - L::NWO) * L::RPW + lane / L::PW;  // rows -2, -1, TY, TY + 1
+    ri = k < 2 ? k - 2 : TY + k - 2;
+  }
+  const int uo = (ri + 4) * L::UX + 4 + 2 * pi;  // of the pair in a u plane
+  const int ps = (ri + 2) * L::SX + 2 + 2 * pi;  // ... in a stress plane
+  // the first halo warp takes the left and right halo pairs of the own rows in a second pass
+  const bool two = warp == L::NWO, xside = two && lane < 2 * TY;
+  const int xpi = (lane & 1) ? L::PW : -1, xri = lane >> 1;
   __syncthreads();
   zm_pdl_wait();
   zm_pdl_trigger();
   const unsigned long long wait_ns = *reinterpret_cast<const volatile unsigned long long*>(ctl + 2);
 
   const int n0 = g.n[0], n1 = g.n[1], n2 = g.n[2];
-  const int ntx = (g.nu[0] + sc.shx + ZM_TX - 1) / ZM_TX, nty = (g.nu[1] + sc.shy + TY - 1) / TY, nz = g.nu[2];
+  const int ntx = (g.nu[0] + sc.shx + TX - 1) / TX, nty = (g.nu[1] + sc.shy + TY - 1) / TY, nz = g.nu[2];
   const long long W = (long long)ntx * nty * nz * g.nrhs;
   const long long wbeg = W * blockIdx.x / gridDim.x, wend = W * (blockIdx.x + 1) / gridDim.x;
-  // this thread's stress-tile pair (nodes X0 - 2 + 2 pi, + 1; row Y0 - 2 + ri) and,
-  // when it lies in the own tile, its own pair (i, r)
-  const int pi = t % 18, ri = t / 18;
-  const bool own = pi >= 1 && pi <= 16 && ri >= 2 && ri < TY + 2;
-  const int i = pi - 1, r = ri - 2;
-  const int F = (int)g.field;
+  const long long F = g.field;
+  const unsigned PL4 = 4u * (unsigned)g.plane;  // bytes of a plane
   const float BT = sc.bt12;
   unsigned phase = 0;  // parity of the next completion of each u slot's mbarrier
   bool alive = true;
@@ -216,334 +361,173 @@ __global__ void __launch_bounds__(zm_threads<TY>(), TY <= 8 ? 2 : 1)
     w += zcount;
     const int rhs = (int)(tile / (ntx * nty));
     const int tt = (int)(tile - (long long)rhs * ntx * nty);
-    const int X0 = g.off[0] - sc.shx + ZM_TX * (tt % ntx), Y0 = g.off[1] - sc.shy + TY * (tt / ntx);
+    const int X0 = g.off[0] - sc.shx + TX * (tt % ntx), Y0 = g.off[1] - sc.shy + TY * (tt / ntx);
     const int za = g.off[2] + zi, zb = za + zcount;
     // stress planes [slo, shi] the outputs read; u planes [ulo, uhi] those read
     const int slo = min(zm_lo(za, n2), zm_lo(zb - 1, n2)), shi = max(zm_hi(za, n2), zm_hi(zb - 1, n2));
     const int ulo = min(zm_lo(slo, n2), zm_lo(shi, n2)), uhi = max(zm_hi(slo, n2), zm_hi(shi, n2));
-    const int hs0 = zm_hi(slo, n2), ho0 = zm_hi(za, n2);
     // bulk-tensor coordinates of the u box (padded x is a multiple of 4: Geom::padx)
     const int cx = X0 - 4 + g.padx, cy = Y0 - 4 + PAD, cc = 3 * rhs;
+    int issued = min(uhi, slo + 3);  // last u plane requested
     __syncthreads();  // every read of the rings by the previous segment is done
     if (t == 0) {
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-      for (int k = ulo; k <= uhi && k < ulo + ZM_PREF; ++k)
+      for (int k = ulo; k <= issued; ++k)
         zm_issue(&tmu, sm + (k & (ZM_RU - 1)) * L::USLOT, bar + (k & (ZM_RU - 1)), cx, cy, k + g.pz, cc,
                  L::TX_BYTES);
     }
-    // the stress pair of this thread and which of its nodes lie in the grid
-    const int sx = X0 - 2 + 2 * pi, sy = Y0 - 2 + ri;
-    const bool syin = sy >= 0 && sy < n1;
-    const bool sg0 = syin && sx >= 0 && sx < n0, sg1 = syin && sx + 1 >= 0 && sx + 1 < n0;
-    const int cx0 = zm_class(sx, n0), cx1 = zm_class(sx + 1, n0), cy0 = zm_class(sy, n1);
-    // warps with a lane on an SBP closure row redo that axis with the class taps
-    const unsigned am = __activemask();
-    const bool wx = __any_sync(am, cx0 != 4 || cx1 != 4), wy = __any_sync(am, cy0 != 4);
-    // own pair: nodes (ox, ox + 1), row oy
-    const int ox = sx, oy = sy;
-    const bool ov0 = own && zm_unknown_x(g, ox) && zm_unknown_y(g, oy);
-    const bool ov1 = own && zm_unknown_x(g, ox + 1) && zm_unknown_y(g, oy);
-    // component offsets of this thread's pairs at plane 0, and the state of this rhs
-    const int PL = (int)g.plane;
-    const int so = zm_off(g, sx, sy);
+    const int sx = X0 + 2 * pi, sy = Y0 + ri;
+    const bool ov0 = own && zm_unknown_x(g, sx) && zm_unknown_y(g, sy);
+    const bool ov1 = own && zm_unknown_x(g, sx + 1) && zm_unknown_y(g, sy);
+    const bool live = ov0 || ov1;
+    const ZmPair pm(g, sx, sy);
+    // warps with a lane on an SBP closure row take that axis by the class taps
+    const bool wx = __any_sync(0xffffffffu, pm.c0 != 4 || pm.c1 != 4), wy = __any_sync(0xffffffffu, pm.cy != 4);
+    const unsigned so = 4u * (unsigned)zm_off(g, sx, sy);  // byte offset of this thread's pair at plane 0
+    const bool fs = pm.g0 && pm.g1, fo = ov0 && ov1;
     const long long ro = (long long)rhs * 3 * g.field;
-    const float* const Dr = f.delta + ro;
-    const float* const Ar = f.acc + ro;
+    float* const Dr = f.delta + ro;
+    float* const Ar = f.acc + ro;
+    float* const Ur = f.u_next + ro;
     const float* const Rr = FORCED ? f.frho + ro : nullptr;
-    float* const Dw = f.delta + ro;
-    float* const Aw = f.acc + ro;
-    float* const Uw = f.u_next + ro;
-    // lambda, mu of the next stress plane, requested one plane ahead
-    float2 lm_l, lm_m;
-    int lm_plane = slo;
-    zm_load_lm(f.lam, f.mu, so + slo * PL, sg0, sg1, lm_l, lm_m);
-    ZmOperands op;
-    int op_plane = -1;
-    if (ov0 || ov1) {
-      zm_load_ops<FORCED>(Dr, Ar, Rr, f.irh2, so + za * PL, F, ov0, ov1, op);
-      op_plane = za;
-    }
+    // own column of the closure planes near the z sides: z stresses (0..2) and
+    // in-plane sums (3..5), written and read by this thread only
+    float* const Sg = f.sigma + (long long)rhs * 6 * g.field;
+    float2 lm_l, lm_m;  // lambda, mu of the next stress plane, requested one plane ahead
+    zm_load_lm(f.lam, f.mu, so + slo * PL4, fs, pm.g0, pm.g1, lm_l, lm_m);
+    // 144 h^2 rho M^{-1} K u of the outputs s - 2 .. s + 1 as far as planes < s give it
+    float2 A0[3], A1[3], A2[3], A3[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) A0[c] = A1[c] = A2[c] = A3[c] = make_float2(0.f, 0.f);
 
-    int next_s = slo, next_o = za, jfail = uhi + 1;
-    bool wait_bad = false;
-    for (int j = ulo; j <= uhi; ++j) {
-      // ---- wait for u plane j (bounded)
-      {
-        const int k = j & (ZM_RU - 1);
-        const unsigned par = (phase >> k) & 1u;
+    int have = ulo - 1, next_o = za;  // last u plane waited for, next output
+    int s = slo;
+    for (; s <= shi; ++s) {
+      // ---- wait for the u planes that stress plane s reads (bounded)
+      bool bad = false;
+      const int need = max(have, zm_hi(s, n2));
+      for (int k = have + 1; k <= need && !bad; ++k) {
+        const int sl = k & (ZM_RU - 1);
+        const unsigned par = (phase >> sl) & 1u;
         bool ok = wait_ns != 0ull;
-        if (ok && !mbar_try(bar + k, par)) {
+        if (ok && !mbar_try(bar + sl, par)) {
           const unsigned long long t0 = zm_ns();
-          while (!mbar_try(bar + k, par)) {
+          while (!mbar_try(bar + sl, par)) {
             if (zm_ns() - t0 > wait_ns) {
               ok = false;
               break;
             }
           }
         }
-        // no barrier here: the threads agree on a failed wait at the next one
-        if (ok) phase ^= 1u << k;
-        wait_bad = !ok;
+        if (ok) phase ^= 1u << sl, have = k;
+        bad = !ok;
       }
-      // ---- stress planes whose u planes have all arrived
-      bool any_sigma = false, failed = false;
-      // the last stress plane complete at this step: every u plane its prefix of
-      // stress planes reads has arrived (the prefix maximum of the reach is
-      // max(hs0, hi(zs)), non-decreasing in zs)
-      const int s_last = zm_last_ready(next_s, shi, hs0, j, n2);
-      for (; next_s <= s_last;) {
-        const int zs = next_s;
-        if (lm_plane != zs) {
-          zm_load_lm(f.lam, f.mu, so + zs * PL, sg0, sg1, lm_l, lm_m);
-          lm_plane = zs;
+      // ---- 12 sigma at the pair (and at the side pair of the first halo warp)
+      float* const sip = sm + L::OFF_SIP + (s & 1) * L::SBUF;
+      const bool zin = s >= 4 && s <= n2 - 5;
+      float2 own_z[3];
+      zm_stress<L>(sm, sip, uo, ps, s, zin, n2, pm, wx, wy, lm_l, lm_m, toff, tcf, own_z);
+      if (two) {
+        const ZmPair px(g, X0 + 2 * xpi, Y0 + xri);
+        const bool vx = xside && (px.c0 != 4 || px.c1 != 4), vy = xside && px.cy != 4;
+        const bool xx = __any_sync(0xffffffffu, vx), xy = __any_sync(0xffffffffu, vy);
+        if (xside) {
+          float2 xl, xm, unused[3];
+          zm_load_lm(f.lam, f.mu, 4u * (unsigned)zm_off(g, X0 + 2 * xpi, Y0 + xri) + s * PL4, px.g0 && px.g1, px.g0, px.g1,
+                     xl, xm);
+          zm_stress<L>(sm, sip, (xri + 4) * L::UX + 4 + 2 * xpi, (xri + 2) * L::SX + 2 + 2 * xpi, s, zin, n2, px, xx, xy,
+                       xl, xm, toff, tcf, unused);
         }
-        const float* U0 = sm + (zs & (ZM_RU - 1)) * L::USLOT;
-        const bool zin = zs >= 4 && zs <= n2 - 5;
-        const int ly = ri + 2, lx = 2 + 2 * pi;  // u tile position of node sx
-        float d0[3][3], d1[3][3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          // central differences of the pair (8-byte loads; the u tile covers +- 4 around
-          // the stress tile, so they stay in bounds even where a closure replaces them)
-          const int o = c * L::UPLANE + ly * ZM_UX + lx;
-          const float* Uc = U0 + o;
-          const float2 a = ld2(Uc - 2), b = ld2(Uc), e = ld2(Uc + 2);
-          d0[c][0] = c4u(a.x, a.y, b.y, e.x);
-          d1[c][0] = c4u(a.y, b.x, e.x, e.y);
-          const float2 m2 = ld2(Uc - 2 * ZM_UX), m1 = ld2(Uc - ZM_UX), p1 = ld2(Uc + ZM_UX), p2 = ld2(Uc + 2 * ZM_UX);
-          d0[c][1] = c4u(m2.x, m1.x, p1.x, p2.x);
-          d1[c][1] = c4u(m2.y, m1.y, p1.y, p2.y);
-          if (zin) {  // uniform per plane
-            const float2 zm2 = ld2(sm + ((zs - 2) & (ZM_RU - 1)) * L::USLOT + o);
-            const float2 zm1 = ld2(sm + ((zs - 1) & (ZM_RU - 1)) * L::USLOT + o);
-            const float2 zp1 = ld2(sm + ((zs + 1) & (ZM_RU - 1)) * L::USLOT + o);
-            const float2 zp2 = ld2(sm + ((zs + 2) & (ZM_RU - 1)) * L::USLOT + o);
-            d0[c][2] = c4u(zm2.x, zm1.x, zp1.x, zp2.x);
-            d1[c][2] = c4u(zm2.y, zm1.y, zp1.y, zp2.y);
-          } else {
-            d0[c][2] = zm_closure12([&](int k) { return sm[((zs + k) & (ZM_RU - 1)) * L::USLOT + o]; }, zs, n2, tab);
-            d1[c][2] = zm_closure12([&](int k) { return sm[((zs + k) & (ZM_RU - 1)) * L::USLOT + o + 1]; }, zs, n2,
-                                    tab);
-          }
-        }
-        // closure rows along x and y (nodes within 4 of a side): the warps that hold
-        // one redo that axis for every lane with the taps of each lane's class
-        if (wx) {
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const float* Uc = U0 + c * L::UPLANE + ly * ZM_UX + lx;
-            d0[c][0] = zm_d12t(Uc, 1, cx0, toff, tcf);
-            d1[c][0] = zm_d12t(Uc + 1, 1, cx1, toff, tcf);
-          }
-        }
-        if (wy) {
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const float* Uc = U0 + c * L::UPLANE + ly * ZM_UX + lx;
-            d0[c][1] = zm_d12t(Uc, ZM_UX, cy0, toff, tcf);
-            d1[c][1] = zm_d12t(Uc + 1, ZM_UX, cy0, toff, tcf);
-          }
-        }
-        float s0[6], s1[6];
-        zm_sigma(d0, lm_l.x, lm_m.x, s0);
-        zm_sigma(d1, lm_l.y, lm_m.y, s1);
-        if (!sg0) {
-#pragma unroll
-          for (int k = 0; k < 6; ++k) s0[k] = 0.f;
-        }
-        if (!sg1) {
-#pragma unroll
-          for (int k = 0; k < 6; ++k) s1[k] = 0.f;
-        }
-        // in-plane components: xx, yy, xy, xz, yz
-        const int ps = ri * ZM_SX + 2 * pi;
-        st2(sip + ps, s0[0], s1[0]);
-        st2(sip + L::SPLANE + ps, s0[1], s1[1]);
-        st2(sip + 2 * L::SPLANE + ps, s0[3], s1[3]);
-        st2(sip + 3 * L::SPLANE + ps, s0[4], s1[4]);
-        st2(sip + 4 * L::SPLANE + ps, s0[5], s1[5]);
-        if (own) {  // own nodes: (xz, yz, zz) into the ring
-          float* SZ = sm + L::OFF_SZ + (zs & (ZM_RS - 1)) * 3 * L::OWN + r * ZM_TX + 2 * i;
-          st2(SZ, s0[4], s1[4]);
-          st2(SZ + L::OWN, s0[5], s1[5]);
-          st2(SZ + 2 * L::OWN, s0[2], s1[2]);
-        }
-        if (zs + 1 <= shi) {
-          zm_load_lm(f.lam, f.mu, so + (zs + 1) * PL, sg0, sg1, lm_l, lm_m);
-          lm_plane = zs + 1;
-        }
-        if (__syncthreads_or(wait_bad)) {  // the stress plane is complete (or a wait gave up)
-          failed = true;
-          break;
-        }
-        any_sigma = true;
-        if (zs >= za && zs < zb && (ov0 || ov1)) {
-          // in-plane part of -D sigma + H^{-1} B sigma at the own pair: central
-          // differences, then the closure rows and boundary terms of nodes within 4 of
-          // a side
-          float kx0[3], kx1[3], ky0[3], ky1[3];
-          constexpr int CX[3] = {0, 2, 3}, CY[3] = {2, 1, 4};  // planes of sigma_{cx}, sigma_{cy}
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const float* Sx = sip + CX[c] * L::SPLANE + ps;
-            const float2 a = ld2(Sx - 2), b = ld2(Sx), e = ld2(Sx + 2);
-            const float* Sy = sip + CY[c] * L::SPLANE + ps;
-            const float2 m2 = ld2(Sy - 2 * ZM_SX), m1 = ld2(Sy - ZM_SX), p1 = ld2(Sy + ZM_SX), p2 = ld2(Sy + 2 * ZM_SX);
-            kx0[c] = c4u(a.x, a.y, b.y, e.x);
-            kx1[c] = c4u(a.y, b.x, e.x, e.y);
-            ky0[c] = c4u(m2.x, m1.x, p1.x, p2.x);
-            ky1[c] = c4u(m2.y, m1.y, p1.y, p2.y);
-          }
-          float k0[3], k1[3];
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            k0[c] = -(kx0[c] + ky0[c]);
-            k1[c] = -(kx1[c] + ky1[c]);
-          }
-          if (wx || wy) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              const float* Sx = sip + CX[c] * L::SPLANE + ps;
-              const float* Sy = sip + CY[c] * L::SPLANE + ps;
-              if (wx) {
-                kx0[c] = zm_d12t(Sx, 1, cx0, toff, tcf);
-                kx1[c] = zm_d12t(Sx + 1, 1, cx1, toff, tcf);
-              }
-              if (wy) {
-                ky0[c] = zm_d12t(Sy, ZM_SX, cy0, toff, tcf);
-                ky1[c] = zm_d12t(Sy + 1, ZM_SX, cy0, toff, tcf);
-              }
-              // boundary terms H^{-1} B sigma on free sides (nodes on the side itself)
-              float b0 = 0.f, b1 = 0.f;
-              if (ox == 0) b0 -= BT * Sx[0];
-              if (ox == n0 - 1) b0 += BT * Sx[0];
-              if (ox + 1 == n0 - 1) b1 += BT * Sx[1];
-              if (oy == 0) b0 -= BT * Sy[0], b1 -= BT * Sy[1];
-              if (oy == n1 - 1) b0 += BT * Sy[0], b1 += BT * Sy[1];
-              k0[c] = -(kx0[c] + ky0[c]) + b0;
-              k1[c] = -(kx1[c] + ky1[c]) + b1;
-            }
-          }
-          float* PD = sm + L::OFF_PD + (zs % ZM_RP) * 3 * L::OWN + r * ZM_TX + 2 * i;
-#pragma unroll
-          for (int c = 0; c < 3; ++c) st2(PD + c * L::OWN, k0[c], k1[c]);
-        }
-        ++next_s;
-        if (next_s <= s_last) __syncthreads();  // another plane follows
       }
-      if (!any_sigma && !failed) failed = __syncthreads_or(wait_bad) != 0;
-      if (failed) {  // a wait gave up: every thread stops here
+      // operands of the next stress plane and of this step's output, in flight across the barrier
+      if (s + 1 <= shi) zm_load_lm(f.lam, f.mu, so + (s + 1) * PL4, fs, pm.g0, pm.g1, lm_l, lm_m);
+      const int o = s - 2;
+      const bool out = o >= max(za, 4) && o <= min(zb - 1, n2 - 5);
+      ZmOperands op;
+      if (out && live) zm_load_ops<MODE, FORCED>(Dr, Ar, Rr, f.irh2, so + o * PL4, F, fo, ov0, ov1, op);
+      // the stress plane is complete (or a wait gave up: every thread stops);
+      // every read of planes below s - 3 and of the other stress buffer is done
+      if (__syncthreads_or(bad)) {
         alive = false;
-        jfail = j;
         break;
       }
-      // ---- output planes whose stress planes all exist
-      const int o_last = zm_last_ready(next_o, zb - 1, ho0, next_s - 1, n2);
-      for (; next_o <= o_last;) {
-        const int zo = next_o;
-        if (ov0 || ov1) {
-          if (op_plane != zo) zm_load_ops<FORCED>(Dr, Ar, Rr, f.irh2, so + zo * PL, F, ov0, ov1, op);
-          const int po = r * ZM_TX + 2 * i;
-          const float* PD = sm + L::OFF_PD + (zo % ZM_RP) * 3 * L::OWN + po;
-          float k0[3], k1[3];
+      if (t == 0 && s + 4 <= uhi && s + 4 > issued) {
+        const int k = (s + 4) & (ZM_RU - 1);
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        zm_issue(&tmu, sm + k * L::USLOT, bar + k, cx, cy, s + 4 + g.pz, cc, L::TX_BYTES);
+      }
+      issued = max(issued, min(uhi, s + 4));
+      if (live) {
+        // in-plane part of -D sigma + H^{-1} B sigma at plane s
+        constexpr int CX[3] = {0, 2, 3}, CY[3] = {2, 1, 4};  // planes of sigma_{cx}, sigma_{cy}
+        float2 kp[3];
 #pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const float2 pd = ld2(PD + c * L::OWN);
-            k0[c] = pd.x;
-            k1[c] = pd.y;
-          }
-          if (zo >= 4 && zo <= n2 - 5) {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-              const int o = L::OFF_SZ + c * L::OWN + po;
-              const float2 m2 = ld2(sm + ((zo - 2) & (ZM_RS - 1)) * 3 * L::OWN + o);
-              const float2 m1 = ld2(sm + ((zo - 1) & (ZM_RS - 1)) * 3 * L::OWN + o);
-              const float2 p1 = ld2(sm + ((zo + 1) & (ZM_RS - 1)) * 3 * L::OWN + o);
-              const float2 p2 = ld2(sm + ((zo + 2) & (ZM_RS - 1)) * 3 * L::OWN + o);
-              k0[c] -= c4u(m2.x, m1.x, p1.x, p2.x);
-              k1[c] -= c4u(m2.y, m1.y, p1.y, p2.y);
-            }
-          } else {
-#pragma unroll
-            for (int c = 0; c < 3; ++c) {
-#pragma unroll
-              for (int e = 0; e < 2; ++e) {
-                const int o = L::OFF_SZ + c * L::OWN + po + e;
-                auto v = [&](int k) { return sm[((zo + k) & (ZM_RS - 1)) * 3 * L::OWN + o]; };
-                float kc = -zm_closure12(v, zo, n2, tab);
-                if (zo == 0) kc -= BT * v(0);
-                else if (zo == n2 - 1) kc += BT * v(0);
-                if (e) k1[c] += kc;
-                else k0[c] += kc;
-              }
-            }
-          }
-          // leapfrog / filter update of the pair (increment form)
-          const float* Uo = sm + (zo & (ZM_RU - 1)) * L::USLOT + (r + 4) * ZM_UX + 4 + 2 * i;
-          const int p = so + zo * PL;
-#pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const float2 u = ld2(Uo + c * L::UPLANE);
-            float a0 = k0[c] * op.irh.x, a1 = k1[c] * op.irh.y;
-            if (FORCED) {
-              a0 += op.f[c].x * sc.fcos144;
-              a1 += op.f[c].y * sc.fcos144;
-            }
-            float dd0, dd1;
-            if (MODE == STEP_FIRST) {
-              dd0 = -0.5f * sc.kt144 * a0;
-              dd1 = -0.5f * sc.kt144 * a1;
-            } else {
-              dd0 = op.d[c].x - sc.kt144 * a0;
-              dd1 = op.d[c].y - sc.kt144 * a1;
-            }
-            const float un0 = u.x + dd0, un1 = u.y + dd1;
-            float ac0, ac1;
-            if (MODE == STEP_FIRST) {
-              ac0 = sc.w0 * u.x + sc.wnew * un0;
-              ac1 = sc.w0 * u.y + sc.wnew * un1;
-            } else {
-              ac0 = op.a[c].x + sc.wnew * un0;
-              ac1 = op.a[c].y + sc.wnew * un1;
-            }
-            const int pc = p + c * F;
-            if (ov0 && ov1) {
-              if (MODE != STEP_LAST) {
-                __stcs(reinterpret_cast<float2*>(Dw + pc), make_float2(dd0, dd1));
-                __stcs(reinterpret_cast<float2*>(Uw + pc), make_float2(un0, un1));
-              }
-              __stcs(reinterpret_cast<float2*>(Aw + pc), make_float2(ac0, ac1));
-            } else {
-              if (ov0) {
-                if (MODE != STEP_LAST) Dw[pc] = dd0, Uw[pc] = un0;
-                Aw[pc] = ac0;
-              }
-              if (ov1) {
-                if (MODE != STEP_LAST) Dw[pc + 1] = dd1, Uw[pc + 1] = un1;
-                Aw[pc + 1] = ac1;
-              }
-            }
+        for (int c = 0; c < 3; ++c) {
+          const float* Sx = sip + CX[c] * L::SPLANE + ps;
+          const float* Sy = sip + CY[c] * L::SPLANE + ps;
+          const float2 kx = wx ? zm_tap_pair_x(Sx, pm.c0, pm.c1, toff, tcf) : c4x(ld2(Sx - 2), ld2(Sx), ld2(Sx + 2));
+          const float2 ky = wy ? zm_tap_pair_y(Sy, L::SX, pm.cy, toff, tcf)
+                               : c4p(ld2(Sy - 2 * L::SX), ld2(Sy - L::SX), ld2(Sy + L::SX), ld2(Sy + 2 * L::SX));
+          kp[c] = make_float2(-(kx.x + ky.x), -(kx.y + ky.y));
+          if (wx || wy) {  // boundary terms H^{-1} B sigma on free sides (nodes on the side itself)
+            float b0 = 0.f, b1 = 0.f;
+            if (sx == 0) b0 -= BT * Sx[0];
+            if (sx == n0 - 1) b0 += BT * Sx[0];
+            if (sx + 1 == n0 - 1) b1 += BT * Sx[1];
+            if (sy == 0) b0 -= BT * Sy[0], b1 -= BT * Sy[1];
+            if (sy == n1 - 1) b0 += BT * Sy[0], b1 += BT * Sy[1];
+            kp[c].x += b0;
+            kp[c].y += b1;
           }
         }
-        ++next_o;
+        // plane s enters the outputs s - 2 .. s + 2
+        float2 k[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const float2 z = own_z[c];
+          k[c] = add2(A0[c], z);
+          A0[c] = fma2(both(-8.0f), z, A1[c]);
+          A1[c] = add2(A2[c], kp[c]);
+          A2[c] = fma2(both(8.0f), z, A3[c]);
+          A3[c] = make_float2(-z.x, -z.y);
+        }
+        const bool near = s <= 5 || s >= n2 - 6;
+        if (near) {  // the outputs on z closure rows read these planes back
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            *zm_at<float2>(Sg + c * F, so + s * PL4) = own_z[c];
+            *zm_at<float2>(Sg + (3 + c) * F, so + s * PL4) = kp[c];
+          }
+        }
+        if (out)
+          zm_update<MODE, FORCED>(sc, op, k, sm + (o & (ZM_RU - 1)) * L::USLOT + uo, L::UPLANE, Dr, Ar, Ur, so + o * PL4,
+                                  F, fo, ov0, ov1);
       }
-      // operands of the next output plane, one plane ahead
-      if (next_o < zb && op_plane != next_o && (ov0 || ov1)) {
-        zm_load_ops<FORCED>(Dr, Ar, Rr, f.irh2, so + next_o * PL, F, ov0, ov1, op);
-        op_plane = next_o;
-      }
-      __syncthreads();  // every read of the slot refilled below is done
-      if (t == 0 && j + ZM_PREF <= uhi) {
-        const int k = (j + ZM_PREF) & (ZM_RU - 1);
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        zm_issue(&tmu, sm + k * L::USLOT, bar + k, cx, cy, j + ZM_PREF + g.pz, cc, L::TX_BYTES);
+      if (out) next_o = o + 1;
+      // ---- outputs on z closure rows whose stress planes all exist
+      for (; next_o < zb && (next_o < 4 || next_o > n2 - 5) && zm_hi(next_o, n2) <= s; ++next_o) {
+        if (!live) continue;
+        const int oz = next_o, cz = zm_class(oz, n2);
+        const unsigned q = so + oz * PL4;
+        ZmOperands po;
+        zm_load_ops<MODE, FORCED>(Dr, Ar, Rr, f.irh2, q, F, fo, ov0, ov1, po);
+        float2 k[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          k[c] = *zm_at<float2>(Sg + (3 + c) * F, q);
+          for (int j = 0; j < 4; ++j)
+            k[c] = fma2(both(-tcf[4 * cz + j]), *zm_at<float2>(Sg + c * F, q + toff[4 * cz + j] * PL4), k[c]);
+          if (oz == 0 || oz == n2 - 1) k[c] = fma2(both(oz == 0 ? -BT : BT), *zm_at<float2>(Sg + c * F, q), k[c]);
+        }
+        zm_update<MODE, FORCED>(sc, po, k, sm + (oz & (ZM_RU - 1)) * L::USLOT + uo, L::UPLANE, Dr, Ar, Ur, q, F, fo,
+                                ov0, ov1);
       }
     }
     if (!alive) {
       // wait (bounded) for this segment's copies still in flight, then stop
       if (t == 0) atomicAdd(ctl + 4, 1u);
       const unsigned long long t0 = zm_ns();
-      for (int k = jfail; k <= uhi && k < jfail + ZM_PREF; ++k) {  // requested, not yet consumed
+      for (int k = have + 1; k <= issued; ++k) {  // requested, not yet consumed
         const int sl = k & (ZM_RU - 1);
         while (!mbar_try(bar + sl, (phase >> sl) & 1u) && zm_ns() - t0 < 1000000000ull) {
         }
@@ -557,7 +541,7 @@ __global__ void __launch_bounds__(zm_threads<TY>(), TY <= 8 ? 2 : 1)
         const int cnt = (int)((wend - ww) < (long long)(nz - z0) ? (wend - ww) : (long long)(nz - z0));
         const int rh = (int)(tl / (ntx * nty));
         const int t2 = (int)(tl - (long long)rh * ntx * nty);
-        const int x = g.off[0] - sc.shx + ZM_TX * (t2 % ntx) + 2 * i, y = g.off[1] - sc.shy + TY * (t2 / ntx) + r;
+        const int x = g.off[0] - sc.shx + TX * (t2 % ntx) + 2 * pi, y = g.off[1] - sc.shy + TY * (t2 / ntx) + ri;
         for (int zz = 0; zz < cnt; ++zz)
           for (int e = 0; e < 2; ++e)
             if (zm_unknown_x(g, x + e) && zm_unknown_y(g, y))
@@ -569,7 +553,7 @@ __global__ void __launch_bounds__(zm_threads<TY>(), TY <= 8 ? 2 : 1)
 }
 
 // ---- host side ----------------------------------------------------------------
-template <int TY>
+template <int TX, int TY>
 cudaError_t zm_map(const Geom& g, const float* u, unsigned char* out) {
   static_assert(sizeof(CUtensorMap) <= ZM_MAP_BYTES, "tensor map storage");
   EncodeTiledFn enc = encode_fn();
@@ -578,7 +562,7 @@ cudaError_t zm_map(const Geom& g, const float* u, unsigned char* out) {
                               (cuuint64_t)(3 * g.nrhs)};
   const cuuint64_t strides[3] = {(cuuint64_t)g.np[0] * sizeof(float), (cuuint64_t)g.plane * sizeof(float),
                                  (cuuint64_t)g.field * sizeof(float)};
-  const cuuint32_t box[4] = {ZM_UX, (cuuint32_t)(TY + 8), 1, 3};
+  const cuuint32_t box[4] = {(cuuint32_t)(TX + 8), (cuuint32_t)(TY + 8), 1, 3};
   const cuuint32_t es[4] = {1, 1, 1, 1};
   CUtensorMap m;
   const CUresult rc = enc(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, const_cast<float*>(u), dims, strides, box, es,
@@ -589,42 +573,44 @@ cudaError_t zm_map(const Geom& g, const float* u, unsigned char* out) {
   return cudaSuccess;
 }
 
-template <int TY>
+template <int TX, int TY>
 void* zm_kernel(int mode, bool forced) {
-  if (mode == STEP_FIRST) return forced ? (void*)step3d_o4_zm<TY, STEP_FIRST, true> : (void*)step3d_o4_zm<TY, STEP_FIRST, false>;
-  if (mode == STEP_MID) return forced ? (void*)step3d_o4_zm<TY, STEP_MID, true> : (void*)step3d_o4_zm<TY, STEP_MID, false>;
-  return forced ? (void*)step3d_o4_zm<TY, STEP_LAST, true> : (void*)step3d_o4_zm<TY, STEP_LAST, false>;
+  if (mode == STEP_FIRST)
+    return forced ? (void*)step3d_o4_zm<TX, TY, STEP_FIRST, true> : (void*)step3d_o4_zm<TX, TY, STEP_FIRST, false>;
+  if (mode == STEP_MID)
+    return forced ? (void*)step3d_o4_zm<TX, TY, STEP_MID, true> : (void*)step3d_o4_zm<TX, TY, STEP_MID, false>;
+  return forced ? (void*)step3d_o4_zm<TX, TY, STEP_LAST, true> : (void*)step3d_o4_zm<TX, TY, STEP_LAST, false>;
 }
 
 
-template <int TY>
+template <int TX, int TY>
 void plan_one(const Geom& g, const float* u_a, const float* u_b, int sms, int smem_max, ZmPlan& p, int k) {
-  using L = ZmLayout<TY>;
+  using L = ZmLayout<TX, TY>;
   p.ok[k] = 0;
   // x: a multiple of 4 keeps the bulk-tensor box 16-byte aligned and the node pairs even
-  p.shx[k] = zm_shift(g.nu[0], ZM_TX, g.hi_free[0] != 0, 4);
+  p.shx[k] = zm_shift(g.nu[0], TX, g.hi_free[0] != 0, 4);
   p.shy[k] = zm_shift(g.nu[1], TY, g.hi_free[1] != 0, 1);
   if (p.shx[k] < 0 || p.shy[k] < 0 || (int)L::BYTES > smem_max) return;
   for (int mode = 0; mode < 3; ++mode)
     for (int fo = 0; fo < 2; ++fo)
-      if (cudaFuncSetAttribute(zm_kernel<TY>(mode, fo != 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
+      if (cudaFuncSetAttribute(zm_kernel<TX, TY>(mode, fo != 0), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                (int)L::BYTES) != cudaSuccess) {
         cudaGetLastError();
         return;
       }
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, zm_kernel<TY>(STEP_MID, false), L::NT, L::BYTES) !=
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, zm_kernel<TX, TY>(STEP_MID, false), L::NT, L::BYTES) !=
           cudaSuccess ||
       per_sm < 1) {
     cudaGetLastError();
     return;
   }
-  if (zm_map<TY>(g, u_a, p.tmap[k][0]) != cudaSuccess || zm_map<TY>(g, u_b, p.tmap[k][1]) != cudaSuccess) {
+  if (zm_map<TX, TY>(g, u_a, p.tmap[k][0]) != cudaSuccess || zm_map<TX, TY>(g, u_b, p.tmap[k][1]) != cudaSuccess) {
     cudaGetLastError();
     return;
   }
   const long long tiles =
-      (long long)((g.nu[0] + p.shx[k] + ZM_TX - 1) / ZM_TX) * ((g.nu[1] + p.shy[k] + TY - 1) / TY) * g.nrhs;
+      (long long)((g.nu[0] + p.shx[k] + TX - 1) / TX) * ((g.nu[1] + p.shy[k] + TY - 1) / TY) * g.nrhs;
   const long long work = tiles * g.nu[2];
   long long grid = (long long)per_sm * sms;
   const char* cap = getenv("EWH_ZM_GRID");  // fewer CTAs: longer (tile, z range) shares per CTA
@@ -634,16 +620,26 @@ void plan_one(const Geom& g, const float* u_a, const float* u_b, int sms, int sm
   p.ok[k] = 1;
   if (getenv("EWH_VERBOSE"))
     fprintf(stderr,
-            "ewh: z-march plan %d (%d rows): %lld tiles (shift %d, %d) x %d planes on %lld CTAs (%d per SM), %zu B "
+            "ewh: z-march plan %d (%d x %d): %lld tiles (shift %d, %d) x %d planes on %lld CTAs (%d per SM), %zu B "
             "shared\n",
-            k, TY, tiles, p.shx[k], p.shy[k], g.nu[2], grid, per_sm, (size_t)L::BYTES);
+            k, TX, TY, tiles, p.shx[k], p.shy[k], g.nu[2], grid, per_sm, (size_t)L::BYTES);
 }
 
-template <int TY, int MODE>
+template <int TX, int TY, int MODE>
 cudaError_t zm_launch(const cudaLaunchConfig_t& cfg, bool forced, const Geom& g, const WaveFields<float>& f,
                       const ZmScalars& sc, unsigned* ctl, const CUtensorMap& tm) {
-  return forced ? cudaLaunchKernelEx(&cfg, step3d_o4_zm<TY, MODE, true>, g, f, sc, ctl, tm)
-                : cudaLaunchKernelEx(&cfg, step3d_o4_zm<TY, MODE, false>, g, f, sc, ctl, tm);
+  return forced ? cudaLaunchKernelEx(&cfg, step3d_o4_zm<TX, TY, MODE, true>, g, f, sc, ctl, tm)
+                : cudaLaunchKernelEx(&cfg, step3d_o4_zm<TX, TY, MODE, false>, g, f, sc, ctl, tm);
+}
+
+template <int TX, int TY>
+cudaError_t zm_launch_mode(cudaLaunchConfig_t& cfg, StepMode mode, bool forced, const Geom& g,
+                           const WaveFields<float>& f, const ZmScalars& sc, unsigned* ctl, const CUtensorMap& tm) {
+  cfg.blockDim = dim3(ZmLayout<TX, TY>::NT);
+  cfg.dynamicSmemBytes = ZmLayout<TX, TY>::BYTES;
+  if (mode == STEP_FIRST) return zm_launch<TX, TY, STEP_FIRST>(cfg, forced, g, f, sc, ctl, tm);
+  if (mode == STEP_MID) return zm_launch<TX, TY, STEP_MID>(cfg, forced, g, f, sc, ctl, tm);
+  return zm_launch<TX, TY, STEP_LAST>(cfg, forced, g, f, sc, ctl, tm);
 }
 
 }  // namespace
@@ -651,10 +647,11 @@ cudaError_t zm_launch(const cudaLaunchConfig_t& cfg, bool forced, const Geom& g,
 // Build the fused-kernel plan of a 3D order-4 FP32 context: tensor maps of
 // both u buffers per shape, the persistent grids, the shared-memory opt-in.
 // A shape is unusable (the per-level pair runs) when the geometry is outside
-// what the kernel handles: fewer than 12 planes along z.
+// what the kernel handles: fewer than 12 planes along z, or 4 GB and more per
+// component (32-bit byte offsets).
 ZmPlan plan_zmarch(const Geom& g, const float* u_a, const float* u_b, unsigned* ctl) {
   ZmPlan p;
-  if (g.dim != 3 || g.mapped || g.n[2] < 12 || g.off[0] + g.padx != 8) return p;
+  if (g.dim != 3 || g.mapped || g.n[2] < 12 || g.off[0] + g.padx != 8 || g.field >= (1LL << 30)) return p;
   int dev = 0, sms = 0, smem_max = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
@@ -662,8 +659,8 @@ ZmPlan plan_zmarch(const Geom& g, const float* u_a, const float* u_b, unsigned* 
     cudaGetLastError();
     return p;
   }
-  plan_one<16>(g, u_a, u_b, sms, smem_max, p, 0);
-  plan_one<8>(g, u_a, u_b, sms, smem_max, p, 1);
+  plan_one<64, 8>(g, u_a, u_b, sms, smem_max, p, 0);
+  plan_one<32, 8>(g, u_a, u_b, sms, smem_max, p, 1);
   p.u_a = u_a;
   p.u_b = u_b;
   p.ctl = ctl;
@@ -678,7 +675,6 @@ cudaError_t launch_zmarch(const Geom& g, const ZmPlan& p, int k, const WaveField
   CUtensorMap tm;
   std::memcpy(&tm, p.tmap[k][b], sizeof(tm));
   ZmScalars sc;
-  for (int q = 0; q < 24; ++q) sc.tab12[q] = (float)(12.0 * SBP_CLOSURE[q / 6][q % 6]);
   sc.kt144 = (float)(s.kt / 144.0);
   sc.w0 = (float)s.w0;
   sc.wnew = (float)s.wnew;
@@ -689,8 +685,6 @@ cudaError_t launch_zmarch(const Geom& g, const ZmPlan& p, int k, const WaveField
   zm_class_taps(sc.toff, sc.tcf);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(p.grid[k]);
-  cfg.blockDim = dim3(k == 0 ? ZmLayout<16>::NT : ZmLayout<8>::NT);
-  cfg.dynamicSmemBytes = k == 0 ? ZmLayout<16>::BYTES : ZmLayout<8>::BYTES;
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -699,14 +693,8 @@ cudaError_t launch_zmarch(const Geom& g, const ZmPlan& p, int k, const WaveField
   const char* e = getenv("EWH_PDL");
   cfg.numAttrs = (e && e[0] == '0') ? 0 : 1;
   const bool forced = f.frho != nullptr;
-  if (k == 0) {
-    if (mode == STEP_FIRST) return zm_launch<16, STEP_FIRST>(cfg, forced, g, f, sc, p.ctl, tm);
-    if (mode == STEP_MID) return zm_launch<16, STEP_MID>(cfg, forced, g, f, sc, p.ctl, tm);
-    return zm_launch<16, STEP_LAST>(cfg, forced, g, f, sc, p.ctl, tm);
-  }
-  if (mode == STEP_FIRST) return zm_launch<8, STEP_FIRST>(cfg, forced, g, f, sc, p.ctl, tm);
-  if (mode == STEP_MID) return zm_launch<8, STEP_MID>(cfg, forced, g, f, sc, p.ctl, tm);
-  return zm_launch<8, STEP_LAST>(cfg, forced, g, f, sc, p.ctl, tm);
+  return k == 0 ? zm_launch_mode<64, 8>(cfg, mode, forced, g, f, sc, p.ctl, tm)
+                : zm_launch_mode<32, 8>(cfg, mode, forced, g, f, sc, p.ctl, tm);
 }
 
 }  // namespace ewh
