@@ -329,150 +329,202 @@ __global__ void __launch_bounds__(256) step3d_o2(Geom g, WaveFields<T> f, StepSc
     leapfrog_update<T, MODE, FORCED>(f, p0 + al * g.field, U(al, 0, 0, 0), Kc[al] * irh, s);
 }
 
-// ---------------------------------------------------------------------------
-// Order 4 (SBP), any dimension: stress pass then divergence + update pass.
-// Stress fields per rhs: 2D (xx, yy, xy); 3D (xx, yy, zz, xy, xz, yz).
-// ---------------------------------------------------------------------------
-template <int DIM>
-__host__ __device__ constexpr int nsig() { return DIM == 2 ? 3 : 6; }
-template <int DIM>
-__device__ __forceinline__ int sig_index(int a, int b) {
-  if (a == b) return a;
-  if (DIM == 2) return 2;
-  const int lo = a < b ? a : b, hi = a < b ? b : a;
-  return lo == 0 ? (hi == 1 ? 3 : 4) : 5;
+// 12 times the interior difference: the order-4 kernels that carry the
+// operator as 12 D (stresses 12 sigma, divergence 144 D sigma) apply the
+// 1 / 144 once per node, with 1 / (rho h^2), instead of once per difference.
+template <typename T>
+__device__ __forceinline__ T c4u(T m2, T m1, T p1, T p2) {
+  return m2 - T(8) * m1 + T(8) * p1 - p2;
 }
 
-// 3D order 4: the 32 x 8 block of this z plane and its 2-node reach lie in
-// rows, columns and planes 4 .. n - 5 (every difference central, every node
-// an unknown): uniform per block, so the fast path never diverges.
-__device__ __forceinline__ bool o4_3d_inner(const Geom& g, int z) {
-  const int x0 = blockIdx.x * blockDim.x, y0 = blockIdx.y * blockDim.y;
-  return x0 >= 4 && x0 + (int)blockDim.x - 1 <= g.n[0] - 5 && y0 >= 4 && y0 + (int)blockDim.y - 1 <= g.n[1] - 5 &&
-         z >= 4 && z <= g.n[2] - 5;
+// ---------------------------------------------------------------------------
+// Order 4 (SBP), 3D: stress pass then divergence + update pass, the operator
+// carried as 12 D (stress fields 12 sigma: xx, yy, zz, xy, xz, yz per rhs).
+// A thread takes one node of a z plane, nodes numbered row after row without
+// padding: no lane of a warp is idle at the end of a row (32 x 8 blocks left a fifth
+// of them idle at 103 nodes).  Closure rows are four taps from a table by the
+// node's class along an axis, for every lane of a warp alike.
+//
+// FP64 is bound by its pipe (2 lanes per clock and SM; 71 to 80% busy): 100
+// FP64 instructions a node, against 159 with 1/12 in every difference and lanes of
+// closure rows in branches of their own.  101 x 93 x 87 nodes: 265 -> 179 us per
+// level, 64^3 122 -> 69 us, 110^3 384 -> 280 us.  FP32 (the z-march takes over above
+// some 10^6 nodes): 64^3 29 -> 17 us.  Registers: 80 / 64 in FP64 for the stress and the
+// divergence kernel (64 spill in the first), 64 in FP32.
+// ---------------------------------------------------------------------------
+constexpr int S3_THREADS = 256;
+
+template <typename T>
+struct S3Taps {  // 12 D per class: closure rows of the low side (0 .. 3), interior, of the high side (5 .. 8)
+  int off[36];
+  T w[36];
+};
+
+// class of line position p
+__device__ __forceinline__ int s3_class(int p, int n) { return p < 4 ? p : (p > n - 5 ? 5 + (n - 1 - p) : 4); }
+
+// 12 D at v along an axis of stride st, by the taps of class cls
+template <typename T>
+__device__ __forceinline__ T s3_taps12(const T* v, int st, int cls, const S3Taps<T>& t) {
+  const int* o = t.off + 4 * cls;
+  const T* w = t.w + 4 * cls;
+  return w[0] * v[o[0] * st] + w[1] * v[o[1] * st] + w[2] * v[o[2] * st] + w[3] * v[o[3] * st];
+}
+template <typename T>
+__device__ __forceinline__ T s3_c12(const T* v, int st) { return c4u(v[-2 * st], v[-st], v[st], v[2 * st]); }
+// FP32: either form per axis (the compiler computes both and selects, which
+// costs less than the registers of a second code path: 117 against 163 us per
+// level at 128^3; in FP64, where an instruction costs forty issue slots, the second
+// path pays: 203 against 286 us at 101 x 93 x 87)
+template <typename T>
+__device__ __forceinline__ T s3_either(const T* v, int st, bool taps, int cls, const S3Taps<T>& t) {
+  return taps ? s3_taps12(v, st, cls, t) : s3_c12(v, st);
 }
 
-template <typename T, int DIM>
-__global__ void __launch_bounds__(256) sbp_stress(Geom g, const T* __restrict__ u, const T* __restrict__ lam,
-                                                  const T* __restrict__ mu, T* __restrict__ sig) {
-  if (g.dim != DIM) return;  // launched for the wrong dimension: touch nothing
+template <typename T>
+__global__ void __launch_bounds__(S3_THREADS, sizeof(T) == 8 ? 3 : 4) sbp_stress3d(Geom g, const T* __restrict__ u, const T* __restrict__ lam,
+                                                           const T* __restrict__ mu, T* __restrict__ sig,
+                                                           const __grid_constant__ S3Taps<T> tp) {
+  if (g.dim != 3) return;
+  __shared__ S3Taps<T> st;
+  if (threadIdx.x < 36) st.off[threadIdx.x] = tp.off[threadIdx.x], st.w[threadIdx.x] = tp.w[threadIdx.x];
+  const int total = g.n[0] * g.n[1];
+  const int i = blockIdx.x * S3_THREADS + threadIdx.x, ii = min(i, total - 1);
+  const int y = ii / g.n[0], x = ii - y * g.n[0], z = blockIdx.y, rhs = blockIdx.z;
+  const long long pc = pidx(g, 0, 0, x, y, z);
+  const T l = lam[pc], m = mu[pc];  // static: read before the wait
+  __syncthreads();
   pdl_wait();
   pdl_trigger();
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  int z = 0, rhs = blockIdx.z;
-  if (DIM == 3) {
-    const int nz = g.n[2];
-    z = blockIdx.z % nz;
-    rhs = blockIdx.z / nz;
-  }
-  if (x >= g.n[0] || y >= g.n[1]) return;
-  if (DIM == 3 && o4_3d_inner(g, z)) {  // central differences only, 32-bit offsets from one base
-    const int sy = g.np[0], sz = (int)g.plane;  // neighbour offsets: 2 planes index in 32 bits
-    const long long fld = g.field;
-    const long long pc = pidx(g, 0, 0, x, y, z);
-    const T* U = u + pidx(g, rhs, 0, x, y, z);
-    T gr[3][3];
+  const int cx = s3_class(x, g.n[0]), cy = s3_class(y, g.n[1]), cz = s3_class(z, g.n[2]);
+  const bool side = __any_sync(0xffffffffu, cx != 4 || cy != 4 || cz != 4);  // of the warp: no per-lane branch
+  const int sy = g.np[0], sz = (int)g.plane;  // neighbour offsets: 5 planes index in 32 bits (checked at launch)
+  const T* const U = u + (long long)rhs * 3 * g.field + pc;
+  T d[3][3];
+  if (sizeof(T) == 4) {
+    const bool wx = __any_sync(0xffffffffu, cx != 4), wy = __any_sync(0xffffffffu, cy != 4), wz = cz != 4;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const T* b = U + c * fld;
-      gr[c][0] = c4(b[-2], b[-1], b[1], b[2]);
-      gr[c][1] = c4(b[-2 * sy], b[-sy], b[sy], b[2 * sy]);
-      gr[c][2] = c4(b[-2 * sz], b[-sz], b[sz], b[2 * sz]);
+      const T* b = U + c * g.field;
+      d[c][0] = s3_either(b, 1, wx, cx, st);
+      d[c][1] = s3_either(b, sy, wy, cy, st);
+      d[c][2] = s3_either(b, sz, wz, cz, st);
     }
-    const T l = lam[pc], m = mu[pc];
-    const T div = gr[0][0] + gr[1][1] + gr[2][2];
-    T* o = sig + (long long)rhs * 6 * g.field + pc;
-    o[0] = l * div + T(2) * m * gr[0][0];
-    o[fld] = l * div + T(2) * m * gr[1][1];
-    o[2 * fld] = l * div + T(2) * m * gr[2][2];
-    o[3 * fld] = m * (gr[0][1] + gr[1][0]);
-    o[4 * fld] = m * (gr[0][2] + gr[2][0]);
-    o[5 * fld] = m * (gr[1][2] + gr[2][1]);
-    return;
+  } else if (!side) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const T* b = U + c * g.field;
+      d[c][0] = s3_c12(b, 1);
+      d[c][1] = s3_c12(b, sy);
+      d[c][2] = s3_c12(b, sz);
+    }
+  } else {
+#pragma unroll 1
+    for (int c = 0; c < 3; ++c) {
+      const T* b = U + c * g.field;
+      const T e0 = s3_taps12(b, 1, cx, st), e1 = s3_taps12(b, sy, cy, st), e2 = s3_taps12(b, sz, cz, st);
+      if (c == 0) d[0][0] = e0, d[0][1] = e1, d[0][2] = e2;
+      else if (c == 1) d[1][0] = e0, d[1][1] = e1, d[1][2] = e2;
+      else d[2][0] = e0, d[2][1] = e1, d[2][2] = e2;
+    }
   }
-  const int pos[3] = {x, y, z};
-  const long long stride[3] = {1, (long long)g.np[0], g.plane};
-  // gradient grad[alpha][a] = D_a u_alpha
-  T grad[DIM][DIM];
-#pragma unroll
-  for (int al = 0; al < DIM; ++al) {
-    const T* base = u + pidx(g, rhs, al, x, y, z);
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) grad[al][a] = sbp_d1<T>(base, stride[a], pos[a], g.n[a]);
-  }
-  const long long pc = pidx(g, 0, 0, x, y, z);
-  const T l = lam[pc], m = mu[pc];
-  T div = T(0);
-#pragma unroll
-  for (int a = 0; a < DIM; ++a) div += grad[a][a];
-  T* out = sig + (long long)rhs * nsig<DIM>() * g.field + (pc - 0);
-#pragma unroll
-  for (int a = 0; a < DIM; ++a) out[(long long)a * g.field] = l * div + T(2) * m * grad[a][a];
-#pragma unroll
-  for (int a = 0; a < DIM; ++a)
-#pragma unroll
-    for (int b = a + 1; b < DIM; ++b)
-      out[(long long)sig_index<DIM>(a, b) * g.field] = m * (grad[a][b] + grad[b][a]);
+  if (i >= total) return;
+  const T ld = l * (d[0][0] + d[1][1] + d[2][2]), m2 = m + m;
+  T* const o = sig + (long long)rhs * 6 * g.field + pc;
+  const long long fld = g.field;
+  o[0] = ld + m2 * d[0][0];
+  o[fld] = ld + m2 * d[1][1];
+  o[2 * fld] = ld + m2 * d[2][2];
+  o[3 * fld] = m * (d[0][1] + d[1][0]);
+  o[4 * fld] = m * (d[0][2] + d[2][0]);
+  o[5 * fld] = m * (d[1][2] + d[2][1]);
 }
 
-template <typename T, int DIM, int MODE, bool FORCED>
-__global__ void __launch_bounds__(256) sbp_divergence_step(Geom g, WaveFields<T> f, StepScalars s) {
-  if (g.dim != DIM) return;
+template <typename T, int MODE, bool FORCED>
+__global__ void __launch_bounds__(S3_THREADS, 4) sbp_div3d(Geom g, WaveFields<T> f, StepScalars s,
+                                                           double kt144, double ktcos,
+                                                           const __grid_constant__ S3Taps<T> tp) {
+  if (g.dim != 3) return;
+  __shared__ S3Taps<T> st;
+  if (threadIdx.x < 36) st.off[threadIdx.x] = tp.off[threadIdx.x], st.w[threadIdx.x] = tp.w[threadIdx.x];
+  const int total = g.nu[0] * g.nu[1];  // unknown nodes of the plane
+  const int i = blockIdx.x * S3_THREADS + threadIdx.x, ii = min(i, total - 1);
+  const int yi = ii / g.nu[0];
+  const int x = ii - yi * g.nu[0] + g.off[0], y = yi + g.off[1], z = blockIdx.y + g.off[2], rhs = blockIdx.z;
+  const long long pc = pidx(g, 0, 0, x, y, z);
+  const T irh = f.irh2[pc];  // static: read before the wait
+  __syncthreads();
   pdl_wait();
   pdl_trigger();
-  const int x = blockIdx.x * blockDim.x + threadIdx.x;
-  const int y = blockIdx.y * blockDim.y + threadIdx.y;
-  int z = 0, rhs = blockIdx.z;
-  if (DIM == 3) {
-    const int nz = g.n[2];
-    z = blockIdx.z % nz;
-    rhs = blockIdx.z / nz;
+  const int cx = s3_class(x, g.n[0]), cy = s3_class(y, g.n[1]), cz = s3_class(z, g.n[2]);
+  const bool side = __any_sync(0xffffffffu, cx != 4 || cy != 4 || cz != 4);
+  const int sy = g.np[0], sz = (int)g.plane;
+  const long long fld = g.field;
+  const T* const S = f.sigma + (long long)rhs * 6 * fld + pc;  // planes xx, yy, zz, xy, xz, yz
+  constexpr int row[3][3] = {{0, 3, 4}, {3, 1, 5}, {4, 5, 2}};
+  T k[3];  // -144 h^2 rho M^{-1} K u
+  const T bt = T(12.0 * 48.0 / 17.0);  // boundary terms of free sides: -D + H^{-1} B
+  if (sizeof(T) == 4) {
+    const bool wx = __any_sync(0xffffffffu, cx != 4), wy = __any_sync(0xffffffffu, cy != 4), wz = cz != 4;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const T* const a = S + row[c][0] * fld;
+      const T* const b = S + row[c][1] * fld;
+      const T* const e = S + row[c][2] * fld;
+      k[c] = s3_either(a, 1, wx, cx, st) + s3_either(b, sy, wy, cy, st) + s3_either(e, sz, wz, cz, st);
+      if (side) {
+        if (x == 0) k[c] += bt * a[0];
+        if (x == g.n[0] - 1) k[c] -= bt * a[0];
+        if (y == 0) k[c] += bt * b[0];
+        if (y == g.n[1] - 1) k[c] -= bt * b[0];
+        if (z == 0) k[c] += bt * e[0];
+        if (z == g.n[2] - 1) k[c] -= bt * e[0];
+      }
+    }
+  } else if (!side) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      k[c] = s3_c12(S + row[c][0] * fld, 1) + s3_c12(S + row[c][1] * fld, sy) + s3_c12(S + row[c][2] * fld, sz);
+  } else {
+#pragma unroll 1
+    for (int c = 0; c < 3; ++c) {
+      const T* const a = S + (c == 0 ? 0 : c == 1 ? 3 : 4) * fld;
+      const T* const b = S + (c == 0 ? 3 : c == 1 ? 1 : 5) * fld;
+      const T* const e = S + (c == 0 ? 4 : c == 1 ? 5 : 2) * fld;
+      T v = s3_taps12(a, 1, cx, st) + s3_taps12(b, sy, cy, st) + s3_taps12(e, sz, cz, st);
+      if (x == 0) v += bt * a[0];
+      if (x == g.n[0] - 1) v -= bt * a[0];
+      if (y == 0) v += bt * b[0];
+      if (y == g.n[1] - 1) v -= bt * b[0];
+      if (z == 0) v += bt * e[0];
+      if (z == g.n[2] - 1) v -= bt * e[0];
+      if (c == 0) k[0] = v;
+      else if (c == 1) k[1] = v;
+      else k[2] = v;
+    }
   }
-  if (DIM == 3 && x < g.n[0] && y < g.n[1] && o4_3d_inner(g, z)) {  // central differences, no boundary terms
-    const int sy = g.np[0], sz = (int)g.plane;  // neighbour offsets: 2 planes index in 32 bits
-    const long long fld = g.field;
-    const long long pc = pidx(g, 0, 0, x, y, z);
-    const T* S = f.sigma + (long long)rhs * 6 * g.field + pc;  // planes xx, yy, zz, xy, xz, yz
-    const T* Sxx = S;
-    const T* Syy = S + fld;
-    const T* Szz = S + 2 * fld;
-    const T* Sxy = S + 3 * fld;
-    const T* Sxz = S + 4 * fld;
-    const T* Syz = S + 5 * fld;
-    const T ku = -(c4(Sxx[-2], Sxx[-1], Sxx[1], Sxx[2]) + c4(Sxy[-2 * sy], Sxy[-sy], Sxy[sy], Sxy[2 * sy]) +
-                   c4(Sxz[-2 * sz], Sxz[-sz], Sxz[sz], Sxz[2 * sz]));
-    const T kv = -(c4(Sxy[-2], Sxy[-1], Sxy[1], Sxy[2]) + c4(Syy[-2 * sy], Syy[-sy], Syy[sy], Syy[2 * sy]) +
-                   c4(Syz[-2 * sz], Syz[-sz], Syz[sz], Syz[2 * sz]));
-    const T kw = -(c4(Sxz[-2], Sxz[-1], Sxz[1], Sxz[2]) + c4(Syz[-2 * sy], Syz[-sy], Syz[sy], Syz[2 * sy]) +
-                   c4(Szz[-2 * sz], Szz[-sz], Szz[sz], Szz[2 * sz]));
-    const T irh = f.irh2[pc];
-    const long long p0 = pidx(g, rhs, 0, x, y, z);
-    leapfrog_update<T, MODE, FORCED>(f, p0, f.u_cur[p0], ku * irh, s);
-    leapfrog_update<T, MODE, FORCED>(f, p0 + fld, f.u_cur[p0 + fld], kv * irh, s);
-    leapfrog_update<T, MODE, FORCED>(f, p0 + 2 * fld, f.u_cur[p0 + 2 * fld], kw * irh, s);
+  if (i >= total) return;
+  const long long p0 = (long long)rhs * 3 * fld + pc;
+  if (MODE == 3) {  // operator only
+    const T a = irh * T(-1.0 / 144.0);
+#pragma unroll
+    for (int c = 0; c < 3; ++c) f.u_next[p0 + c * fld] = k[c] * a;
     return;
   }
-  if (!is_unknown(g, x, y, z)) return;
-  const int pos[3] = {x, y, z};
-  const long long stride[3] = {1, (long long)g.np[0], g.plane};
-  const long long pc = pidx(g, 0, 0, x, y, z);
-  const T* sig = f.sigma + (long long)rhs * nsig<DIM>() * g.field + pc;
-  const T inv_h0 = T(48.0 / 17.0);
-  const T irh = f.irh2[pc];
-  const long long p0 = pidx(g, rhs, 0, x, y, z);
+  const T cs = irh * T(kt144), fc = T(ktcos);
 #pragma unroll
-  for (int al = 0; al < DIM; ++al) {
-    T k = T(0);
-#pragma unroll
-    for (int a = 0; a < DIM; ++a) {
-      const T* sa = sig + (long long)sig_index<DIM>(al, a) * g.field;
-      k -= sbp_d1<T>(sa, stride[a], pos[a], g.n[a]);
-      if (pos[a] == 0) k -= inv_h0 * sa[0];                 // free low side
-      else if (pos[a] == g.n[a] - 1) k += inv_h0 * sa[0];   // free high side
+  for (int c = 0; c < 3; ++c) {
+    const long long p = p0 + c * fld;
+    const T uv = f.u_cur[p];
+    T d = MODE == STEP_FIRST ? k[c] * cs : f.delta[p] + k[c] * cs;
+    if (FORCED) d -= fc * f.frho[p];
+    if (MODE == STEP_FIRST) d *= T(0.5);
+    const T un = uv + d;
+    if (MODE != STEP_LAST) {
+      f.delta[p] = d;
+      f.u_next[p] = un;
     }
-    const long long p = p0 + al * g.field;
-    leapfrog_update<T, MODE, FORCED>(f, p, f.u_cur[p], k * irh, s);
+    f.acc[p] = MODE == STEP_FIRST ? T(s.w0) * uv + T(s.wnew) * un : f.acc[p] + T(s.wnew) * un;
   }
 }
 
@@ -485,14 +537,6 @@ __global__ void __launch_bounds__(256) sbp_divergence_step(Geom g, WaveFields<T>
 // run the generic per-node code from global memory.
 // ---------------------------------------------------------------------------
 constexpr int TL_H = 2;
-
-// 12 times the interior difference: the order-4 kernels that carry the
-// operator as 12 D (stresses 12 sigma, divergence 144 D sigma) apply the
-// 1 / 144 once per node, with 1 / (rho h^2), instead of once per difference.
-template <typename T>
-__device__ __forceinline__ T c4u(T m2, T m1, T p1, T p2) {
-  return m2 - T(8) * m1 + T(8) * p1 - p2;
-}
 
 // every node of the block and its 2-node reach lies in rows/columns 4..N-5
 template <int TL_TX, int TL_TY>
@@ -1097,6 +1141,25 @@ cudaError_t launch_curv_metrics(int n0, int n1, double h, const double* X, const
   return cudaGetLastError();
 }
 
+// The taps of 12 D per class (see S3Taps).
+template <typename T>
+static const S3Taps<T>& s3_taps() {
+  static const S3Taps<T> t = [] {
+    static const int cols[4][4] = {{0, 1, 2, 3}, {0, 2, -1, -1}, {0, 1, 3, 4}, {0, 2, 4, 5}};
+    static const int in_off[4] = {-2, -1, 1, 2};
+    static const double in_w[4] = {1.0, -8.0, 8.0, -1.0};
+    S3Taps<T> q;
+    for (int c = 0; c < 9; ++c)
+      for (int k = 0; k < 4; ++k) {
+        const int r = c < 4 ? c : c - 5, j = c == 4 ? 0 : cols[r][k];
+        q.off[4 * c + k] = c == 4 ? in_off[k] : (j < 0 ? 0 : (c < 4 ? j - r : r - j));
+        q.w[4 * c + k] = (T)(c == 4 ? in_w[k] : (j < 0 ? 0.0 : (c < 4 ? 12.0 : -12.0) * SBP_CLOSURE[r][j]));
+      }
+    return q;
+  }();
+  return t;
+}
+
 template <typename T, int MODE, bool FORCED, int TX, int TY>
 static cudaError_t launch_split_o4(const Geom& g, const WaveFields<T>& f, const StepScalars& s, cudaStream_t st) {
   dim3 tgrd((g.n[0] + TX - 1) / TX, (g.n[1] + TY - 1) / TY, g.nrhs);
@@ -1180,8 +1243,6 @@ static cudaError_t launch_mode(const Geom& g, int order, const WaveFields<T>& f,
     if (nl) *nl += 1;
     return cudaGetLastError();
   }
-  dim3 blk(32, 8);
-  dim3 grd((g.n[0] + 31) / 32, (g.n[1] + 7) / 8, g.dim == 2 ? g.nrhs : g.n[2] * g.nrhs);
   if (g.dim == 2) {
     cudaError_t e;
     if constexpr (sizeof(T) == 8) {
@@ -1208,9 +1269,14 @@ static cudaError_t launch_mode(const Geom& g, int order, const WaveFields<T>& f,
         return cudaGetLastError();
       }
     }
-    cudaError_t e = launch_k(sbp_stress<T, 3>, grd, blk, st, g, (const T*)f.u_cur, f.lam, f.mu, f.sigma);
+    if (5 * g.plane >= (1LL << 31) || (long long)g.n[0] * g.n[1] >= (1LL << 31) - S3_THREADS) return cudaErrorInvalidValue;
+    const S3Taps<T>& tp = s3_taps<T>();
+    auto blocks = [](long long n) { return (unsigned)((n + S3_THREADS - 1) / S3_THREADS); };
+    cudaError_t e = launch_k(sbp_stress3d<T>, dim3(blocks((long long)g.n[0] * g.n[1]), g.n[2], g.nrhs), dim3(S3_THREADS),
+                             st, g, (const T*)f.u_cur, f.lam, f.mu, f.sigma, tp);
     if (e != cudaSuccess) return e;
-    e = launch_k(sbp_divergence_step<T, 3, MODE, FORCED>, grd, blk, st, g, f, s);
+    e = launch_k(sbp_div3d<T, MODE, FORCED>, dim3(blocks((long long)g.nu[0] * g.nu[1]), g.nu[2], g.nrhs), dim3(S3_THREADS),
+                 st, g, f, s, s.kt / 144.0, s.kt * s.cosn, tp);
     if (e != cudaSuccess) return e;
   }
   if (nl) *nl += 2;
