@@ -231,102 +231,212 @@ __global__ void __launch_bounds__(32 * TYV) step2d_o2(Geom g, WaveFields<T> f, S
 }
 
 // ---------------------------------------------------------------------------
-// Order 2, 3D: 32 x 4 x 2 tile, halo 1.
+// Order 2, 3D: a CTA of 32 x 8 threads walks its columns of unknowns along z.
+// u, lambda and mu of a plane (with a halo of one node) are staged in a ring of
+// four planes (three in FP64, with a second barrier per plane); the next plane's
+// loads are in flight while a plane is computed.  Nodes off the free sides take one formula
+// without a test: a transposed centred difference needs no mask, because u
+// vanishes on a Dirichlet plane and with it every difference along the plane.
+// Warps with a node on a free side take the form with weights.
+//
+// 128^3 FP32: 122 -> 42 us per level (0.53 of the copy rate in the 72-byte count),
+// 1740 -> 370 instructions a node; bound by shared-memory reads (59 a node) and by
+// the barrier.  FP64, bound by its pipe: 1325 -> 475 us, 61^3 141 -> 62 us.  With
+// every side free: 129 -> 61 us and 1481 -> 738 us.
 // ---------------------------------------------------------------------------
-template <typename T, int MODE, bool FORCED>
-__global__ void __launch_bounds__(256) step3d_o2(Geom g, WaveFields<T> f, StepScalars s) {
-  if (g.dim != 3) return;
-  pdl_wait();
-  pdl_trigger();
-  constexpr int TX = 32, TY = 4, TZ = 2, SX = TX + 2, SY = TY + 2, SZ = TZ + 2;
-  __shared__ T su[3][SZ][SY][SX];
-  __shared__ T sl[SZ][SY][SX];
-  __shared__ T sm[SZ][SY][SX];
-  const int nzb = (g.n[2] + TZ - 1) / TZ;
-  const int rhs = blockIdx.z / nzb;
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY, z0 = (blockIdx.z % nzb) * TZ;
-  const int tid = (threadIdx.z * TY + threadIdx.y) * TX + threadIdx.x;
-  for (int i = tid; i < SX * SY * SZ; i += TX * TY * TZ) {
-    const int lx = i % SX, ly = (i / SX) % SY, lz = i / (SX * SY);
-    const int gx = x0 - 1 + lx, gy = y0 - 1 + ly, gz = z0 - 1 + lz;
-    const long long pu = pidx(g, rhs, 0, gx, gy, gz);
-    su[0][lz][ly][lx] = f.u_cur[pu];
-    su[1][lz][ly][lx] = f.u_cur[pu + g.field];
-    su[2][lz][ly][lx] = f.u_cur[pu + 2 * g.field];
-    const long long pc = pidx(g, 0, 0, gx, gy, gz);
-    sl[lz][ly][lx] = f.lam[pc];
-    sm[lz][ly][lx] = f.mu[pc];
+constexpr int O2_TX = 32, O2_TY = 8, O2_SX = O2_TX + 2, O2_SY = O2_TY + 2, O2_PLANE = O2_SX * O2_SY;
+
+// Planes per CTA: the walk of the busiest SM is shortest (two planes stand for a
+// CTA's prologue).  21^3: 1, 61^3: 7, 128^3: 16 (FP32, at most 16: with 19, three CTAs an SM
+// for four, 51 us for 42) or 19 (FP64).  At a fixed 16, 61^3 took 17 us in FP32 and 138
+// in FP64 for 8.5 and 62, 21^3 17 and 176 for 2.6 and 13.
+inline int o2_planes(int tiles, int nz, int most) {
+  int best = 1;
+  long long cost = 1LL << 62;
+  for (int zc = 1; zc <= most && zc <= nz; ++zc) {
+    const long long ctas = (long long)tiles * ((nz + zc - 1) / zc), c = (ctas + 151) / 152 * (zc + 2);
+    if (c < cost) cost = c, best = zc;
   }
-  __syncthreads();
-  const int pos[3] = {x0 + (int)threadIdx.x, y0 + (int)threadIdx.y, z0 + (int)threadIdx.z};
-  if (!is_unknown(g, pos[0], pos[1], pos[2])) return;
-  const int t0[3] = {(int)threadIdx.x + 1, (int)threadIdx.y + 1, (int)threadIdx.z + 1};
-  const bool lo[3] = {pos[0] == 0, pos[1] == 0, pos[2] == 0};
-  const bool hi[3] = {pos[0] == g.n[0] - 1, pos[1] == g.n[1] - 1, pos[2] == g.n[2] - 1};
+  return best;
+}
 
-  auto U = [&](int c, int dx, int dy, int dz) -> T { return su[c][t0[2] + dz][t0[1] + dy][t0[0] + dx]; };
-  auto L = [&](int dx, int dy, int dz) -> T { return sl[t0[2] + dz][t0[1] + dy][t0[0] + dx]; };
-  auto Mu = [&](int dx, int dy, int dz) -> T { return sm[t0[2] + dz][t0[1] + dy][t0[0] + dx]; };
-  auto Uo = [&](int c, const int* o) -> T { return U(c, o[0], o[1], o[2]); };
-
-  T Kc[3];
-#pragma unroll
-  for (int al = 0; al < 3; ++al) {
-    T acc = T(0);
-    // pure terms along every axis
+// 2 h^2 rho M^{-1} K u at the node v of the middle plane: five fields (u, v, w,
+// lambda, mu) O2_PLANE apart, dm and dp the ways to planes z - 1 and z + 1.  SIDE:
+// the node may lie on a free side (lo, hi).  There a difference takes the node itself
+// for the neighbour that is missing, over half the width (w = 2), which also drops
+// that edge's pure term; the transposed difference weighs its two members by ga, gb
+// (G(-1) - G(1) inside, 2 G(-1) + 2 G(0) and -2 G(0) - 2 G(1) at the ends).
+template <typename T, bool SIDE>
+__device__ __forceinline__ void o2_node(const T* v, int dm, int dp, const bool lo[3], const bool hi[3], T k[3]) {
+  constexpr int F = O2_PLANE;
+  int nb[3][2] = {{-1, 1}, {-O2_SX, O2_SX}, {dm, dp}};
+  T w[3], ga[3], gb[3];
+  if (SIDE) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
-      int e[3] = {0, 0, 0};
-      e[a] = 1;
-      const T c0 = (al == a) ? L(0, 0, 0) + T(2) * Mu(0, 0, 0) : Mu(0, 0, 0);
-      T t = T(0);
-      if (pos[a] > 0) {
-        const T cl = (al == a) ? L(-e[0], -e[1], -e[2]) + T(2) * Mu(-e[0], -e[1], -e[2]) : Mu(-e[0], -e[1], -e[2]);
-        t += T(0.5) * (c0 + cl) * (U(al, 0, 0, 0) - U(al, -e[0], -e[1], -e[2]));
-      }
-      if (pos[a] < g.n[a] - 1) {
-        const T cr = (al == a) ? L(e[0], e[1], e[2]) + T(2) * Mu(e[0], e[1], e[2]) : Mu(e[0], e[1], e[2]);
-        t -= T(0.5) * (c0 + cr) * (U(al, e[0], e[1], e[2]) - U(al, 0, 0, 0));
-      }
-      acc += (lo[a] || hi[a]) ? T(2) * t : t;
+      w[a] = lo[a] || hi[a] ? T(2) : T(1);
+      ga[a] = lo[a] ? T(-2) : w[a];
+      gb[a] = hi[a] ? T(-2) : w[a];
+      if (lo[a]) nb[a][0] = 0;
+      if (hi[a]) nb[a][1] = 0;
     }
-    // mixed terms: for each beta != alpha
-    //   Z_alpha( lambda C_beta u_beta ) + Z_beta( mu C_alpha u_beta )
-#pragma unroll
-    for (int be = 0; be < 3; ++be) {
-      if (be == al) continue;
-#pragma unroll
-      for (int term = 0; term < 2; ++term) {
-        const int za = term == 0 ? al : be;   // axis of the transposed difference
-        const int cb = term == 0 ? be : al;   // axis of the inner difference
-        auto G = [&](int k) -> T {
-          int o[3] = {0, 0, 0};
-          o[za] = k;
-          if (!is_unknown(g, pos[0] + o[0], pos[1] + o[1], pos[2] + o[2])) return T(0);
-          int op[3] = {o[0], o[1], o[2]}, om[3] = {o[0], o[1], o[2]};
-          op[cb] += 1;
-          om[cb] -= 1;
-          T d;
-          if (hi[cb]) d = Uo(be, o) - Uo(be, om);
-          else if (lo[cb]) d = Uo(be, op) - Uo(be, o);
-          else d = T(0.5) * (Uo(be, op) - Uo(be, om));
-          const T cf = term == 0 ? L(o[0], o[1], o[2]) : Mu(o[0], o[1], o[2]);
-          return cf * d;
-        };
-        T z;
-        if (hi[za]) z = G(-1) + G(0);
-        else if (lo[za]) z = -(G(0) + G(1));
-        else z = T(0.5) * (G(-1) - G(1));
-        acc += z;
-      }
-    }
-    Kc[al] = acc;
   }
-  const T irh = f.irh2[pidx(g, 0, 0, pos[0], pos[1], pos[2])];
-  const long long p0 = pidx(g, rhs, 0, pos[0], pos[1], pos[2]);
+  const T l0 = v[3 * F], m0 = v[4 * F], p0 = l0 + T(2) * m0;
+  T lam[3][2], mu[3][2];
 #pragma unroll
-  for (int al = 0; al < 3; ++al)
-    leapfrog_update<T, MODE, FORCED>(f, p0 + al * g.field, U(al, 0, 0, 0), Kc[al] * irh, s);
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int e = 0; e < 2; ++e) lam[a][e] = v[3 * F + nb[a][e]], mu[a][e] = v[4 * F + nb[a][e]];
+  T pure[3];
+#pragma unroll
+  for (int al = 0; al < 3; ++al) {
+    const T u0 = v[al * F];
+    T t = T(0);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {  // edges along a: twice the mean coefficient
+      const T cl = al == a ? p0 + (lam[a][0] + T(2) * mu[a][0]) : m0 + mu[a][0];
+      const T cr = al == a ? p0 + (lam[a][1] + T(2) * mu[a][1]) : m0 + mu[a][1];
+      const T dl = u0 - v[al * F + nb[a][0]], dr = u0 - v[al * F + nb[a][1]];
+      if (SIDE) {
+        t += w[a] * (cl * dl + cr * dr);
+      } else {
+        t += cl * dl;
+        t += cr * dr;
+      }
+    }
+    pure[al] = t;
+  }
+  if (SIDE) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) lam[a][0] *= ga[a], lam[a][1] *= gb[a], mu[a][0] *= ga[a], mu[a][1] *= gb[a];
+  }
+  T mixed[3] = {T(0), T(0), T(0)};  // four times the mixed terms
+#pragma unroll
+  for (int be = 0; be < 3; ++be)
+#pragma unroll
+    for (int al = 0; al < 3; ++al) {
+      if (al == be) continue;
+      // u_be at the four corners of the (al, be) square: (al side, be side)
+      const T* const q = v + be * F;
+      const T pp = q[nb[al][1] + nb[be][1]], pm = q[nb[al][1] + nb[be][0]];
+      const T mp = q[nb[al][0] + nb[be][1]], mm = q[nb[al][0] + nb[be][0]];
+      // Z_al(lambda C_be u_be) + Z_be(mu C_al u_be)
+      T t = mixed[al];
+      if (SIDE) {
+        t += w[be] * (lam[al][0] * (mp - mm) - lam[al][1] * (pp - pm));
+        t += w[al] * (mu[be][0] * (pm - mm) - mu[be][1] * (pp - mp));
+      } else {
+        t += lam[al][0] * (mp - mm);
+        t -= lam[al][1] * (pp - pm);
+        t += mu[be][0] * (pm - mm);
+        t -= mu[be][1] * (pp - mp);
+      }
+      mixed[al] = t;
+    }
+#pragma unroll
+  for (int al = 0; al < 3; ++al) k[al] = pure[al] + T(0.5) * mixed[al];
+}
+
+template <typename T, int MODE, bool FORCED>
+__global__ void __launch_bounds__(O2_TX * O2_TY, sizeof(T) == 8 ? 2 : 4) step3d_o2(Geom g, WaveFields<T> f, StepScalars s, double kt2, int zc) {
+  if (g.dim != 3) return;
+  constexpr int R = sizeof(T) == 8 ? 3 : 4;
+  __shared__ T ring[R][5 * O2_PLANE];
+  const int t = threadIdx.y * O2_TX + threadIdx.x;
+  const int nzc = (g.nu[2] + zc - 1) / zc;
+  const int rhs = blockIdx.z / nzc;
+  const int X0 = g.off[0] + (int)blockIdx.x * O2_TX, Y0 = g.off[1] + (int)blockIdx.y * O2_TY;
+  const int z0 = g.off[2] + (int)(blockIdx.z % nzc) * zc, z1 = min(z0 + zc, g.off[2] + g.nu[2]);
+  const long long ro = (long long)rhs * 3 * g.field;
+  // the tile positions this thread brings in: two of the 34 x 10
+  const int j0 = t, j1 = t + O2_TX * O2_TY;
+  const bool two = j1 < O2_PLANE;
+  const int q0 = (int)pidx(g, 0, 0, X0 - 1 + j0 % O2_SX, Y0 - 1 + j0 / O2_SX, 0);
+  const int q1 = two ? (int)pidx(g, 0, 0, X0 - 1 + j1 % O2_SX, Y0 - 1 + j1 / O2_SX, 0) : q0;
+  const int PL = (int)g.plane;
+  const T* const U = f.u_cur + ro;
+  T v[2][5];
+  auto load = [&](int z) {
+#pragma unroll
+    for (int e = 0; e < 2; ++e) {
+      const int q = (e ? q1 : q0) + z * PL;
+      if (e && !two) break;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) v[e][c] = U[c * g.field + q];
+      v[e][3] = __ldg(f.lam + q);
+      v[e][4] = __ldg(f.mu + q);
+    }
+  };
+  auto store = [&](int slot) {
+    T* const r = ring[slot];
+#pragma unroll
+    for (int c = 0; c < 5; ++c) {
+      r[c * O2_PLANE + j0] = v[0][c];
+      if (two) r[c * O2_PLANE + j1] = v[1][c];
+    }
+  };
+  pdl_wait();
+  pdl_trigger();
+  for (int z = z0 - 1; z <= z0 + 1; ++z) {  // z0 - 1 >= -1: ghost planes are zero
+    load(z);
+    store(z - z0 + 1);
+  }
+  int sa = 0, sb = 1, sc = 2;  // slots of planes z - 1, z, z + 1
+  const int x = X0 + threadIdx.x, y = Y0 + threadIdx.y;
+  const bool live = x < g.off[0] + g.nu[0] && y < g.off[1] + g.nu[1];
+  // of the warp: one lane on a free side takes all of them through the general form
+  const bool wside = __any_sync(0xffffffffu, live && (x == 0 || x == g.n[0] - 1 || y == 0 || y == g.n[1] - 1));
+  const int o = (threadIdx.y + 1) * O2_SX + threadIdx.x + 1;
+  const long long pc0 = pidx(g, 0, 0, x, y, 0);
+  const T cs = T(kt2), fc = T(s.kt * s.cosn), w0 = T(s.w0), wnew = T(s.wnew);
+  for (int z = z0; z < z1; ++z) {
+    if (z + 1 < z1) load(z + 2);  // in flight during this plane
+    const long long pc = pc0 + (long long)z * PL;
+    T irh = T(0), dl[3], ap[3], fr[3];
+    if (live) {
+      irh = __ldg(f.irh2 + pc);
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const long long p = ro + c * g.field + pc;
+        dl[c] = (MODE == STEP_MID || MODE == STEP_LAST) ? f.delta[p] : T(0);
+        ap[c] = (MODE == STEP_MID || MODE == STEP_LAST) ? f.acc[p] : T(0);
+        fr[c] = FORCED ? __ldg(f.frho + p) : T(0);
+      }
+    }
+    __syncthreads();  // plane z + 1 is in the ring; plane z - 2 is no longer read
+    const bool side = wside || z == 0 || z == g.n[2] - 1;
+    if (live) {
+      const T* const b = ring[sb] + o;
+      const int dm = (sa - sb) * (5 * O2_PLANE), dp = (sc - sb) * (5 * O2_PLANE);
+      const bool lo[3] = {x == 0, y == 0, z == 0}, hi[3] = {x == g.n[0] - 1, y == g.n[1] - 1, z == g.n[2] - 1};
+      T k[3];
+      if (side)
+        o2_node<T, true>(b, dm, dp, lo, hi, k);
+      else
+        o2_node<T, false>(b, dm, dp, lo, hi, k);
+#pragma unroll
+      for (int e = 0; e < 3; ++e) {
+        const long long p = ro + e * g.field + pc;
+        if (MODE == 3) {  // operator only
+          f.u_next[p] = k[e] * (T(0.5) * irh);
+          continue;
+        }
+        T ka = k[e] * (irh * cs);
+        if (FORCED) ka += fc * fr[e];
+        const T uv = b[e * O2_PLANE];
+        const T d = MODE == STEP_FIRST ? T(-0.5) * ka : dl[e] - ka, un = uv + d;
+        if (MODE != STEP_LAST) {
+          f.delta[p] = d;
+          f.u_next[p] = un;
+        }
+        f.acc[p] = MODE == STEP_FIRST ? w0 * uv + wnew * un : ap[e] + wnew * un;
+      }
+    }
+    if (R == 3) __syncthreads();  // plane z - 1 is no longer read
+    const int sn = R == 3 ? sa : (sc + 1) & 3;  // R = 4: the slot of plane z - 2
+    if (z + 1 < z1) store(sn);
+    sa = sb, sb = sc, sc = sn;
+  }
 }
 
 // 12 times the interior difference: the order-4 kernels that carry the
@@ -1182,8 +1292,10 @@ static cudaError_t launch_mode(const Geom& g, int order, const WaveFields<T>& f,
                                  : launch_k(step2d_o2<T, MODE, FORCED, 8>, grd, blk, st, g, f, s);
       if (e != cudaSuccess) return e;
     } else {
-      dim3 blk(32, 4, 2), grd((g.n[0] + 31) / 32, (g.n[1] + 3) / 4, ((g.n[2] + 1) / 2) * g.nrhs);
-      cudaError_t e = launch_k(step3d_o2<T, MODE, FORCED>, grd, blk, st, g, f, s);
+      const int tx = (g.nu[0] + O2_TX - 1) / O2_TX, ty = (g.nu[1] + O2_TY - 1) / O2_TY;
+      const int zc = o2_planes(tx * ty * g.nrhs, g.nu[2], sizeof(T) == 8 ? 32 : 16);
+      dim3 blk(O2_TX, O2_TY), grd(tx, ty, (g.nu[2] + zc - 1) / zc * g.nrhs);
+      cudaError_t e = launch_k(step3d_o2<T, MODE, FORCED>, grd, blk, st, g, f, s, 0.5 * s.kt, zc);
       if (e != cudaSuccess) return e;
     }
     if (nl) *nl += 1;
