@@ -25,6 +25,7 @@
 #include <cstring>
 
 #include "ewh_internal.cuh"
+#include "ewh_order2.cuh"
 
 namespace ewh {
 
@@ -138,96 +139,112 @@ __device__ __forceinline__ void leapfrog_update_pre(const WaveFields<T>& f, long
 
 
 // ---------------------------------------------------------------------------
-// Order 2, 2D: 32 x 8 tile, one node per thread, halo 1 in shared memory.
+// Order 2, 2D: 32 x TYV tile, one node per thread, halo 1 in shared memory.  The
+// medium is staged before the wait for the previous level.  Warps off the free sides
+// take the row without weights; next to one, a difference takes the node itself
+// for the neighbour that is missing, over half the width, and the transposed
+// difference weighs its two members (ga, gb).
+//
+// Small grids are latency: 62^2 4.0 -> 1.4 us per level in FP32, 7.0 -> 3.7 us in FP64
+// (medium staged early, fewer FP64 instructions: some 55 a node for 122).  Larger ones
+// are bound by the FP64 pipe, in FP32 by L2 and HBM: 1024^2 214 -> 124 us and
+// 19.7 -> 10.2 us, 2000^2 786 -> 474 us and 77 -> 54 us.
 // ---------------------------------------------------------------------------
 template <typename T, int MODE, bool FORCED, int TYV>
 __global__ void __launch_bounds__(32 * TYV) step2d_o2(Geom g, WaveFields<T> f, StepScalars s) {
   if (g.dim != 2) return;
+  constexpr int TX = 32, TY = TYV, SX = TX + 2, SY = TY + 2, PL = SX * SY;
+  __shared__ T su[2 * PL], sl[PL], sm[PL];
+  const int rhs = blockIdx.z;
+  const int x0 = g.off[0] + blockIdx.x * TX, y0 = g.off[1] + blockIdx.y * TY;
+  const int tid = threadIdx.y * TX + threadIdx.x;
+  constexpr int NL = (PL + TX * TY - 1) / (TX * TY);
+  int q[NL];  // padded offsets of the tile positions this thread stages
+#pragma unroll
+  for (int k = 0; k < NL; ++k) {
+    const int i = tid + k * TX * TY, ly = i / SX;
+    q[k] = (int)pidx(g, 0, 0, x0 - 1 + (i - ly * SX), y0 - 1 + ly, 0);
+    if (i < PL) sl[i] = f.lam[q[k]], sm[i] = f.mu[q[k]];
+  }
+  const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
+  const bool live = x < g.off[0] + g.nu[0] && y < g.off[1] + g.nu[1];
+  const long long pc = pidx(g, 0, 0, x, y, 0), p = (long long)rhs * 2 * g.field + pc;
+  T irh = T(0), fr[2] = {T(0), T(0)}, dl[2], ap[2];
+  if (live) {
+    irh = f.irh2[pc];
+    if (FORCED) fr[0] = f.frho[p], fr[1] = f.frho[p + g.field];
+  }
   pdl_wait();
   pdl_trigger();
-  constexpr int TX = 32, TY = TYV, SX = TX + 2, SY = TY + 2;
-  __shared__ T su[2][SY][SX];
-  __shared__ T sl[SY][SX];
-  __shared__ T sm[SY][SX];
-  const int rhs = blockIdx.z;
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-  const int tid = threadIdx.y * TX + threadIdx.x;
-  for (int i = tid; i < SX * SY; i += TX * TY) {
-    const int lx = i % SX, ly = i / SX;
-    const int gx = x0 - 1 + lx, gy = y0 - 1 + ly;
-    const long long pu = pidx(g, rhs, 0, gx, gy, 0);
-    su[0][ly][lx] = f.u_cur[pu];
-    su[1][ly][lx] = f.u_cur[pu + g.field];
-    const long long pc = pidx(g, 0, 0, gx, gy, 0);
-    sl[ly][lx] = f.lam[pc];
-    sm[ly][lx] = f.mu[pc];
+  const T* const U = f.u_cur + (long long)rhs * 2 * g.field;
+#pragma unroll
+  for (int k = 0; k < NL; ++k) {
+    const int i = tid + k * TX * TY;
+    if (i < PL) su[i] = U[q[k]], su[PL + i] = U[g.field + q[k]];
+  }
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const bool rd = live && (MODE == STEP_MID || MODE == STEP_LAST);
+    dl[c] = rd ? f.delta[p + c * g.field] : T(0);
+    ap[c] = rd ? f.acc[p + c * g.field] : T(0);
   }
   __syncthreads();
-  const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
-  if (!is_unknown(g, x, y, 0)) return;
-  const int tx = threadIdx.x + 1, ty = threadIdx.y + 1;
-  const int nx = g.n[0], ny = g.n[1];
-  // at an unknown node, sitting on the first/last grid line means a free side
-  const bool fxl = (x == 0), fxh = (x == nx - 1), fyl = (y == 0), fyh = (y == ny - 1);
-
-  auto U = [&](int c, int dx, int dy) -> T { return su[c][ty + dy][tx + dx]; };
-  auto L = [&](int dx, int dy) -> T { return sl[ty + dy][tx + dx]; };
-  auto M = [&](int dx, int dy) -> T { return sm[ty + dy][tx + dx]; };
-  auto coef = [&](bool p_wave, int dx, int dy) -> T {
-    return p_wave ? L(dx, dy) + T(2) * M(dx, dy) : M(dx, dy);
+  const bool lo[2] = {x == 0, y == 0}, hi[2] = {x == g.n[0] - 1, y == g.n[1] - 1};
+  // of the warp: one lane on a free side takes all of them through the general form
+  const bool side = __any_sync(0xffffffffu, live && (lo[0] || hi[0] || lo[1] || hi[1]));
+  if (!live) return;
+  const int o = (threadIdx.y + 1) * SX + threadIdx.x + 1;
+  const T l0 = sl[o], m0 = sm[o], p0 = l0 + T(2) * m0;
+  const T ks = T(0.5 * s.kt) * irh, kc = FORCED ? T(s.kt * s.cosn) : T(0);
+  auto node = [&](auto tag) {
+    constexpr bool SIDE = decltype(tag)::value;
+    int nb[2][2] = {{-1, 1}, {-SX, SX}};
+    T w[2] = {T(1), T(1)}, ga[2], gb[2];
+    if (SIDE) {
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        w[a] = lo[a] || hi[a] ? T(2) : T(1);
+        ga[a] = lo[a] ? T(-2) : w[a];
+        gb[a] = hi[a] ? T(-2) : w[a];
+        if (lo[a]) nb[a][0] = 0;
+        if (hi[a]) nb[a][1] = 0;
+      }
+    }
+    T lam[2][2], mu[2][2];
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) lam[a][e] = sl[o + nb[a][e]], mu[a][e] = sm[o + nb[a][e]];
+#pragma unroll
+    for (int c = 0; c < 2; ++c) {
+      const int b = 1 - c;
+      const T *const u = su + c * PL + o, *const v = su + b * PL + o;
+      O2Row<T> r{p0 + (lam[c][0] + T(2) * mu[c][0]), p0 + (lam[c][1] + T(2) * mu[c][1]), m0 + mu[b][0], m0 + mu[b][1],
+                 T(0.5) * lam[c][0], T(0.5) * lam[c][1], T(0.5) * mu[b][0], T(0.5) * mu[b][1]};
+      if (SIDE) {  // powers of two: exact
+        r.ca0 *= w[c], r.ca1 *= w[c], r.cb0 *= w[b], r.cb1 *= w[b];
+        r.la0 *= ga[c] * w[b], r.la1 *= gb[c] * w[b], r.mb0 *= ga[b] * w[c], r.mb1 *= gb[b] * w[c];
+      }
+      const O2Vals<T> n{u[nb[c][0]], u[nb[c][1]], u[nb[b][0]], u[nb[b][1]],
+                        v[nb[c][0] + nb[b][0]], v[nb[c][0] + nb[b][1]], v[nb[c][1] + nb[b][0]], v[nb[c][1] + nb[b][1]]};
+      const T uv = u[0], k = o2_row(r, uv, n);
+      const long long pp = p + c * g.field;
+      if (MODE == 3) {  // operator only
+        f.u_next[pp] = k * (T(0.5) * irh);
+        continue;
+      }
+      const T d = o2_delta<T, FORCED>(MODE == STEP_FIRST, ks, k, kc, fr[c], dl[c]), un = o2_add(uv, d);
+      if (MODE != STEP_LAST) {
+        f.delta[pp] = d;
+        f.u_next[pp] = un;
+      }
+      f.acc[pp] = o2_filter(MODE == STEP_FIRST, T(s.w0), T(s.wnew), uv, un, ap[c]);
+    }
   };
-  // pure terms (edges), already divided by the trapezoid factor of the node
-  auto pureX = [&](int c, bool p_wave) -> T {
-    const T c0 = coef(p_wave, 0, 0);
-    T t = T(0);
-    if (x > 0) t += T(0.5) * (c0 + coef(p_wave, -1, 0)) * (U(c, 0, 0) - U(c, -1, 0));
-    if (x < nx - 1) t -= T(0.5) * (c0 + coef(p_wave, 1, 0)) * (U(c, 1, 0) - U(c, 0, 0));
-    return (fxl || fxh) ? T(2) * t : t;
-  };
-  auto pureY = [&](int c, bool p_wave) -> T {
-    const T c0 = coef(p_wave, 0, 0);
-    T t = T(0);
-    if (y > 0) t += T(0.5) * (c0 + coef(p_wave, 0, -1)) * (U(c, 0, 0) - U(c, 0, -1));
-    if (y < ny - 1) t -= T(0.5) * (c0 + coef(p_wave, 0, 1)) * (U(c, 0, 1) - U(c, 0, 0));
-    return (fyl || fyh) ? T(2) * t : t;
-  };
-  // centred differences at the node offset by dx (resp. dy)
-  auto CyAt = [&](int c, int dx) -> T {
-    if (fyh) return U(c, dx, 0) - U(c, dx, -1);
-    if (fyl) return U(c, dx, 1) - U(c, dx, 0);
-    return T(0.5) * (U(c, dx, 1) - U(c, dx, -1));
-  };
-  auto CxAt = [&](int c, int dy) -> T {
-    if (fxh) return U(c, 0, dy) - U(c, -1, dy);
-    if (fxl) return U(c, 1, dy) - U(c, 0, dy);
-    return T(0.5) * (U(c, 1, dy) - U(c, -1, dy));
-  };
-  // transposed centred difference (divided by the node's trapezoid factor)
-  auto Gx = [&](bool use_lam, int c, int dx) -> T {
-    if (!is_unknown(g, x + dx, y, 0)) return T(0);
-    return (use_lam ? L(dx, 0) : M(dx, 0)) * CyAt(c, dx);
-  };
-  auto Gy = [&](bool use_lam, int c, int dy) -> T {
-    if (!is_unknown(g, x, y + dy, 0)) return T(0);
-    return (use_lam ? L(0, dy) : M(0, dy)) * CxAt(c, dy);
-  };
-  auto Zx = [&](bool use_lam, int c) -> T {
-    if (fxh) return Gx(use_lam, c, -1) + Gx(use_lam, c, 0);
-    if (fxl) return -(Gx(use_lam, c, 0) + Gx(use_lam, c, 1));
-    return T(0.5) * (Gx(use_lam, c, -1) - Gx(use_lam, c, 1));
-  };
-  auto Zy = [&](bool use_lam, int c) -> T {
-    if (fyh) return Gy(use_lam, c, -1) + Gy(use_lam, c, 0);
-    if (fyl) return -(Gy(use_lam, c, 0) + Gy(use_lam, c, 1));
-    return T(0.5) * (Gy(use_lam, c, -1) - Gy(use_lam, c, 1));
-  };
-  // K u for u (x-displacement) and v (y-displacement)
-  const T Ku = pureX(0, true) + pureY(0, false) + Zx(true, 1) + Zy(false, 1);
-  const T Kv = pureX(1, false) + pureY(1, true) + Zy(true, 0) + Zx(false, 0);
-  const T irh = f.irh2[pidx(g, 0, 0, x, y, 0)];
-  const long long p0 = pidx(g, rhs, 0, x, y, 0);
-  leapfrog_update<T, MODE, FORCED>(f, p0, U(0, 0, 0), Ku * irh, s);
-  leapfrog_update<T, MODE, FORCED>(f, p0 + g.field, U(1, 0, 0), Kv * irh, s);
+  if (side)
+    node(std::true_type{});
+  else
+    node(std::false_type{});
 }
 
 // ---------------------------------------------------------------------------
@@ -1286,7 +1303,7 @@ static cudaError_t launch_mode(const Geom& g, int order, const WaveFields<T>& f,
     if (g.dim == 2) {
       // tile height chosen per context (autotuner): 0 -> 8, 1 -> 4, 2 -> 16 rows
       const int ty = g.variant == 1 ? 4 : (g.variant == 2 ? 16 : 8);
-      dim3 blk(32, ty), grd((g.n[0] + 31) / 32, (g.n[1] + ty - 1) / ty, g.nrhs);
+      dim3 blk(32, ty), grd((g.nu[0] + 31) / 32, (g.nu[1] + ty - 1) / ty, g.nrhs);
       cudaError_t e = ty == 4    ? launch_k(step2d_o2<T, MODE, FORCED, 4>, grd, blk, st, g, f, s)
                       : ty == 16 ? launch_k(step2d_o2<T, MODE, FORCED, 16>, grd, blk, st, g, f, s)
                                  : launch_k(step2d_o2<T, MODE, FORCED, 8>, grd, blk, st, g, f, s);
