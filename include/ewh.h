@@ -271,7 +271,8 @@ ewh_status ewh_reset_stats(ewh_ctx* ctx);
  * counterpart in the paper): the grid barrier of the on-chip wave solve (2D,
  * every time level in one cooperative launch per group of right-hand sides,
  * CTAs meeting once per level) and the mbarrier waits of the marching kernels
- * (2D y-march, 3D z-march) for their bulk-tensor copies.  Every wait is
+ * (2D y-march, 3D z-march) for their bulk-tensor copies; the FP32 limit of the
+ * on-chip solve of small order-2 grids (its FP64 waits keep the default).  Every wait is
  * bounded: after ns nanoseconds (default 1e9; the grid barrier also after 2^22
  * polls) the waiting CTA gives up (the on-chip solve raises an error flag and
  * every CTA leaves at its next barrier; a marching CTA waits, bounded, for its

@@ -17,7 +17,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libewh.so")
-SOURCES = ["ewh_stencil.cu", "ewh_zmarch.cu", "ewh_ymarch.cu", "ewh_krylov.cu", "ewh_api.cu", "ewh_fx2d.cu",
+SOURCES = ["ewh_stencil.cu", "ewh_zmarch.cu", "ewh_ymarch.cu", "ewh_krylov.cu", "ewh_api.cu", "ewh_fx2d.cu", "ewh_small2d.cu",
            "ewh_net.cu", "ewh_conv.cu", "ewh_peak.cu"]
 HEADERS = [os.path.join(CSRC, h) for h in ("ewh_internal.cuh", "ewh_march.cuh", "ewh_conv.cuh", "ewh_fixed.cuh",
                                                   "ewh_order2.cuh")]

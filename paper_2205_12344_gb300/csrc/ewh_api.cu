@@ -46,12 +46,15 @@ struct Wave {
   int fallback = 0;           // fastest variant that is not the resident solve
   float variant_ms[YM_VARIANT + 1] = {};  // per time level
   bool ready = false;
-  // on-chip resident solve (2D order 4 FP32, one rhs): per-level scalars,
+  // on-chip solves (2D order 4 FP32; small 2D grids of order 2): per-level scalars,
   // barrier words and the partition per CTA shape
   double* d_cosn = nullptr;
   double* d_wnew = nullptr;
   unsigned* bar = nullptr;
   ResidentPlan rplan[RS_SHAPES];
+  // on-chip solve of small order-2 2D grids: its tiles and exchange words
+  Small2dPlan splan;
+  unsigned long long* xbuf = nullptr;
   // fused marching FP32 order-4 step (3D z-march, 2D y-march): bulk-tensor
   // maps of u_a / u_b, grid (control words in bar)
   ZmPlan zm;
@@ -253,7 +256,11 @@ ewh_status build_wave(ewh_ctx* ctx, Wave<T>& w, const double* d_rho, const doubl
       }
   }
   EWH_CU(cudaGetLastError());
-  if (sizeof(T) == 4 && g.dim == 2 && ctx->order == 4 && !g.mapped) {
+  if (g.dim == 2 && ctx->order == 2 && !g.mapped && !ctx->implicit && !ctx->batch_member) {
+    w.splan = plan_small2d<T>(g);
+    if (w.splan.ok) EWH_CU(cudaMalloc(&w.xbuf, small2d_words(g, sizeof(T)) * sizeof(unsigned long long)));
+  }
+  if (w.splan.ok || (sizeof(T) == 4 && g.dim == 2 && ctx->order == 4 && !g.mapped)) {
     const int N = ctx->nt * ctx->periods;
     std::vector<double> hc(N), hw(N);
     for (int n = 0; n < N; ++n) {  // the same values as the per-level launches get
@@ -268,7 +275,7 @@ ewh_status build_wave(ewh_ctx* ctx, Wave<T>& w, const double* d_rho, const doubl
     EWH_CU(cudaMemcpy(w.bar + 2, &wait_ns, sizeof(wait_ns), cudaMemcpyHostToDevice));
     EWH_CU(cudaMemcpy(w.d_cosn, hc.data(), sizeof(double) * N, cudaMemcpyHostToDevice));
     EWH_CU(cudaMemcpy(w.d_wnew, hw.data(), sizeof(double) * N, cudaMemcpyHostToDevice));
-    for (int k = 0; k < RS_SHAPES; ++k) w.rplan[k] = plan_resident_o4(g, k);
+    for (int k = 0; k < RS_SHAPES && ctx->order == 4; ++k) w.rplan[k] = plan_resident_o4(g, k);
   }
   if (sizeof(T) == 4 && ctx->order == 4 && !g.mapped) {  // marching steps: 3D z-march, 2D y-march
     if (!w.bar) {
@@ -301,6 +308,7 @@ void free_wave(Wave<T>& w) {
   cudaFree(w.d_cosn);
   cudaFree(w.d_wnew);
   cudaFree(w.bar);
+  cudaFree(w.xbuf);
   w = Wave<T>();
 }
 
@@ -389,6 +397,7 @@ std::string tune_key(const ewh_ctx* ctx) {
     for (int k = 0; k < RS_SHAPES; ++k)
       restricted = restricted || (ctx->w32.rplan[k].ok && (long long)ctx->w32.rplan[k].bx * ctx->w32.rplan[k].by <
                                                               RS_BATCH_MIN_BLOCK);
+  if (ctx->batch_member && (sizeof(T) == 4 ? ctx->w32.splan.ok : ctx->w64.splan.ok)) restricted = true;  // small2d_ok
   return name + "|v5" + (restricted ? "b" : "") + (g.mapped ? "|map" : "") + (g.contrast ? "|c" : "") + "|d" + std::to_string(g.dim) +
          "|o" + std::to_string(ctx->order) + "|" +
          (sizeof(T) == 8 ? "f64" : "f32") + "|" + std::to_string(g.n[0]) + "x" + std::to_string(g.n[1]) + "x" +
@@ -442,6 +451,27 @@ cudaError_t enqueue_resident(ewh_ctx* ctx, Wave<T>& w, int v, bool forced, int n
   }
 }
 
+// The on-chip solve of small order-2 2D grids usable by this context?  (Not in a batch:
+// its members' launches run side by side, and this one wants the GPU.)
+template <typename T>
+bool small2d_ok(const ewh_ctx* ctx, const Wave<T>& w) {
+  const char* e = getenv("EWH_RESIDENT");
+  return w.splan.ok && !ctx->batch_member && !(e && e[0] == '0');
+}
+
+// The variant runs all levels of a wave solve in one launch?
+template <typename T>
+bool is_small2d(const ewh_ctx* ctx, const Wave<T>& w, int v) {
+  return v == SMALL2D_VARIANT && w.splan.ok && ctx->order == 2;
+}
+
+template <typename T>
+cudaError_t enqueue_small2d(ewh_ctx* ctx, Wave<T>& w, bool forced, int nsteps) {
+  const Small2dIO<T> io{w.u_a,    w.acc,  w.lam,   w.mu,   w.irh2, forced ? w.frho : nullptr, w.d_cosn,
+                        w.d_wnew, ctx->kt, ctx->weights[0], nsteps, w.xbuf, w.bar};
+  return launch_small2d<T>(ctx->g, w.splan, io, ctx->st);
+}
+
 // The 2D order-4 FP32 y-march usable by this context?
 template <typename T>
 bool ymarch_ok(const ewh_ctx* ctx, const Wave<T>& w) {
@@ -459,7 +489,8 @@ void autotune(ewh_ctx* ctx, Wave<T>& w) {
   const bool ym = ymarch_ok<T>(ctx, w) && !forced_launcher;
   // candidates: the launcher's own variants [0, nbase), the resident shapes,
   // the y-march (only the launcher's own when the environment names one)
-  const int nv = ym ? YM_VARIANT + 1 : (any_res ? VARIANT_RESIDENT + RS_SHAPES : nbase);
+  const bool sm = small2d_ok<T>(ctx, w);
+  const int nv = ym ? YM_VARIANT + 1 : (any_res ? VARIANT_RESIDENT + RS_SHAPES : (sm ? SMALL2D_VARIANT + 1 : nbase));
   w.fallback = 0;
   if (force && force[0] == 'r') {  // EWH_STEP2D_O4=r, r0, r1, r2: resident solve of that CTA shape
     const int k = (force[1] >= '0' && force[1] < '0' + RS_SHAPES) ? force[1] - '0' : 0;
@@ -470,6 +501,11 @@ void autotune(ewh_ctx* ctx, Wave<T>& w) {
   }
   if (force && strcmp(force, "ym") == 0 && ymarch_ok<T>(ctx, w)) {  // EWH_STEP2D_O4=ym: the y-march
     w.variant = YM_VARIANT;
+    return;
+  }
+  const char* force2 = getenv("EWH_STEP2D_O2");  // EWH_STEP2D_O2=r: the small grids' on-chip solve
+  if (force2 && force2[0] == 'r' && sm) {
+    w.variant = SMALL2D_VARIANT;
     return;
   }
   const char* off = getenv("EWH_AUTOTUNE");
@@ -489,7 +525,8 @@ void autotune(ewh_ctx* ctx, Wave<T>& w) {
   auto cache = read_tune_cache(path);
   for (auto& kv : cache)
     if (kv.first == key && kv.second >= 0 && kv.second < nv &&
-        (kv.second < nbase || (any_res && resident_ok<T>(ctx, w, kv.second)) || (kv.second == YM_VARIANT && ym))) {
+        (kv.second < nbase || (any_res && resident_ok<T>(ctx, w, kv.second)) || (kv.second == YM_VARIANT && ym) ||
+         (sm && kv.second == SMALL2D_VARIANT))) {
       w.variant = kv.second;
       return;
     }
@@ -517,12 +554,14 @@ void autotune(ewh_ctx* ctx, Wave<T>& w) {
   const int N = ctx->nt * ctx->periods;
   for (int v = 0; v < nv; ++v) {
     float per_level = 1e30f;
-    if (is_resident_variant(v)) {
-      if (any_res && resident_ok<T>(ctx, w, v)) {  // not when the environment names a per-level launcher
+    if (is_resident_variant(v) || (sm && v == SMALL2D_VARIANT)) {
+      const bool small = sm && v == SMALL2D_VARIANT;
+      auto run = [&](int ns) { return small ? enqueue_small2d<T>(ctx, w, false, ns) : enqueue_resident<T>(ctx, w, v, false, ns); };
+      if (small || (any_res && resident_ok<T>(ctx, w, v))) {  // not when the environment names a per-level launcher
         const int ns = std::min(N, 40);
-        bool ok = enqueue_resident<T>(ctx, w, v, false, std::min(N, 8)) == cudaSuccess;  // warm-up
+        bool ok = run(std::min(N, 8)) == cudaSuccess;  // warm-up
         cudaEventRecord(e0, ctx->st);
-        ok = ok && enqueue_resident<T>(ctx, w, v, false, ns) == cudaSuccess;
+        ok = ok && run(ns) == cudaSuccess;
         cudaEventRecord(e1, ctx->st);
         float ms = 1e30f;
         if (ok && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess)
@@ -582,6 +621,10 @@ cudaError_t enqueue_steps(ewh_ctx* ctx, Wave<T>& w, bool forced, long long* nl) 
     if (e == cudaSuccess && nl) *nl += w.rplan[w.variant - VARIANT_RESIDENT].groups;
     return e;
   }
+  if (is_small2d<T>(ctx, w, w.variant)) {
+    if (nl) *nl += 1;
+    return enqueue_small2d<T>(ctx, w, forced, N);
+  }
   Geom gv = ctx->g;
   gv.variant = w.variant < 0 ? 0 : w.variant;
   WaveFields<T> f{};
@@ -634,7 +677,7 @@ ewh_status ensure_graph(ewh_ctx* ctx, bool forced) {
     }
     ge = nullptr;
     cudaGetLastError();
-    if (attempt == 0 && is_resident_variant(w.variant)) {  // not capturable here: per-level launches
+    if (attempt == 0 && (is_resident_variant(w.variant) || is_small2d<T>(ctx, w, w.variant))) {  // not capturable here: per-level launches
       w.variant = w.fallback;
       continue;
     }
@@ -2557,6 +2600,17 @@ ewh_status ewh_batch_solve(ewh_batch* b, double tol, int maxit, double* const* v
   return s;
 }
 
+// launches of either precision whose wait gave up
+static bool read_timeouts(ewh_ctx* ctx, long long* out) {
+  *out = 0;
+  for (const unsigned* bar : {ctx->w32.bar, ctx->w64.bar}) {
+    unsigned n = 0;
+    if (bar && cudaMemcpy(&n, bar + 4, sizeof(n), cudaMemcpyDeviceToHost) != cudaSuccess) return false;
+    *out += n;
+  }
+  return true;
+}
+
 ewh_status ewh_get_stats(ewh_ctx* ctx, ewh_stats* out) {
   if (!ctx || !out) return EWH_EINVAL;
   if (cudaStreamSynchronize(ctx->st) != cudaSuccess) return fail(ctx, EWH_ECUDA, "synchronise failed");
@@ -2570,12 +2624,8 @@ ewh_status ewh_get_stats(ewh_ctx* ctx, ewh_stats* out) {
   }
   out->launches = ctx->launches;
   out->grid_wait_timeouts = 0;
-  if (ctx->w32.bar) {
-    unsigned n = 0;
-    if (cudaMemcpy(&n, ctx->w32.bar + 4, sizeof(n), cudaMemcpyDeviceToHost) != cudaSuccess)
-      return fail(ctx, EWH_ECUDA, "reading the grid wait counter failed");
-    out->grid_wait_timeouts = (long long)n - ctx->grid_timeouts_base;
-  }
+  if (!read_timeouts(ctx, &out->grid_wait_timeouts)) return fail(ctx, EWH_ECUDA, "reading the grid wait counter failed");
+  out->grid_wait_timeouts -= ctx->grid_timeouts_base;
   return EWH_OK;
 }
 
@@ -2587,12 +2637,7 @@ ewh_status ewh_reset_stats(ewh_ctx* ctx) {
     ctx->wave_ms[k] = 0, ctx->wave_steps[k] = 0, ctx->wave_count[k] = 0, ctx->loop_steps[k] = 0,
     ctx->loop_waves[k] = 0;
   ctx->launches = 0;
-  if (ctx->w32.bar) {
-    unsigned n = 0;
-    if (cudaMemcpy(&n, ctx->w32.bar + 4, sizeof(n), cudaMemcpyDeviceToHost) != cudaSuccess)
-      return fail(ctx, EWH_ECUDA, "reading the grid wait counter failed");
-    ctx->grid_timeouts_base = (long long)n;
-  }
+  if (!read_timeouts(ctx, &ctx->grid_timeouts_base)) return fail(ctx, EWH_ECUDA, "reading the grid wait counter failed");
   return EWH_OK;
 }
 

@@ -225,6 +225,38 @@ constexpr int RS_BAR_WORDS = 8;
 constexpr unsigned long long RS_WAIT_NS_DEFAULT = 1000000000ull;  // one barrier wait, 1 s
 cudaError_t launch_resident_o4(const Geom& g, const ResidentPlan& p, const ResidentIO& io, cudaStream_t st);
 
+// ---- on-chip wave solve of small order-2 2D grids (ewh_small2d.cu) -------------
+// Step-kernel variant of the 2D order-2 launcher (after its three tiles).
+constexpr int SMALL2D_VARIANT = 3;
+constexpr int SMALL2D_THREADS = 1024;  // most threads of a CTA: one per node and component
+struct Small2dPlan {
+  int ok = 0;
+  int px = 0, py = 0;  // CTAs per axis and right-hand side (all co-resident)
+  int bx = 0, by = 0;  // nodes per CTA
+  int P = 0;           // threads per component
+  size_t smem = 0;     // dynamic shared memory per CTA in bytes
+};
+template <typename T>
+struct Small2dIO {
+  const T* u0;  // u^0 (padded, 2 components per right-hand side)
+  T* acc;       // filter accumulator, written at the end (unknowns only)
+  const T* lam;
+  const T* mu;
+  const T* irh2;
+  const T* frho;       // null: unforced
+  const double* cosn;  // [nsteps] as in ResidentIO
+  const double* wnew;
+  double kt, w0;
+  int nsteps;
+  unsigned long long* xbuf;  // [small2d_words] error flag, then the rims (zeroed by the launcher)
+  unsigned* bar;             // [2..3] limit of a wait in ns (u64, 0 = give up at once), [4] launches that gave up
+};
+template <typename T>
+Small2dPlan plan_small2d(const Geom& g);
+size_t small2d_words(const Geom& g, size_t elem);  // u64 words of xbuf
+template <typename T>
+cudaError_t launch_small2d(const Geom& g, const Small2dPlan& p, const Small2dIO<T>& io, cudaStream_t st);
+
 // ---- fused 3D order-4 FP32 step (ewh_zmarch.cu) ------------------------------
 ZmPlan plan_zmarch(const Geom& g, const float* u_a, const float* u_b, unsigned* ctl);
 cudaError_t launch_zmarch(const Geom& g, const ZmPlan& p, int shape, const WaveFields<float>& f, StepMode mode,

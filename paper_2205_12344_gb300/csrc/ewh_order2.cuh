@@ -39,19 +39,12 @@ __device__ __forceinline__ T o2_row(const O2Row<T>& c, T u, const O2Vals<T>& n) 
   return o2_add(k1, k2);
 }
 
-// Leapfrog and filter with k = o2_row, ks = kt / (2 rho h^2), kc = kt cos(w t_n).
+// delta^{n+1} with k = o2_row, ks = kt / (2 rho h^2), kc = kt cos(w t_n); the first level
+// (Taylor start) has half of ks and kc and d = 0.
 template <typename T, bool FORCED>
-__device__ __forceinline__ T o2_delta(bool first, T ks, T k, T kc, T fr, T d) {
-  if (first) {
-    const T r = o2_mul(o2_mul(T(-0.5), ks), k);
-    return FORCED ? o2_fma(o2_mul(T(-0.5), kc), fr, r) : r;
-  }
+__device__ __forceinline__ T o2_delta(T ks, T k, T kc, T fr, T d) {
   const T r = o2_fma(-ks, k, d);
   return FORCED ? o2_fma(-kc, fr, r) : r;
-}
-template <typename T>
-__device__ __forceinline__ T o2_filter(bool first, T w0, T wnew, T u, T un, T acc) {
-  return first ? o2_fma(w0, u, o2_mul(wnew, un)) : o2_fma(wnew, un, acc);
 }
 
 }  // namespace ewh

@@ -195,7 +195,8 @@ __global__ void __launch_bounds__(32 * TYV) step2d_o2(Geom g, WaveFields<T> f, S
   if (!live) return;
   const int o = (threadIdx.y + 1) * SX + threadIdx.x + 1;
   const T l0 = sl[o], m0 = sm[o], p0 = l0 + T(2) * m0;
-  const T ks = T(0.5 * s.kt) * irh, kc = FORCED ? T(s.kt * s.cosn) : T(0);
+  const double kt = MODE == STEP_FIRST ? 0.5 * s.kt : s.kt;
+  const T ks = T(0.5 * kt) * irh, kc = FORCED ? T(kt * s.cosn) : T(0);
   auto node = [&](auto tag) {
     constexpr bool SIDE = decltype(tag)::value;
     int nb[2][2] = {{-1, 1}, {-SX, SX}};
@@ -233,12 +234,12 @@ __global__ void __launch_bounds__(32 * TYV) step2d_o2(Geom g, WaveFields<T> f, S
         f.u_next[pp] = k * (T(0.5) * irh);
         continue;
       }
-      const T d = o2_delta<T, FORCED>(MODE == STEP_FIRST, ks, k, kc, fr[c], dl[c]), un = o2_add(uv, d);
+      const T d = o2_delta<T, FORCED>(ks, k, kc, fr[c], dl[c]), un = o2_add(uv, d);
       if (MODE != STEP_LAST) {
         f.delta[pp] = d;
         f.u_next[pp] = un;
       }
-      f.acc[pp] = o2_filter(MODE == STEP_FIRST, T(s.w0), T(s.wnew), uv, un, ap[c]);
+      f.acc[pp] = o2_fma(T(s.wnew), un, MODE == STEP_FIRST ? o2_mul(T(s.w0), uv) : ap[c]);
     }
   };
   if (side)
