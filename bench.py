@@ -455,17 +455,16 @@ def mapped_measurement(nu, applies, stream, flush):
     return wave_measurement(mapped_workload(nu),
                             "layered2d_%d on an annular sector (mapped grid), order-4 SBP, S applies" % nu,
                             {"fp32": applies, "fp64": applies}, ALG_BYTES_MAPPED, stream, flush,
-                            {0: "curv_step2d (fused, 32x8)", 1: "curv_stress2d + curv_div2d",
-                             2: "curv_step2d (fused, 32x16)"})
+                            {0: "curv_stress2d + curv_div2d"})
 
 
 ALG_BYTES_3D = {"fp32": 72.0, "fp64": 144.0}      # read u, u_prev, acc + write u', acc (3 comps) + lambda, mu, 1/M
 
 
-KERNELS_3D = {0: "sbp_stress + sbp_divergence_step (3D, per level)",
+KERNELS_3D = {0: "sbp_stress3d + sbp_div3d (3D, per level)",
               1: "step3d_o4_zm<64, 8> (fused z-march, 64x8 tiles, per level)",
               2: "step3d_o4_zm<32, 8> (fused z-march, 32x8 tiles, per level)",
-              "fp64": "sbp_stress + sbp_divergence_step (3D, per level; FP64 has no fused z-march)"}
+              "fp64": "sbp_stress3d + sbp_div3d (3D, per level; FP64 has no fused z-march)"}
 
 
 def threed_measurement(nu, stream, flush, peaks_fma=None, small_nu=48, e2e_iters=5):

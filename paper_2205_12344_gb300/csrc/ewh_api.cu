@@ -480,7 +480,7 @@ bool ymarch_ok(const ewh_ctx* ctx, const Wave<T>& w) {
 
 template <typename T>
 void autotune(ewh_ctx* ctx, Wave<T>& w) {
-  const int nbase = ctx->g.mapped ? 3 : step_variant_count(ctx->g.dim, ctx->order);
+  const int nbase = ctx->g.mapped ? 1 : step_variant_count(ctx->g.dim, ctx->order);
   const char* force = getenv("EWH_STEP2D_O4");
   // a launcher named by the environment (the y-march exists in FP32 only)
   const bool forced_launcher = force && (force[0] == 's' || force[0] == 'f' || (force[0] == 'y' && sizeof(T) == 4));

@@ -931,16 +931,6 @@ static cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, cud
 // ewh_fx2d.cu), 4 = single fused launch, YM_VARIANT = the FP32 y-march
 // (ewh_ymarch.cu).  EWH_STEP2D_O4=fused|split|ym|fx overrides it (read whenever
 // launches are enqueued; a context captures its step graph once, on first use).
-// Mapped 2D grids: 0 = fused curv_step2d with 32x8 outputs per block, 1 =
-// curv_stress2d + curv_div2d, 2 = fused with 32x16 outputs (FP32; FP64 runs 32x8).  Geom::variant
-// from the autotuner; EWH_CURV=fused|fused16|split overrides it.
-static int curv_variant(const Geom& g) {
-  const char* e = getenv("EWH_CURV");
-  if (e && e[0] == 'f') return strcmp(e, "fused16") == 0 ? 2 : 0;
-  if (e && e[0] == 's') return 1;
-  return (g.variant == 1 || g.variant == 2) ? g.variant : 0;
-}
-
 static int step2d_o4_variant(const Geom& g) {
   const char* e = getenv("EWH_STEP2D_O4");
   if (e && e[0] == 'f' && e[1] != 'x') return 1;
@@ -964,279 +954,247 @@ static int step2d_o4_tile(const Geom& g) {
 //   F^q_v = y_r s_xy - x_r s_yy,  F^r_v = -y_q s_xy + x_q s_yy;
 // the divergence kernel forms -D_q F^q - D_r F^r + H^{-1} B F (the Cartesian
 // kernel with the fluxes in place of the stresses) times 1/(rho J h^2).
-// One node per thread, global memory (the grid sizes of mapped problems are
-// moderate); the metric planes are (y_r, -x_r, -y_q, x_q).
+// The metric planes are (y_r, -x_r, -y_q, x_q).
+//
+// The pair: a thread takes 16 bytes' worth of nodes along x (four in FP32, two
+// in FP64) of the rectangle where every difference is central and every node an
+// unknown, with 16-byte loads (14 for the differences of four FP32 nodes instead of
+// 64).  Rectangle and frame (the nodes within some four of a side, general form, one
+// per thread) are numbered apart, so no warp runs both forms; the frame's blocks
+// come first, since its threads take longest.  What no level writes is read before the
+// wait for the previous kernel.
+//
+// Per level, stress and divergence: 1026 x 1026 nodes 21.9 -> 14.6 us in FP32 (122 MB,
+// mostly out of L2), 144 -> 131 us in FP64 (its pipe); 66 x 66 7.2 -> 3.6 us and 11.3 -> 7.1
+// us.  A fused form (u, metrics and fluxes of a tile in shared memory) took 6.9 us at
+// 66^2 and 38 us at 1026^2 in FP32.
 // ---------------------------------------------------------------------------
-// The block's nodes and their 2-node reach lie in rows and columns 4 .. n - 5
-// (every difference central, every node an unknown): uniform per block.
-__device__ __forceinline__ bool curv_block_inner(const Geom& g) {
-  const int x0 = blockIdx.x * blockDim.x, y0 = blockIdx.y * blockDim.y;
-  return x0 >= 4 && x0 + (int)blockDim.x - 1 <= g.n[0] - 5 && y0 >= 4 && y0 + (int)blockDim.y - 1 <= g.n[1] - 5;
+struct CurvPart {
+  int xa, ngx, nr;  // first column of the rectangle, its groups per row, its rows (from row 4)
+  int nfc;          // frame columns in the rectangle's rows
+  int nbf;          // blocks of frame nodes, in front
+  int frame;        // frame nodes
+};
+constexpr int CURV_THREADS = 64;
+
+template <typename T>
+struct Vec16;
+template <>
+struct Vec16<float> {
+  using type = float4;
+};
+template <>
+struct Vec16<double> {
+  using type = double2;
+};
+// W vectors of 16 bytes at p (aligned), s elements apart
+template <typename T, int W>
+__device__ __forceinline__ void ld16(const T* p, T (*out)[16 / sizeof(T)], int s = 16 / sizeof(T)) {
+#pragma unroll
+  for (int k = 0; k < W; ++k)
+    *reinterpret_cast<typename Vec16<T>::type*>(out[k]) = *reinterpret_cast<const typename Vec16<T>::type*>(p + k * s);
+}
+template <typename T>
+__device__ __forceinline__ void st16(T* p, const T* v) {
+  *reinterpret_cast<typename Vec16<T>::type*>(p) = *reinterpret_cast<const typename Vec16<T>::type*>(v);
+}
+
+// Central differences of a group at v: along x from the 16 bytes before, at and
+// after it, along y from the rows at -2, -1, 1 and 2.
+template <typename T>
+__device__ __forceinline__ void curv_dx(const T* v, T* d) {
+  constexpr int V = 16 / sizeof(T);
+  alignas(16) T w[3][V];
+  ld16<T, 3>(v - V, w);
+  const T* const c = &w[0][0] + V;
+#pragma unroll
+  for (int k = 0; k < V; ++k) d[k] = c4(c[k - 2], c[k - 1], c[k + 1], c[k + 2]);
+}
+template <typename T>
+__device__ __forceinline__ void curv_dy(const T* v, int sy, T* d) {
+  constexpr int V = 16 / sizeof(T);
+  alignas(16) T lo[2][V], hi[2][V];
+  ld16<T, 2>(v - 2 * sy, lo, sy);
+  ld16<T, 2>(v + sy, hi, sy);
+#pragma unroll
+  for (int k = 0; k < V; ++k) d[k] = c4(lo[0][k], lo[1][k], hi[0][k], hi[1][k]);
+}
+
+// Position of a thread: frame node (true) or first node of a group; x < 0: none.
+__device__ __forceinline__ bool curv_pos(const Geom& g, const CurvPart& c, int V, int& x, int& y) {
+  x = -1;
+  if ((int)blockIdx.x < c.nbf) {
+    int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= c.frame) return true;
+    if (j < 8 * g.n[0]) {
+      y = j / g.n[0];
+      x = j - y * g.n[0];
+      if (y >= 4) y += g.n[1] - 8;
+    } else {
+      j -= 8 * g.n[0];
+      y = j / c.nfc;
+      x = j - y * c.nfc;
+      if (x >= c.xa) x += c.ngx * V;
+      y += 4;
+    }
+    return true;
+  }
+  const int i = (blockIdx.x - c.nbf) * blockDim.x + threadIdx.x;
+  if (i >= c.ngx * c.nr) return false;
+  y = i / c.ngx;
+  x = c.xa + (i - y * c.ngx) * V;
+  y += 4;
+  return false;
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) curv_stress2d(Geom g, const T* __restrict__ u, const T* __restrict__ lam,
-                                                     const T* __restrict__ mu, const T* __restrict__ met,
-                                                     T* __restrict__ sig) {
-  if (g.dim != 2) return;
-  pdl_wait();
-  pdl_trigger();
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int rhs = blockIdx.z;
-  if (x >= g.n[0] || y >= g.n[1]) return;
-  const long long sy = g.np[0];
-  const long long pc = pidx(g, 0, 0, x, y, 0);
-  const T* U = u + pidx(g, rhs, 0, x, y, 0);
-  const T* V = U + g.field;
-  T uq, ur, vq, vr;
-  if (curv_block_inner(g)) {  // central differences, 32-bit offsets
-    const int s1 = g.np[0];
-    uq = c4(U[-2], U[-1], U[1], U[2]);
-    vq = c4(V[-2], V[-1], V[1], V[2]);
-    ur = c4(U[-2 * s1], U[-s1], U[s1], U[2 * s1]);
-    vr = c4(V[-2 * s1], V[-s1], V[s1], V[2 * s1]);
-  } else {
-    uq = sbp_d1<T>(U, 1, x, g.n[0]);
-    ur = sbp_d1<T>(U, sy, y, g.n[1]);
-    vq = sbp_d1<T>(V, 1, x, g.n[0]);
-    vr = sbp_d1<T>(V, sy, y, g.n[1]);
-  }
-  const T a0 = met[pc], a1 = met[g.field + pc], a2 = met[2 * g.field + pc], a3 = met[3 * g.field + pc];
+__device__ __forceinline__ void curv_flux(T uq, T ur, T vq, T vr, T a0, T a1, T a2, T a3, T l, T m, T* o0, T* o1, T* o2,
+                                          T* o3) {
   const T u_x = a0 * uq + a2 * ur, u_y = a1 * uq + a3 * ur;  // J times the physical gradient
   const T v_x = a0 * vq + a2 * vr, v_y = a1 * vq + a3 * vr;
-  const T l = lam[pc], m = mu[pc];                            // lambda / J, mu / J
   const T div = u_x + v_y;
   const T sxx = l * div + T(2) * m * u_x, syy = l * div + T(2) * m * v_y, sxy = m * (u_y + v_x);
-  T* out = sig + (long long)rhs * 4 * g.field + pc;
-  out[0] = a0 * sxx + a1 * sxy;
-  out[g.field] = a2 * sxx + a3 * sxy;
-  out[2 * g.field] = a0 * sxy + a1 * syy;
-  out[3 * g.field] = a2 * sxy + a3 * syy;
+  *o0 = a0 * sxx + a1 * sxy;
+  *o1 = a2 * sxx + a3 * sxy;
+  *o2 = a0 * sxy + a1 * syy;
+  *o3 = a2 * sxy + a3 * syy;
+}
+
+// The closure taps into shared memory (frame blocks; blockDim.x >= 32)
+template <typename T>
+__device__ __forceinline__ void curv_taps(const S3Taps<T>& tp, S3Taps<T>& st) {
+  for (int i = threadIdx.x; i < 36; i += blockDim.x) st.off[i] = tp.off[i], st.w[i] = tp.w[i];
+  __syncthreads();
+}
+
+template <typename T>
+__global__ void __launch_bounds__(CURV_THREADS) curv_stress2d(Geom g, CurvPart cp, const T* __restrict__ u,
+                                                              const T* __restrict__ lam, const T* __restrict__ mu,
+                                                              const T* __restrict__ met, T* __restrict__ sig,
+                                                              const __grid_constant__ S3Taps<T> tp) {
+  if (g.dim != 2) return;
+  constexpr int V = 16 / sizeof(T);
+  int x, y;
+  const bool frame = curv_pos(g, cp, V, x, y);
+  const int rhs = blockIdx.y;
+  const long long pc = x < 0 ? 0 : pidx(g, 0, 0, x, y, 0);  // lam, mu: lambda / J, mu / J
+  const T* const U = u + (long long)rhs * 2 * g.field + pc;
+  T* const out = sig + (long long)rhs * 4 * g.field + pc;
+  if (frame) {
+    __shared__ S3Taps<T> taps;
+    curv_taps(tp, taps);
+    const T l = lam[pc], m = mu[pc], a0 = met[pc], a1 = met[g.field + pc], a2 = met[2 * g.field + pc];
+    const T a3 = met[3 * g.field + pc];
+    pdl_wait();
+    pdl_trigger();
+    if (x < 0) return;
+    const T* const Vv = U + g.field;
+    const int sy = g.np[0], cx = s3_class(x, g.n[0]), cy = s3_class(y, g.n[1]);
+    const T w = T(1.0 / 12.0);
+    const T uq = w * s3_taps12(U, 1, cx, taps), ur = w * s3_taps12(U, sy, cy, taps);
+    const T vq = w * s3_taps12(Vv, 1, cx, taps), vr = w * s3_taps12(Vv, sy, cy, taps);
+    curv_flux(uq, ur, vq, vr, a0, a1, a2, a3, l, m, out, out + g.field, out + 2 * g.field, out + 3 * g.field);
+    return;
+  }
+  alignas(16) T a[4][V], l[1][V], m[1][V];
+  if (x >= 0) {
+#pragma unroll
+    for (int k = 0; k < 4; ++k) ld16<T, 1>(met + k * g.field + pc, a + k);
+    ld16<T, 1>(lam + pc, l);
+    ld16<T, 1>(mu + pc, m);
+  }
+  pdl_wait();
+  pdl_trigger();
+  if (x < 0) return;
+  const int sy = g.np[0];
+  T uq[V], ur[V], vq[V], vr[V];
+  curv_dx(U, uq);
+  curv_dx(U + g.field, vq);
+  curv_dy(U, sy, ur);
+  curv_dy(U + g.field, sy, vr);
+  alignas(16) T o[4][V];
+#pragma unroll
+  for (int k = 0; k < V; ++k)
+    curv_flux(uq[k], ur[k], vq[k], vr[k], a[0][k], a[1][k], a[2][k], a[3][k], l[0][k], m[0][k], &o[0][k], &o[1][k],
+              &o[2][k], &o[3][k]);
+#pragma unroll
+  for (int k = 0; k < 4; ++k) st16(out + k * g.field, o[k]);
 }
 
 template <typename T, int MODE, bool FORCED>
-__global__ void __launch_bounds__(256) curv_div2d(Geom g, WaveFields<T> f, StepScalars s) {
+__global__ void __launch_bounds__(CURV_THREADS) curv_div2d(Geom g, CurvPart cp, WaveFields<T> f, StepScalars s,
+                                                           const __grid_constant__ S3Taps<T> tp) {
   if (g.dim != 2) return;
-  pdl_wait();
-  pdl_trigger();
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y * blockDim.y + threadIdx.y;
-  const int rhs = blockIdx.z;
-  if (!is_unknown(g, x, y, 0)) return;
-  const long long sy = g.np[0];
-  const long long pc = pidx(g, 0, 0, x, y, 0);
-  const T* fqu = f.sigma + (long long)rhs * 4 * g.field + pc;
-  const T* fru = fqu + g.field;
-  const T* fqv = fqu + 2 * g.field;
-  const T* frv = fqu + 3 * g.field;
-  if (curv_block_inner(g)) {  // central differences, no boundary terms
-    const int s1 = g.np[0];
-    const T ku = -c4(fqu[-2], fqu[-1], fqu[1], fqu[2]) - c4(fru[-2 * s1], fru[-s1], fru[s1], fru[2 * s1]);
-    const T kv = -c4(fqv[-2], fqv[-1], fqv[1], fqv[2]) - c4(frv[-2 * s1], frv[-s1], frv[s1], frv[2 * s1]);
-    const T irh = f.irh2[pc];
-    const long long p0 = pidx(g, rhs, 0, x, y, 0);
-    leapfrog_update<T, MODE, FORCED>(f, p0, f.u_cur[p0], ku * irh, s);
-    leapfrog_update<T, MODE, FORCED>(f, p0 + g.field, f.u_cur[p0 + g.field], kv * irh, s);
+  constexpr int V = 16 / sizeof(T);
+  int x, y;
+  const bool frame = curv_pos(g, cp, V, x, y);
+  const int rhs = blockIdx.y;
+  const long long pc = x < 0 ? 0 : pidx(g, 0, 0, x, y, 0);
+  const long long p0 = (long long)rhs * 2 * g.field + pc;
+  const T* const fqu = f.sigma + (long long)rhs * 4 * g.field + pc;
+  const T* const fru = fqu + g.field;
+  const T* const fqv = fqu + 2 * g.field;
+  const T* const frv = fqu + 3 * g.field;
+  if (frame) {
+    __shared__ S3Taps<T> taps;
+    curv_taps(tp, taps);
+    const bool unk = x >= 0 && is_unknown(g, x, y, 0);
+    const T irh = f.irh2[pc];  // 1 / (rho J h^2)
+    const T fr0 = FORCED ? f.frho[p0] : T(0), fr1 = FORCED ? f.frho[p0 + g.field] : T(0);
+    pdl_wait();
+    pdl_trigger();
+    if (!unk) return;
+    constexpr bool RD = MODE == STEP_MID || MODE == STEP_LAST;
+    const T u0 = f.u_cur[p0], u1 = f.u_cur[p0 + g.field];
+    const T d0 = RD ? f.delta[p0] : T(0), d1 = RD ? f.delta[p0 + g.field] : T(0);
+    const T a0 = RD ? f.acc[p0] : T(0), a1 = RD ? f.acc[p0 + g.field] : T(0);
+    const int sy = g.np[0], cx = s3_class(x, g.n[0]), cy = s3_class(y, g.n[1]);
+    const T w = T(-1.0 / 12.0), ih = T(48.0 / 17.0);
+    const T bx = x == 0 ? -ih : (x == g.n[0] - 1 ? ih : T(0)), by = y == 0 ? -ih : (y == g.n[1] - 1 ? ih : T(0));
+    const T ku = w * (s3_taps12(fqu, 1, cx, taps) + s3_taps12(fru, sy, cy, taps)) + bx * fqu[0] + by * fru[0];
+    const T kv = w * (s3_taps12(fqv, 1, cx, taps) + s3_taps12(frv, sy, cy, taps)) + bx * fqv[0] + by * frv[0];
+    leapfrog_update_pre<T, MODE, FORCED>(f, p0, u0, ku * irh, s, d0, a0, fr0);
+    leapfrog_update_pre<T, MODE, FORCED>(f, p0 + g.field, u1, kv * irh, s, d1, a1, fr1);
     return;
   }
-  T ku = -sbp_d1<T>(fqu, 1, x, g.n[0]) - sbp_d1<T>(fru, sy, y, g.n[1]);
-  T kv = -sbp_d1<T>(fqv, 1, x, g.n[0]) - sbp_d1<T>(frv, sy, y, g.n[1]);
-  const T inv_h0 = T(48.0 / 17.0);
-  if (x == 0) {
-    ku -= inv_h0 * fqu[0];
-    kv -= inv_h0 * fqv[0];
-  } else if (x == g.n[0] - 1) {
-    ku += inv_h0 * fqu[0];
-    kv += inv_h0 * fqv[0];
-  }
-  if (y == 0) {
-    ku -= inv_h0 * fru[0];
-    kv -= inv_h0 * frv[0];
-  } else if (y == g.n[1] - 1) {
-    ku += inv_h0 * fru[0];
-    kv += inv_h0 * frv[0];
-  }
-  const T irh = f.irh2[pc];  // 1 / (rho J h^2)
-  const long long p0 = pidx(g, rhs, 0, x, y, 0);
-  leapfrog_update<T, MODE, FORCED>(f, p0, f.u_cur[p0], ku * irh, s);
-  leapfrog_update<T, MODE, FORCED>(f, p0 + g.field, f.u_cur[p0 + g.field], kv * irh, s);
-}
-
-// Fused form of the two kernels above: one launch per time level, blocks of
-// 32 x 8 threads and 32 x (8 RPT) output nodes (RPT rows per thread).  The
-// block stages u (both components) and the six coefficient planes (y_r, -x_r,
-// -y_q, x_q, lambda / J, mu / J) on a tile of (32 + 6) x (8 RPT + 6) nodes in
-// shared memory, then forms the four fluxes in place of the first four
-// planes.  The tile starts 2 nodes before the block, or at n - 6 when that is
-// lower, so it holds every flux a central or SBP-closure difference of the
-// block's nodes reads.  Blocks whose tile lies in rows and columns 4 .. n - 5
-// (every difference central, every node an unknown) take a path with no
-// per-node tests; the others difference fluxes at nodes within 4 of a side
-// with the SBP closure applied to u in global memory.  Every load is issued
-// before the first barrier: the coefficients (static) ahead of the wait on the
-// previous level, the state and the update's operands after it.
-template <typename T, int MODE, bool FORCED, int RPT>
-__global__ void __launch_bounds__(256) curv_step2d(Geom g, WaveFields<T> f, StepScalars s) {
-  if (g.dim != 2) return;
-  constexpr int TX = 32, TY = 8 * RPT;
-  constexpr int FX = TX + 6, FY = TY + 6;  // flux / coefficient tile
-  constexpr int UX = FX + 4, UY = FY + 4;  // u tile: 2-node reach of the central fluxes
-  __shared__ T su[2][UY][UX];
-  __shared__ T sc[6][FY][FX];
-  const int nx = g.n[0], ny = g.n[1];
-  const int rhs = blockIdx.z;
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-  const int xs = min(x0 - 2, nx - 6), ys = min(y0 - 2, ny - 6);
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int sy = g.np[0];
-  const int fld = (int)g.field;  // one padded component indexes in 32 bits
-  const bool inner = xs >= 4 && xs + FX - 1 <= nx - 5 && ys >= 4 && ys + FY - 1 <= ny - 5;
-  const long long cbase = pidx(g, 0, 0, xs, ys, 0);  // coefficient tile origin
-  const T* M0 = f.met + cbase;
-  const T* LA = f.lam + cbase;
-  const T* MU = f.mu + cbase;
-  if (inner) {
-    for (int r = ty; r < FY; r += 8)
-      for (int c = tx; c < FX; c += 32) {
-        const int q = r * sy + c;
-        sc[0][r][c] = M0[q];
-        sc[1][r][c] = M0[fld + q];
-        sc[2][r][c] = M0[2 * fld + q];
-        sc[3][r][c] = M0[3 * fld + q];
-        sc[4][r][c] = LA[q];
-        sc[5][r][c] = MU[q];
-      }
-  } else {
-    for (int r = ty; r < FY; r += 8)
-      for (int c = tx; c < FX; c += 32) {
-        const int gx = xs + c, gy = ys + r;
-        const bool in = gx >= 0 && gx < nx && gy >= 0 && gy < ny;
-        const int q = r * sy + c;
-        sc[0][r][c] = in ? M0[q] : T(0);
-        sc[1][r][c] = in ? M0[fld + q] : T(0);
-        sc[2][r][c] = in ? M0[2 * fld + q] : T(0);
-        sc[3][r][c] = in ? M0[3 * fld + q] : T(0);
-        sc[4][r][c] = in ? LA[q] : T(0);
-        sc[5][r][c] = in ? MU[q] : T(0);
-      }
-  }
-  // this thread's output nodes: (x0 + tx, y0 + ty + 8 k)
-  const int x = x0 + tx;
-  const long long p00 = pidx(g, rhs, 0, x, y0 + ty, 0);
-  const long long c00 = pidx(g, 0, 0, x, y0 + ty, 0);
-  bool unk[RPT];
-  T irh[RPT], fr0[RPT], fr1[RPT];
-#pragma unroll
-  for (int k = 0; k < RPT; ++k) {
-    unk[k] = inner || is_unknown(g, x, y0 + ty + 8 * k, 0);
-    irh[k] = unk[k] ? f.irh2[c00 + 8 * k * sy] : T(0);  // 1 / (rho J h^2)
-    fr0[k] = (FORCED && unk[k]) ? f.frho[p00 + 8 * k * sy] : T(0);
-    fr1[k] = (FORCED && unk[k]) ? f.frho[p00 + 8 * k * sy + fld] : T(0);
+  alignas(16) T irh[1][V], fr[2][V];
+  if (x >= 0) {
+    ld16<T, 1>(f.irh2 + pc, irh);
+    if (FORCED) ld16<T, 1>(f.frho + p0, fr), ld16<T, 1>(f.frho + p0 + g.field, fr + 1);
   }
   pdl_wait();
   pdl_trigger();
-  const T* U0 = f.u_cur + pidx(g, rhs, 0, 0, 0, 0);
-  {
-    const T* Ut = f.u_cur + pidx(g, rhs, 0, xs - 2, ys - 2, 0);  // inside the padding (PAD >= 4)
-    for (int r = ty; r < UY; r += 8)
-      for (int c = tx; c < UX; c += 32) {
-        const int gx = xs - 2 + c, gy = ys - 2 + r;
-        const bool in = inner || (gx >= 0 && gx < nx && gy >= 0 && gy < ny);
-        const int q = r * sy + c;
-        su[0][r][c] = in ? Ut[q] : T(0);
-        su[1][r][c] = in ? Ut[fld + q] : T(0);
-      }
-  }
-  T d0[RPT], d1[RPT], ac0[RPT], ac1[RPT];
+  if (x < 0) return;
+  const int sy = g.np[0];
+  alignas(16) T uv[2][V], dl[2][V], ac[2][V], dq[2][V], dr[2][V];
 #pragma unroll
-  for (int k = 0; k < RPT; ++k) {
-    const bool ld = MODE != 3 && MODE != STEP_FIRST && unk[k];
-    const long long p = p00 + 8 * k * sy;
-    d0[k] = ld ? f.delta[p] : T(0);
-    d1[k] = ld ? f.delta[p + fld] : T(0);
-    ac0[k] = ld ? f.acc[p] : T(0);
-    ac1[k] = ld ? f.acc[p + fld] : T(0);
+  for (int c = 0; c < 2; ++c) {  // all loads before the first store
+    const long long p = p0 + c * g.field;
+    ld16<T, 1>(f.u_cur + p, uv + c);
+    if (MODE == STEP_MID || MODE == STEP_LAST) ld16<T, 1>(f.delta + p, dl + c), ld16<T, 1>(f.acc + p, ac + c);
+    curv_dx(c ? fqv : fqu, dq[c]);
+    curv_dy(c ? frv : fru, sy, dr[c]);
   }
-  __syncthreads();
-  for (int r = ty; r < FY; r += 8)
-    for (int c = tx; c < FX; c += 32) {
-      const int gx = xs + c, gy = ys + r;
-      T uq, ur, vq, vr;
-      const int ux = c + 2, uy = r + 2;
-      if (inner || (gx >= 4 && gx <= nx - 5)) {
-        uq = c4(su[0][uy][ux - 2], su[0][uy][ux - 1], su[0][uy][ux + 1], su[0][uy][ux + 2]);
-        vq = c4(su[1][uy][ux - 2], su[1][uy][ux - 1], su[1][uy][ux + 1], su[1][uy][ux + 2]);
-      } else {
-        if (gx < 0 || gx >= nx || gy < 0 || gy >= ny) continue;  // never read
-        const long long q = (long long)gy * sy + gx;
-        uq = sbp_d1<T>(U0 + q, 1, gx, nx);
-        vq = sbp_d1<T>(U0 + fld + q, 1, gx, nx);
-      }
-      if (inner || (gy >= 4 && gy <= ny - 5)) {
-        ur = c4(su[0][uy - 2][ux], su[0][uy - 1][ux], su[0][uy + 1][ux], su[0][uy + 2][ux]);
-        vr = c4(su[1][uy - 2][ux], su[1][uy - 1][ux], su[1][uy + 1][ux], su[1][uy + 2][ux]);
-      } else {
-        if (gx < 0 || gx >= nx || gy < 0 || gy >= ny) continue;  // never read
-        const long long q = (long long)gy * sy + gx;
-        ur = sbp_d1<T>(U0 + q, sy, gy, ny);
-        vr = sbp_d1<T>(U0 + fld + q, sy, gy, ny);
-      }
-      const T a0 = sc[0][r][c], a1 = sc[1][r][c], a2 = sc[2][r][c], a3 = sc[3][r][c];
-      const T l = sc[4][r][c], m = sc[5][r][c];
-      const T u_x = a0 * uq + a2 * ur, u_y = a1 * uq + a3 * ur;
-      const T v_x = a0 * vq + a2 * vr, v_y = a1 * vq + a3 * vr;
-      const T div = u_x + v_y;
-      const T sxx = l * div + T(2) * m * u_x, syy = l * div + T(2) * m * v_y, sxy = m * (u_y + v_x);
-      sc[0][r][c] = a0 * sxx + a1 * sxy;
-      sc[1][r][c] = a2 * sxx + a3 * sxy;
-      sc[2][r][c] = a0 * sxy + a1 * syy;
-      sc[3][r][c] = a2 * sxy + a3 * syy;
-    }
-  __syncthreads();
-  const int lx = x - xs;
 #pragma unroll
-  for (int k = 0; k < RPT; ++k) {
-    if (!unk[k]) continue;
-    const int y = y0 + ty + 8 * k;
-    const int ly = y - ys;
-    const T* fqu = &sc[0][ly][lx];
-    const T* fru = &sc[1][ly][lx];
-    const T* fqv = &sc[2][ly][lx];
-    const T* frv = &sc[3][ly][lx];
-    T ku, kv;
-    if (inner || (x >= 4 && x <= nx - 5)) {
-      ku = -c4(fqu[-2], fqu[-1], fqu[1], fqu[2]);
-      kv = -c4(fqv[-2], fqv[-1], fqv[1], fqv[2]);
-    } else {
-      ku = -sbp_d1<T>(fqu, 1, x, nx);
-      kv = -sbp_d1<T>(fqv, 1, x, nx);
-    }
-    if (inner || (y >= 4 && y <= ny - 5)) {
-      ku -= c4(fru[-2 * FX], fru[-FX], fru[FX], fru[2 * FX]);
-      kv -= c4(frv[-2 * FX], frv[-FX], frv[FX], frv[2 * FX]);
-    } else {
-      ku -= sbp_d1<T>(fru, FX, y, ny);
-      kv -= sbp_d1<T>(frv, FX, y, ny);
-    }
-    if (!inner) {
-      const T inv_h0 = T(48.0 / 17.0);
-      if (x == 0) {
-        ku -= inv_h0 * fqu[0];
-        kv -= inv_h0 * fqv[0];
-      } else if (x == nx - 1) {
-        ku += inv_h0 * fqu[0];
-        kv += inv_h0 * fqv[0];
+  for (int c = 0; c < 2; ++c) {
+    const long long p = p0 + c * g.field;
+    alignas(16) T un[V];
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      T a = (-dq[c][k] - dr[c][k]) * irh[0][k];
+      if (MODE == 3) {  // operator only
+        un[k] = a;
+        continue;
       }
-      if (y == 0) {
-        ku -= inv_h0 * fru[0];
-        kv -= inv_h0 * frv[0];
-      } else if (y == ny - 1) {
-        ku += inv_h0 * fru[0];
-        kv += inv_h0 * frv[0];
-      }
+      if (FORCED) a += fr[c][k] * T(s.cosn);
+      const T d = MODE == STEP_FIRST ? T(-0.5) * T(s.kt) * a : dl[c][k] - T(s.kt) * a;
+      un[k] = uv[c][k] + d;
+      ac[c][k] = MODE == STEP_FIRST ? T(s.w0) * uv[c][k] + T(s.wnew) * un[k] : ac[c][k] + T(s.wnew) * un[k];
+      dl[c][k] = d;
     }
-    const long long p = p00 + 8 * k * sy;
-    leapfrog_update_pre<T, MODE, FORCED>(f, p, su[0][ly + 2][lx + 2], ku * irh[k], s, d0[k], ac0[k], fr0[k]);
-    leapfrog_update_pre<T, MODE, FORCED>(f, p + fld, su[1][ly + 2][lx + 2], kv * irh[k], s, d1[k], ac1[k], fr1[k]);
+    if (MODE != STEP_LAST) st16(f.u_next + p, un);
+    if (MODE == STEP_FIRST || MODE == STEP_MID) st16(f.delta + p, dl[c]);
+    if (MODE != 3) st16(f.acc + p, ac[c]);
   }
 }
 
@@ -1319,25 +1277,23 @@ static cudaError_t launch_mode(const Geom& g, int order, const WaveFields<T>& f,
     if (nl) *nl += 1;
     return cudaGetLastError();
   }
-  if (g.mapped) {  // curvilinear 2D order 4: fused 32x8 (0) or 32x16 (2, FP32), stress + divergence (1)
-    const int cv = curv_variant(g);
-    if (cv != 1) {
-      cudaError_t e;
-      if (cv == 2 && sizeof(T) == 4) {  // 32 x 16 outputs per block
-        dim3 blk(32, 8), grd((g.n[0] + 31) / 32, (g.n[1] + 15) / 16, g.nrhs);
-        e = launch_k(curv_step2d<T, MODE, FORCED, sizeof(T) == 4 ? 2 : 1>, grd, blk, st, g, f, s);
-      } else {
-        dim3 blk(32, 8), grd((g.n[0] + 31) / 32, (g.n[1] + 7) / 8, g.nrhs);
-        e = launch_k(curv_step2d<T, MODE, FORCED, 1>, grd, blk, st, g, f, s);
-      }
-      if (e != cudaSuccess) return e;
-      if (nl) *nl += 1;
-      return cudaGetLastError();
-    }
-    dim3 blk(32, 8), grd((g.n[0] + 31) / 32, (g.n[1] + 7) / 8, g.nrhs);
-    cudaError_t e = launch_k(curv_stress2d<T>, grd, blk, st, g, (const T*)f.u_cur, f.lam, f.mu, f.met, f.sigma);
+  if (g.mapped) {  // curvilinear 2D order 4: stress + divergence
+    constexpr int V = 16 / sizeof(T);
+    CurvPart cp;
+    cp.xa = 4 + (V - (4 + g.padx) % V) % V;
+    cp.nr = g.n[1] - 8;
+    cp.ngx = cp.nr > 0 ? std::max(0, (g.n[0] - 4 - cp.xa) / V) : 0;
+    cp.nfc = g.n[0] - V * cp.ngx;
+    cp.frame = 8 * g.n[0] + cp.nfc * cp.nr;
+    // blocks of 64 threads (1026^2 FP32: 14.6 us a level, with 256 14.9, with 32 19.0), of one
+    // warp where those would leave SMs short (202^2 FP64: 8.9 us, with 64 12.0)
+    const int nt = (long long)(cp.frame + cp.ngx * cp.nr) * g.nrhs < 4LL * 152 * CURV_THREADS ? 32 : CURV_THREADS;
+    cp.nbf = (cp.frame + nt - 1) / nt;
+    dim3 blk(nt), grd(cp.nbf + (cp.ngx * cp.nr + nt - 1) / nt, g.nrhs);
+    cudaError_t e = launch_k(curv_stress2d<T>, grd, blk, st, g, cp, (const T*)f.u_cur, f.lam, f.mu, f.met, f.sigma,
+                             s3_taps<T>());
     if (e != cudaSuccess) return e;
-    e = launch_k(curv_div2d<T, MODE, FORCED>, grd, blk, st, g, f, s);
+    e = launch_k(curv_div2d<T, MODE, FORCED>, grd, blk, st, g, cp, f, s, s3_taps<T>());
     if (e != cudaSuccess) return e;
     if (nl) *nl += 2;
     return cudaGetLastError();
