@@ -2544,40 +2544,47 @@ const char* ewh_batch_last_error(const ewh_batch* b) { return b ? b->err.c_str()
 
 ewh_status ewh_batch_apply_S(ewh_batch* b, const double* const* v_in, double* const* v_out) {
   if (!b || !v_in || !v_out) return EWH_EINVAL;
-  std::vector<int> members;
-  for (int k = 0; k < (int)b->p.size(); ++k) {
-    members.push_back(k);
-    const ewh_status s0 = b->precision == EWH_FP64 ? ensure_graph<double>(b->p[k], false)
-                                                   : ensure_graph<float>(b->p[k], false);
-    if (s0 != EWH_OK) return bfail(b, s0, b->p[k]->err);
+  const bool f64 = b->precision == EWH_FP64;
+  // Each member's own step graph, captured once, between its pack and unpack: the
+  // members side by side, or one after another when one of them runs on chip (see
+  // capture_branches).  A graph that has to be built is built while the members before
+  // it run.  Capturing all levels of all members anew for every call took 2.2 ms of 33.6 with
+  // per-level launches
+  // (258, 386 and 514 nodes a side, 22 right-hand sides each, FP32).
+  bool serial = false;
+  for (ewh_ctx* c : b->p) {  // variants first: the members' timings must not overlap
+    if (f64 && c->w64.variant < 0 && !c->w64.graph_S) autotune<double>(c, c->w64);
+    if (!f64 && c->w32.variant < 0 && !c->w32.graph_S) autotune<float>(c, c->w32);
+    serial = serial || (!f64 && is_resident_variant(c->w32.variant));
   }
-  cudaEventRecord(b->fork, b->user_stream);
-  cudaStreamWaitEvent(b->master, b->fork, 0);
-  cudaGraphExec_t ge = nullptr;
-  auto body = [&](int k) -> ewh_status {
-    ewh_ctx* ctx = b->p[k];
-    if (b->precision == EWH_FP64) {
-      Wave<double>& w = ctx->w64;
-      if (launch_pack<double>(ctx->g, v_in[k], w.u_a, ctx->st) != cudaSuccess) return EWH_ECUDA;
-      long long cnt = 0;
-      if (enqueue_steps<double>(ctx, w, false, &cnt) != cudaSuccess) return EWH_ECUDA;
-      if (launch_unpack<double>(ctx->g, w.acc, v_out[k], nullptr, ctx->st) != cudaSuccess) return EWH_ECUDA;
-      b->launches += cnt + 2;
-    } else {
-      Wave<float>& w = ctx->w32;
-      if (launch_pack<float>(ctx->g, v_in[k], w.u_a, ctx->st) != cudaSuccess) return EWH_ECUDA;
-      long long cnt = 0;
-      if (enqueue_steps<float>(ctx, w, false, &cnt) != cudaSuccess) return EWH_ECUDA;
-      if (launch_unpack<float>(ctx->g, w.acc, v_out[k], nullptr, ctx->st) != cudaSuccess) return EWH_ECUDA;
-      b->launches += cnt + 2;
-    }
-    return EWH_OK;
+  cudaError_t e = cudaEventRecord(b->fork, b->user_stream);
+  if (e == cudaSuccess) e = cudaStreamWaitEvent(b->master, b->fork, 0);
+  if (e == cudaSuccess) e = cudaEventRecord(b->fork, b->master);
+  cudaEvent_t prev = b->fork;
+  ewh_status st = EWH_OK;
+  int at = 0;
+  auto run = [&](auto& w, ewh_ctx* ctx, int k) {
+    using T = std::remove_reference_t<decltype(*w.u_a)>;
+    st = ensure_graph<T>(ctx, false);
+    if (st != EWH_OK) return cudaSuccess;
+    cudaError_t r = cudaStreamWaitEvent(ctx->st, serial ? prev : b->fork, 0);
+    if (r == cudaSuccess) r = launch_pack<T>(ctx->g, v_in[k], w.u_a, ctx->st);
+    if (r == cudaSuccess) r = cudaGraphLaunch(w.graph_S, ctx->st);
+    if (r == cudaSuccess) r = launch_unpack<T>(ctx->g, w.acc, v_out[k], nullptr, ctx->st);
+    b->launches += w.graph_S_kernels + 2;
+    // joined on an error too
+    const cudaError_t r2 = cudaEventRecord(b->joins[k], ctx->st);
+    if (r2 == cudaSuccess) cudaStreamWaitEvent(b->master, b->joins[k], 0);
+    prev = b->joins[k];
+    return r != cudaSuccess ? r : r2;
   };
-  ewh_status s = capture_branches(b, members, body, &ge);
-  if (s != EWH_OK) return s;
-  cudaError_t e = cudaGraphLaunch(ge, b->master);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(b->master);
-  cudaGraphExecDestroy(ge);
+  for (int k = 0; k < (int)b->p.size() && e == cudaSuccess && st == EWH_OK; ++k) {
+    at = k;
+    e = f64 ? run(b->p[k]->w64, b->p[k], k) : run(b->p[k]->w32, b->p[k], k);
+  }
+  const cudaError_t e2 = cudaStreamSynchronize(b->master);
+  if (st != EWH_OK) return bfail(b, st, b->p[at]->err);
+  if (e == cudaSuccess) e = e2;
   if (e != cudaSuccess) return bfail(b, EWH_ECUDA, std::string("batch apply failed: ") + cudaGetErrorString(e));
   cudaEventRecord(b->fork, b->master);
   cudaStreamWaitEvent(b->user_stream, b->fork, 0);
