@@ -107,12 +107,9 @@ def kernel_source_hash():
 
 def step_kernel_name(variant):
     """The 2D order-4 FP32 step kernel behind an autotuner variant number."""
-    tiles = {0: "32x8", 1: "32x16", 2: "64x8", 3: "64x4"}
     shapes = {5: "1024, 4", 6: "768, 5", 7: "512, 7"}
-    if variant in tiles:
-        return "sbp_stress2d_tl + sbp_div2d_tl (%s tiles), per time level" % tiles[variant]
-    if variant == 4:
-        return "step2d_o4_fused, per time level"
+    if variant == 0:
+        return "sbp_stress2d + sbp_div2d, per time level"
     if variant in shapes:
         return "step2d_o4_resident<%s> (all levels of a wave solve in one cooperative launch), per time level" % shapes[variant]
     return "unknown variant %d" % variant

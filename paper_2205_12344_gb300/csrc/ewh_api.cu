@@ -65,14 +65,14 @@ struct Wave {
   long long cg_loop_kernels = 0;  // kernels of one pass
 };
 
-// step-kernel variants of the 2D order-4 FP32 solve beyond the launcher's
-// own (split tiles 0..3, fused 4): 5 + shape = resident solve of that shape
+// step-kernel variants of the 2D order-4 FP32 solve beyond the launcher's own
+// pair (0): 5 + shape = resident solve of that shape
 constexpr int VARIANT_RESIDENT = 5;
 // least nodes per CTA block of a batch member's on-chip solve (resident_ok)
 constexpr long long RS_BATCH_MIN_BLOCK = 2048;
 // longest window of CG iterations under device control between host polls
 constexpr int CG_WINDOW_MAX = 256;
-static_assert(VARIANT_RESIDENT + RS_SHAPES == YM_VARIANT, "2D order-4 variants: split 0..3, fused 4, resident, y-march");
+static_assert(VARIANT_RESIDENT + RS_SHAPES == YM_VARIANT, "2D order-4 variants: pair 0, resident 5..7, y-march 8");
 inline bool is_resident_variant(int v) { return v >= VARIANT_RESIDENT && v < VARIANT_RESIDENT + RS_SHAPES; }
 
 }  // namespace
@@ -322,8 +322,8 @@ Wave<float>& wave_of<float>(ewh_ctx* c) { return c->w32; }
 // ---------------------------------------------------------------------------
 // Autotuner: pick the step-kernel variant of a context by timing.
 //
-// The candidates (split or fused order-4 2D kernel; tile height of the
-// order-2 2D kernel) are timed on the context's own buffers with 2 warm-up and
+// The candidates (order-4 pair, fixed-point, marching and on-chip forms; tile
+// height of the order-2 2D kernel or its on-chip form) are timed on the context's own buffers with 2 warm-up and
 // 8 timed leapfrog levels each; the fastest wins.  Results are kept in a JSON
 // file ($EWH_TUNE_CACHE, else $HOME/.cache/ewh/tune.json) keyed by the GPU and
 // the problem's shape, so a shape is timed once per machine.  EWH_AUTOTUNE=0
@@ -398,7 +398,7 @@ std::string tune_key(const ewh_ctx* ctx) {
       restricted = restricted || (ctx->w32.rplan[k].ok && (long long)ctx->w32.rplan[k].bx * ctx->w32.rplan[k].by <
                                                               RS_BATCH_MIN_BLOCK);
   if (ctx->batch_member && (sizeof(T) == 4 ? ctx->w32.splan.ok : ctx->w64.splan.ok)) restricted = true;  // small2d_ok
-  return name + "|v5" + (restricted ? "b" : "") + (g.mapped ? "|map" : "") + (g.contrast ? "|c" : "") + "|d" + std::to_string(g.dim) +
+  return name + "|v6" + (restricted ? "b" : "") + (g.mapped ? "|map" : "") + (g.contrast ? "|c" : "") + "|d" + std::to_string(g.dim) +
          "|o" + std::to_string(ctx->order) + "|" +
          (sizeof(T) == 8 ? "f64" : "f32") + "|" + std::to_string(g.n[0]) + "x" + std::to_string(g.n[1]) + "x" +
          std::to_string(g.n[2]) + "|r" + std::to_string(g.nrhs);
@@ -480,7 +480,7 @@ bool ymarch_ok(const ewh_ctx* ctx, const Wave<T>& w) {
 
 template <typename T>
 void autotune(ewh_ctx* ctx, Wave<T>& w) {
-  const int nbase = ctx->g.mapped ? 1 : step_variant_count(ctx->g.dim, ctx->order);
+  const int nbase = ctx->g.mapped ? 1 : step_variant_count(ctx->g.dim, ctx->order, sizeof(T));
   const char* force = getenv("EWH_STEP2D_O4");
   // a launcher named by the environment (the y-march exists in FP32 only)
   const bool forced_launcher = force && (force[0] == 's' || force[0] == 'f' || (force[0] == 'y' && sizeof(T) == 4));

@@ -85,31 +85,6 @@ __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.lau
 // ---------------------------------------------------------------------------
 // Time update shared by all kernels.  a = M^{-1} K u (FP of the state).
 // ---------------------------------------------------------------------------
-template <typename T, int MODE, bool FORCED>
-__device__ __forceinline__ void leapfrog_update(const WaveFields<T>& f, long long p, T uval, T a,
-                                                const StepScalars& s) {
-  if (MODE == 3) {  // operator only
-    f.u_next[p] = a;
-    return;
-  }
-  if (FORCED) a += f.frho[p] * T(s.cosn);
-  if (MODE == STEP_FIRST) {
-    const T d = T(-0.5) * T(s.kt) * a;
-    const T un = uval + d;
-    f.delta[p] = d;
-    f.u_next[p] = un;
-    f.acc[p] = T(s.w0) * uval + T(s.wnew) * un;
-  } else {
-    const T d = f.delta[p] - T(s.kt) * a;
-    const T un = uval + d;
-    if (MODE == STEP_MID) {
-      f.delta[p] = d;
-      f.u_next[p] = un;
-    }
-    f.acc[p] += T(s.wnew) * un;
-  }
-}
-
 // The same update with delta^n, acc and f/rho already loaded (dprev, accprev
 // are not read at the first level; fr only when FORCED).
 template <typename T, int MODE, bool FORCED>
@@ -657,250 +632,6 @@ __global__ void __launch_bounds__(S3_THREADS, 4) sbp_div3d(Geom g, WaveFields<T>
 }
 
 // ---------------------------------------------------------------------------
-// Order 4 (SBP), 2D, split into two launches (stresses, then divergence and
-// update), one node per thread, 32 x 8 blocks.  Blocks whose nodes and stencil
-// reach lie inside the grid away from every SBP closure row stage their
-// operands (tile + 2-node halo) in shared memory with a few independent
-// coalesced loads per thread and difference them there; blocks near a side
-// run the generic per-node code from global memory.
-// ---------------------------------------------------------------------------
-constexpr int TL_H = 2;
-
-// every node of the block and its 2-node reach lies in rows/columns 4..N-5
-template <int TL_TX, int TL_TY>
-__device__ __forceinline__ bool tl_block_interior(const Geom& g, int x0, int y0) {
-  return x0 >= 4 && x0 + TL_TX - 1 <= g.n[0] - 5 && y0 >= 4 && y0 + TL_TY - 1 <= g.n[1] - 5;
-}
-
-template <typename T>
-__device__ __forceinline__ void stress2d_node(const Geom& g, const T* u, const T* lam, const T* mu, T* sig, int rhs,
-                                              int x, int y) {
-  const long long sy = g.np[0];
-  const T* U = u + pidx(g, rhs, 0, x, y, 0);
-  const T* V = U + g.field;
-  const T u_x = sbp_d1<T>(U, 1, x, g.n[0]);
-  const T u_y = sbp_d1<T>(U, sy, y, g.n[1]);
-  const T v_x = sbp_d1<T>(V, 1, x, g.n[0]);
-  const T v_y = sbp_d1<T>(V, sy, y, g.n[1]);
-  const long long pc = pidx(g, 0, 0, x, y, 0);
-  const T l = lam[pc], m = mu[pc];
-  const T div = u_x + v_y;
-  T* out = sig + (long long)rhs * 3 * g.field + pc;  // 12 sigma, as the interior tiles store it
-  out[0] = T(12) * (l * div + T(2) * m * u_x);
-  out[g.field] = T(12) * (l * div + T(2) * m * v_y);
-  out[2 * g.field] = T(12) * (m * (u_y + v_x));
-}
-
-template <typename T, int TL_TX, int TL_TY>
-__global__ void __launch_bounds__(TL_TX * TL_TY) sbp_stress2d_tl(Geom g, const T* __restrict__ u,
-                                                                 const T* __restrict__ lam, const T* __restrict__ mu,
-                                                                 T* __restrict__ sig) {
-  if (g.dim != 2) return;
-  constexpr int SX = TL_TX + 2 * TL_H, SY = TL_TY + 2 * TL_H;
-  __shared__ T su[2][SY][SX];
-  const int rhs = blockIdx.z;
-  const int x0 = blockIdx.x * TL_TX, y0 = blockIdx.y * TL_TY;
-  const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
-  if (!tl_block_interior<TL_TX, TL_TY>(g, x0, y0)) {  // uniform per block
-    pdl_wait();
-    pdl_trigger();
-    if (x < g.n[0] && y < g.n[1]) stress2d_node<T>(g, u, lam, mu, sig, rhs, x, y);
-    return;
-  }
-  const long long pc = pidx(g, 0, 0, x, y, 0);
-  const T l = lam[pc], m = mu[pc];               // static: read before the wait
-  pdl_wait();
-  pdl_trigger();
-  const T* U = u + pidx(g, rhs, 0, x0 - TL_H, y0 - TL_H, 0);
-  const int tid = threadIdx.y * TL_TX + threadIdx.x;
-  for (int i = tid; i < SX * SY; i += TL_TX * TL_TY) {
-    const int lx = i % SX, ly = i / SX;
-    const long long off = (long long)ly * g.np[0] + lx;
-    su[0][ly][lx] = U[off];
-    su[1][ly][lx] = U[off + g.field];
-  }
-  __syncthreads();
-  const int cx = threadIdx.x + TL_H, cy = threadIdx.y + TL_H;
-  // 12 D u and 12 sigma
-  const T u_x = c4u(su[0][cy][cx - 2], su[0][cy][cx - 1], su[0][cy][cx + 1], su[0][cy][cx + 2]);
-  const T v_x = c4u(su[1][cy][cx - 2], su[1][cy][cx - 1], su[1][cy][cx + 1], su[1][cy][cx + 2]);
-  const T u_y = c4u(su[0][cy - 2][cx], su[0][cy - 1][cx], su[0][cy + 1][cx], su[0][cy + 2][cx]);
-  const T v_y = c4u(su[1][cy - 2][cx], su[1][cy - 1][cx], su[1][cy + 1][cx], su[1][cy + 2][cx]);
-  const T div = u_x + v_y;
-  T* out = sig + (long long)rhs * 3 * g.field + pc;
-  out[0] = l * div + T(2) * m * u_x;
-  out[g.field] = l * div + T(2) * m * v_y;
-  out[2 * g.field] = m * (u_y + v_x);
-}
-
-template <typename T, int MODE, bool FORCED>
-__device__ __forceinline__ void div2d_node(const Geom& g, const WaveFields<T>& f, const StepScalars& s, int rhs, int x,
-                                           int y) {
-  if (!is_unknown(g, x, y, 0)) return;
-  const long long sy = g.np[0];
-  const long long pc = pidx(g, 0, 0, x, y, 0);
-  const T* sg = f.sigma + (long long)rhs * 3 * g.field + pc;
-  const T* sxx = sg;
-  const T* syy = sg + g.field;
-  const T* sxy = sg + 2 * g.field;
-  T ku = -sbp_d1<T>(sxx, 1, x, g.n[0]) - sbp_d1<T>(sxy, sy, y, g.n[1]);
-  T kv = -sbp_d1<T>(sxy, 1, x, g.n[0]) - sbp_d1<T>(syy, sy, y, g.n[1]);
-  const T inv_h0 = T(48.0 / 17.0);
-  if (x == 0) {
-    ku -= inv_h0 * sxx[0];
-    kv -= inv_h0 * sxy[0];
-  } else if (x == g.n[0] - 1) {
-    ku += inv_h0 * sxx[0];
-    kv += inv_h0 * sxy[0];
-  }
-  if (y == 0) {
-    ku -= inv_h0 * sxy[0];
-    kv -= inv_h0 * syy[0];
-  } else if (y == g.n[1] - 1) {
-    ku += inv_h0 * sxy[0];
-    kv += inv_h0 * syy[0];
-  }
-  const T irh = f.irh2[pc] * T(1.0 / 12.0);  // the scratch holds 12 sigma
-  const long long p0 = pidx(g, rhs, 0, x, y, 0);
-  leapfrog_update<T, MODE, FORCED>(f, p0, f.u_cur[p0], ku * irh, s);
-  leapfrog_update<T, MODE, FORCED>(f, p0 + g.field, f.u_cur[p0 + g.field], kv * irh, s);
-}
-
-template <typename T, int MODE, bool FORCED, int TL_TX, int TL_TY>
-__global__ void __launch_bounds__(TL_TX * TL_TY) sbp_div2d_tl(Geom g, WaveFields<T> f, StepScalars s) {
-  if (g.dim != 2) return;
-  constexpr int SX = TL_TX + 2 * TL_H, SY = TL_TY + 2 * TL_H;
-  __shared__ T sxx[TL_TY][SX];   // x-halo only
-  __shared__ T syy[SY][TL_TX];   // y-halo only
-  __shared__ T sxy[SY][SX];      // both
-  const int rhs = blockIdx.z;
-  const int x0 = blockIdx.x * TL_TX, y0 = blockIdx.y * TL_TY;
-  const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
-  if (!tl_block_interior<TL_TX, TL_TY>(g, x0, y0)) {
-    pdl_wait();
-    pdl_trigger();
-    div2d_node<T, MODE, FORCED>(g, f, s, rhs, x, y);
-    return;
-  }
-  const long long pc = pidx(g, 0, 0, x, y, 0);
-  const long long p0 = pidx(g, rhs, 0, x, y, 0);
-  const T irh = f.irh2[pc];                       // static: read before the wait
-  pdl_wait();
-  pdl_trigger();
-  const T* base = f.sigma + (long long)rhs * 3 * g.field;
-  const T* Gxx = base + pidx(g, 0, 0, x0 - TL_H, y0, 0);
-  const T* Gyy = base + g.field + pidx(g, 0, 0, x0, y0 - TL_H, 0);
-  const T* Gxy = base + 2 * g.field + pidx(g, 0, 0, x0 - TL_H, y0 - TL_H, 0);
-  const int tid = threadIdx.y * TL_TX + threadIdx.x;
-  for (int i = tid; i < SX * SY; i += TL_TX * TL_TY) {
-    const int lx = i % SX, ly = i / SX;
-    sxy[ly][lx] = Gxy[(long long)ly * g.np[0] + lx];
-    if (ly < TL_TY) sxx[ly][lx] = Gxx[(long long)ly * g.np[0] + lx];
-    if (lx < TL_TX) syy[ly][lx] = Gyy[(long long)ly * g.np[0] + lx];
-  }
-  const T u0 = f.u_cur[p0], u1 = f.u_cur[p0 + g.field];
-  __syncthreads();
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int cx = tx + TL_H, cy = ty + TL_H;
-  // 144 D sigma from 12 sigma
-  const T ku = -c4u(sxx[ty][cx - 2], sxx[ty][cx - 1], sxx[ty][cx + 1], sxx[ty][cx + 2]) -
-               c4u(sxy[cy - 2][cx], sxy[cy - 1][cx], sxy[cy + 1][cx], sxy[cy + 2][cx]);
-  const T kv = -c4u(sxy[cy][cx - 2], sxy[cy][cx - 1], sxy[cy][cx + 1], sxy[cy][cx + 2]) -
-               c4u(syy[cy - 2][tx], syy[cy - 1][tx], syy[cy + 1][tx], syy[cy + 2][tx]);
-  const T irs = irh * T(1.0 / 144.0);
-  leapfrog_update<T, MODE, FORCED>(f, p0, u0, ku * irs, s);
-  leapfrog_update<T, MODE, FORCED>(f, p0 + g.field, u1, kv * irs, s);
-}
-
-// ---------------------------------------------------------------------------
-// Order 4 (SBP), 2D, fused: one launch per time level.  A 32 x 16 tile (32 x 8
-// in FP64, to stay within 48 KB of static shared memory) stages
-// u on tile +- 6 nodes and lambda, mu on tile +- 3 in shared memory, forms the
-// stresses on tile +- 3 (the closure rows reach 3 nodes), then the divergence
-// and the leapfrog/filter update of its own nodes.
-// ---------------------------------------------------------------------------
-template <typename T>
-__host__ __device__ constexpr int o4_tile_y() { return sizeof(T) == 8 ? 8 : 16; }
-
-template <typename T, int MODE, bool FORCED>
-__global__ void __launch_bounds__(512) step2d_o4_fused(Geom g, WaveFields<T> f, StepScalars s) {
-  if (g.dim != 2) return;
-  pdl_wait();
-  pdl_trigger();
-  constexpr int TX = 32, TY = o4_tile_y<T>(), HU = 6, HS = 3;
-  constexpr int UX = TX + 2 * HU, UY = TY + 2 * HU;
-  constexpr int SX = TX + 2 * HS, SY = TY + 2 * HS;
-  __shared__ T su[2][UY][UX];
-  __shared__ T sl[SY][SX];
-  __shared__ T sm[SY][SX];
-  __shared__ T ss[3][SY][SX];  // xx, yy, xy
-  const int rhs = blockIdx.z;
-  const int x0 = blockIdx.x * TX, y0 = blockIdx.y * TY;
-  const int tid = threadIdx.y * TX + threadIdx.x;
-  const int nx = g.n[0], ny = g.n[1];
-  for (int i = tid; i < UX * UY; i += TX * TY) {
-    const int lx = i % UX, ly = i / UX;
-    const long long pu = pidx(g, rhs, 0, x0 - HU + lx, y0 - HU + ly, 0);
-    su[0][ly][lx] = f.u_cur[pu];
-    su[1][ly][lx] = f.u_cur[pu + g.field];
-  }
-  for (int i = tid; i < SX * SY; i += TX * TY) {
-    const int lx = i % SX, ly = i / SX;
-    const long long pc = pidx(g, 0, 0, x0 - HS + lx, y0 - HS + ly, 0);
-    sl[ly][lx] = f.lam[pc];
-    sm[ly][lx] = f.mu[pc];
-  }
-  __syncthreads();
-  // stresses on the tile +- HS (nodes of the full grid only)
-  for (int i = tid; i < SX * SY; i += TX * TY) {
-    const int lx = i % SX, ly = i / SX;
-    const int qx = x0 - HS + lx, qy = y0 - HS + ly;
-    T sxx = T(0), syy = T(0), sxy = T(0);
-    if (qx >= 0 && qx < nx && qy >= 0 && qy < ny) {
-      const int ux = lx + (HU - HS), uy = ly + (HU - HS);
-      const T u_x = sbp_d1<T>(&su[0][uy][ux], 1, qx, nx);
-      const T u_y = sbp_d1<T>(&su[0][uy][ux], UX, qy, ny);
-      const T v_x = sbp_d1<T>(&su[1][uy][ux], 1, qx, nx);
-      const T v_y = sbp_d1<T>(&su[1][uy][ux], UX, qy, ny);
-      const T l = sl[ly][lx], m = sm[ly][lx];
-      const T div = u_x + v_y;
-      sxx = l * div + T(2) * m * u_x;
-      syy = l * div + T(2) * m * v_y;
-      sxy = m * (u_y + v_x);
-    }
-    ss[0][ly][lx] = sxx;
-    ss[1][ly][lx] = syy;
-    ss[2][ly][lx] = sxy;
-  }
-  __syncthreads();
-  const int x = x0 + threadIdx.x, y = y0 + threadIdx.y;
-  if (!is_unknown(g, x, y, 0)) return;
-  const int lx = threadIdx.x + HS, ly = threadIdx.y + HS;
-  const T inv_h0 = T(48.0 / 17.0);
-  // K u_x = -D_x sxx - D_y sxy (+ boundary terms on free sides)
-  T ku = -sbp_d1<T>(&ss[0][ly][lx], 1, x, nx) - sbp_d1<T>(&ss[2][ly][lx], SX, y, ny);
-  T kv = -sbp_d1<T>(&ss[2][ly][lx], 1, x, nx) - sbp_d1<T>(&ss[1][ly][lx], SX, y, ny);
-  if (x == 0) {
-    ku -= inv_h0 * ss[0][ly][lx];
-    kv -= inv_h0 * ss[2][ly][lx];
-  } else if (x == nx - 1) {
-    ku += inv_h0 * ss[0][ly][lx];
-    kv += inv_h0 * ss[2][ly][lx];
-  }
-  if (y == 0) {
-    ku -= inv_h0 * ss[2][ly][lx];
-    kv -= inv_h0 * ss[1][ly][lx];
-  } else if (y == ny - 1) {
-    ku += inv_h0 * ss[2][ly][lx];
-    kv += inv_h0 * ss[1][ly][lx];
-  }
-  const T irh = f.irh2[pidx(g, 0, 0, x, y, 0)];
-  const long long p0 = pidx(g, rhs, 0, x, y, 0);
-  leapfrog_update<T, MODE, FORCED>(f, p0, su[0][threadIdx.y + HU][threadIdx.x + HU], ku * irh, s);
-  leapfrog_update<T, MODE, FORCED>(f, p0 + g.field, su[1][threadIdx.y + HU][threadIdx.x + HU], kv * irh, s);
-}
-
-// ---------------------------------------------------------------------------
 // Launchers
 // ---------------------------------------------------------------------------
 // Launch with programmatic stream serialization (see pdl_wait); EWH_PDL=0
@@ -926,56 +657,35 @@ static cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, cud
 }
 
 // 2D order-4 kernel variants (Geom::variant, chosen per context by the
-// autotuner): 0..3 = stress + divergence launches with 32x8, 32x16, 64x8 or
-// 64x4 blocks (FP64: 0 = 32x8, FX_VARIANT + shape = the block-fixed-point step,
-// ewh_fx2d.cu), 4 = single fused launch, YM_VARIANT = the FP32 y-march
-// (ewh_ymarch.cu).  EWH_STEP2D_O4=fused|split|ym|fx overrides it (read whenever
+// autotuner): 0 = stress + divergence pair, FX_VARIANT + shape = the FP64
+// block-fixed-point step (ewh_fx2d.cu), YM_VARIANT = the FP32 y-march
+// (ewh_ymarch.cu).  EWH_STEP2D_O4=split|ym|fx overrides it (read whenever
 // launches are enqueued; a context captures its step graph once, on first use).
-static int step2d_o4_variant(const Geom& g) {
-  const char* e = getenv("EWH_STEP2D_O4");
-  if (e && e[0] == 'f' && e[1] != 'x') return 1;
-  if (e && e[0] == 's') return 0;
-  return g.variant == 4 ? 1 : 0;
-}
-static int step2d_o4_tile(const Geom& g) {
-  const char* e = getenv("EWH_STEP2D_O4");
-  if (e && e[0] == 's') return 0;
-  return (g.variant >= 0 && g.variant <= 3) ? g.variant : 0;
-}
-
 // ---------------------------------------------------------------------------
-// Order 4 (SBP), 2D, curvilinear grid (Section 4.1, curvilinear form): the
-// node grid is the image of (q, r) = (i h, j h) under a smooth mapping.  The
-// stress kernel forms physical derivatives from the SBP derivatives in q and
-// r, u_x = (y_r u_q - y_q u_r) / J, u_y = (x_q u_r - x_r u_q) / J, the
-// stresses (the 1/J rides on lambda / J and mu / J, which the context stores
-// in place of lambda and mu), and the four J-weighted fluxes
-//   F^q_u = y_r s_xx - x_r s_xy,  F^r_u = -y_q s_xx + x_q s_xy,
-//   F^q_v = y_r s_xy - x_r s_yy,  F^r_v = -y_q s_xy + x_q s_yy;
-// the divergence kernel forms -D_q F^q - D_r F^r + H^{-1} B F (the Cartesian
-// kernel with the fluxes in place of the stresses) times 1/(rho J h^2).
-// The metric planes are (y_r, -x_r, -y_q, x_q).
+// Order 4 (SBP), 2D, in two launches: stresses, then divergence and update.  A
+// thread takes 16 bytes' worth of nodes along x (four in FP32, two in FP64) of the
+// rectangle where every difference is central and every node an unknown, with
+// 16-byte loads (14 for the differences of four FP32 nodes instead of 64).
+// Rectangle and frame (the nodes within some four of a side, one per thread, their
+// closure rows as taps from a table) are numbered apart, so no warp runs both forms;
+// the frame's blocks come first.  What no level writes is read before the wait for the
+// previous kernel, and all loads precede the first store.  The operator is carried as
+// 12 D (stresses 12 sigma, divergence 144 D sigma).
 //
-// The pair: a thread takes 16 bytes' worth of nodes along x (four in FP32, two
-// in FP64) of the rectangle where every difference is central and every node an
-// unknown, with 16-byte loads (14 for the differences of four FP32 nodes instead of
-// 64).  Rectangle and frame (the nodes within some four of a side, general form, one
-// per thread) are numbered apart, so no warp runs both forms; the frame's blocks
-// come first, since its threads take longest.  What no level writes is read before the
-// wait for the previous kernel.
-//
-// Per level, stress and divergence: 1026 x 1026 nodes 21.9 -> 14.6 us in FP32 (122 MB,
-// mostly out of L2), 144 -> 131 us in FP64 (its pipe); 66 x 66 7.2 -> 3.6 us and 11.3 -> 7.1
-// us.  A fused form (u, metrics and fluxes of a tile in shared memory) took 6.9 us at
-// 66^2 and 38 us at 1026^2 in FP32.
+// Per level, against one node a thread in shared-memory tiles with six-tap closures: FP32
+// 66^2 6.4 -> 3.6 us, 258^2 6.6 -> 3.9, 514^2 9.5 -> 6.1, 1026^2 22.6 -> 12.6, 2002^2
+// 94 -> 59 us; FP64 66^2 10.1 -> 5.5, 1026^2 106 -> 90 us.  Small grids are bound by the two
+// launches, FP32 by L2 and HBM (88 bytes a node and level; 2002^2: 0.88 of the copy
+// rate), FP64 by its pipe.  One launch over tiles with recomputed stresses was slower
+// at every size.
 // ---------------------------------------------------------------------------
-struct CurvPart {
+struct Part2d {
   int xa, ngx, nr;  // first column of the rectangle, its groups per row, its rows (from row 4)
   int nfc;          // frame columns in the rectangle's rows
   int nbf;          // blocks of frame nodes, in front
   int frame;        // frame nodes
 };
-constexpr int CURV_THREADS = 64;
+constexpr int P2_THREADS = 64;
 
 template <typename T>
 struct Vec16;
@@ -999,29 +709,29 @@ __device__ __forceinline__ void st16(T* p, const T* v) {
   *reinterpret_cast<typename Vec16<T>::type*>(p) = *reinterpret_cast<const typename Vec16<T>::type*>(v);
 }
 
-// Central differences of a group at v: along x from the 16 bytes before, at and
+// 12 D (central) of a group at v: along x from the 16 bytes before, at and
 // after it, along y from the rows at -2, -1, 1 and 2.
 template <typename T>
-__device__ __forceinline__ void curv_dx(const T* v, T* d) {
+__device__ __forceinline__ void dx16(const T* v, T* d) {
   constexpr int V = 16 / sizeof(T);
   alignas(16) T w[3][V];
   ld16<T, 3>(v - V, w);
   const T* const c = &w[0][0] + V;
 #pragma unroll
-  for (int k = 0; k < V; ++k) d[k] = c4(c[k - 2], c[k - 1], c[k + 1], c[k + 2]);
+  for (int k = 0; k < V; ++k) d[k] = c4u(c[k - 2], c[k - 1], c[k + 1], c[k + 2]);
 }
 template <typename T>
-__device__ __forceinline__ void curv_dy(const T* v, int sy, T* d) {
+__device__ __forceinline__ void dy16(const T* v, int sy, T* d) {
   constexpr int V = 16 / sizeof(T);
   alignas(16) T lo[2][V], hi[2][V];
   ld16<T, 2>(v - 2 * sy, lo, sy);
   ld16<T, 2>(v + sy, hi, sy);
 #pragma unroll
-  for (int k = 0; k < V; ++k) d[k] = c4(lo[0][k], lo[1][k], hi[0][k], hi[1][k]);
+  for (int k = 0; k < V; ++k) d[k] = c4u(lo[0][k], lo[1][k], hi[0][k], hi[1][k]);
 }
 
 // Position of a thread: frame node (true) or first node of a group; x < 0: none.
-__device__ __forceinline__ bool curv_pos(const Geom& g, const CurvPart& c, int V, int& x, int& y) {
+__device__ __forceinline__ bool part2d_pos(const Geom& g, const Part2d& c, int V, int& x, int& y) {
   x = -1;
   if ((int)blockIdx.x < c.nbf) {
     int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1047,6 +757,169 @@ __device__ __forceinline__ bool curv_pos(const Geom& g, const CurvPart& c, int V
   return false;
 }
 
+// The closure taps into shared memory (frame blocks; blockDim.x >= 32)
+template <typename T>
+__device__ __forceinline__ void load_taps(const S3Taps<T>& tp, S3Taps<T>& st) {
+  for (int i = threadIdx.x; i < 36; i += blockDim.x) st.off[i] = tp.off[i], st.w[i] = tp.w[i];
+  __syncthreads();
+}
+
+template <typename T>
+__global__ void __launch_bounds__(P2_THREADS) sbp_stress2d(Geom g, Part2d cp, const T* __restrict__ u,
+                                                           const T* __restrict__ lam, const T* __restrict__ mu,
+                                                           T* __restrict__ sig, const __grid_constant__ S3Taps<T> tp) {
+  if (g.dim != 2) return;
+  constexpr int V = 16 / sizeof(T);
+  int x, y;
+  const bool frame = part2d_pos(g, cp, V, x, y);
+  const int rhs = blockIdx.y;
+  const long long pc = x < 0 ? 0 : pidx(g, 0, 0, x, y, 0);
+  const T* const U = u + (long long)rhs * 2 * g.field + pc;
+  T* const out = sig + (long long)rhs * 3 * g.field + pc;
+  const int sy = g.np[0];
+  if (frame) {
+    __shared__ S3Taps<T> taps;
+    load_taps(tp, taps);
+    const T l = lam[pc], m = mu[pc];
+    pdl_wait();
+    pdl_trigger();
+    if (x < 0) return;
+    const T* const W = U + g.field;
+    const int cx = s3_class(x, g.n[0]), cy = s3_class(y, g.n[1]);
+    const T u_x = s3_taps12(U, 1, cx, taps), u_y = s3_taps12(U, sy, cy, taps);
+    const T v_x = s3_taps12(W, 1, cx, taps), v_y = s3_taps12(W, sy, cy, taps);
+    const T ld = l * (u_x + v_y);
+    out[0] = ld + T(2) * m * u_x;
+    out[g.field] = ld + T(2) * m * v_y;
+    out[2 * g.field] = m * (u_y + v_x);
+    return;
+  }
+  alignas(16) T l[1][V], m[1][V];
+  if (x >= 0) ld16<T, 1>(lam + pc, l), ld16<T, 1>(mu + pc, m);
+  pdl_wait();
+  pdl_trigger();
+  if (x < 0) return;
+  T u_x[V], u_y[V], v_x[V], v_y[V];
+  dx16(U, u_x);
+  dx16(U + g.field, v_x);
+  dy16(U, sy, u_y);
+  dy16(U + g.field, sy, v_y);
+  alignas(16) T o[3][V];
+#pragma unroll
+  for (int k = 0; k < V; ++k) {
+    const T ld = l[0][k] * (u_x[k] + v_y[k]);
+    o[0][k] = ld + T(2) * m[0][k] * u_x[k];
+    o[1][k] = ld + T(2) * m[0][k] * v_y[k];
+    o[2][k] = m[0][k] * (u_y[k] + v_x[k]);
+  }
+#pragma unroll
+  for (int k = 0; k < 3; ++k) st16(out + k * g.field, o[k]);
+}
+
+// Divergence and update of both kinds of grid: component c from the fields at qc (along
+// x) and rc (along y), in units of 1 / scale.
+template <typename T, int MODE, bool FORCED>
+__device__ __forceinline__ void div2d_part(const Geom& g, const Part2d& cp, const WaveFields<T>& f, const StepScalars& s,
+                                           const S3Taps<T>& tp, int nf, int qu, int ru, int qv, int rv, T scale, T bscale) {
+  constexpr int V = 16 / sizeof(T);
+  constexpr bool RD = MODE == STEP_MID || MODE == STEP_LAST;
+  int x, y;
+  const bool frame = part2d_pos(g, cp, V, x, y);
+  const int rhs = blockIdx.y;
+  const long long pc = x < 0 ? 0 : pidx(g, 0, 0, x, y, 0);
+  const long long p0 = (long long)rhs * 2 * g.field + pc;
+  const T* const sg = f.sigma + (long long)rhs * nf * g.field + pc;
+  const T *const fqu = sg + qu * g.field, *const fru = sg + ru * g.field;
+  const T *const fqv = sg + qv * g.field, *const frv = sg + rv * g.field;
+  const int sy = g.np[0];
+  if (frame) {
+    __shared__ S3Taps<T> taps;
+    load_taps(tp, taps);
+    const bool unk = x >= 0 && is_unknown(g, x, y, 0);
+    const T irh = f.irh2[pc] * scale;
+    const T fr0 = FORCED ? f.frho[p0] : T(0), fr1 = FORCED ? f.frho[p0 + g.field] : T(0);
+    pdl_wait();
+    pdl_trigger();
+    if (!unk) return;
+    const T u0 = f.u_cur[p0], u1 = f.u_cur[p0 + g.field];
+    const T d0 = RD ? f.delta[p0] : T(0), d1 = RD ? f.delta[p0 + g.field] : T(0);
+    const T a0 = RD ? f.acc[p0] : T(0), a1 = RD ? f.acc[p0 + g.field] : T(0);
+    const int cx = s3_class(x, g.n[0]), cy = s3_class(y, g.n[1]);
+    const T ih = bscale * T(48.0 / 17.0);
+    const T bx = x == 0 ? -ih : (x == g.n[0] - 1 ? ih : T(0)), by = y == 0 ? -ih : (y == g.n[1] - 1 ? ih : T(0));
+    const T ku = bx * fqu[0] + by * fru[0] - (s3_taps12(fqu, 1, cx, taps) + s3_taps12(fru, sy, cy, taps));
+    const T kv = bx * fqv[0] + by * frv[0] - (s3_taps12(fqv, 1, cx, taps) + s3_taps12(frv, sy, cy, taps));
+    leapfrog_update_pre<T, MODE, FORCED>(f, p0, u0, ku * irh, s, d0, a0, fr0);
+    leapfrog_update_pre<T, MODE, FORCED>(f, p0 + g.field, u1, kv * irh, s, d1, a1, fr1);
+    return;
+  }
+  alignas(16) T irh[1][V], fr[2][V];
+  if (x >= 0) {
+    ld16<T, 1>(f.irh2 + pc, irh);
+    if (FORCED) ld16<T, 1>(f.frho + p0, fr), ld16<T, 1>(f.frho + p0 + g.field, fr + 1);
+  }
+  pdl_wait();
+  pdl_trigger();
+  if (x < 0) return;
+  alignas(16) T uv[2][V], dl[2][V], ac[2][V], dq[2][V], dr[2][V];
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {  // all loads before the first store
+    const long long p = p0 + c * g.field;
+    ld16<T, 1>(f.u_cur + p, uv + c);
+    if (RD) ld16<T, 1>(f.delta + p, dl + c), ld16<T, 1>(f.acc + p, ac + c);
+    dx16(c ? fqv : fqu, dq[c]);
+    dy16(c ? frv : fru, sy, dr[c]);
+  }
+#pragma unroll
+  for (int c = 0; c < 2; ++c) {
+    const long long p = p0 + c * g.field;
+    alignas(16) T un[V];
+#pragma unroll
+    for (int k = 0; k < V; ++k) {
+      T a = (-dq[c][k] - dr[c][k]) * (irh[0][k] * scale);
+      if (MODE == 3) {  // operator only
+        un[k] = a;
+        continue;
+      }
+      if (FORCED) a += fr[c][k] * T(s.cosn);
+      const T d = MODE == STEP_FIRST ? T(-0.5) * T(s.kt) * a : dl[c][k] - T(s.kt) * a;
+      un[k] = uv[c][k] + d;
+      ac[c][k] = MODE == STEP_FIRST ? T(s.w0) * uv[c][k] + T(s.wnew) * un[k] : ac[c][k] + T(s.wnew) * un[k];
+      dl[c][k] = d;
+    }
+    if (MODE != STEP_LAST) st16(f.u_next + p, un);
+    if (MODE == STEP_FIRST || MODE == STEP_MID) st16(f.delta + p, dl[c]);
+    if (MODE != 3) st16(f.acc + p, ac[c]);
+  }
+}
+
+// stresses xx, yy, xy (12 sigma)
+template <typename T, int MODE, bool FORCED>
+__global__ void __launch_bounds__(P2_THREADS) sbp_div2d(Geom g, Part2d cp, WaveFields<T> f, StepScalars s,
+                                                        const __grid_constant__ S3Taps<T> tp) {
+  if (g.dim != 2) return;
+  div2d_part<T, MODE, FORCED>(g, cp, f, s, tp, 3, 0, 2, 2, 1, T(1.0 / 144.0), T(12));
+}
+
+// ---------------------------------------------------------------------------
+// Order 4 (SBP), 2D, curvilinear grid (Section 4.1, curvilinear form): the
+// node grid is the image of (q, r) = (i h, j h) under a smooth mapping.  The
+// stress kernel forms physical derivatives from the SBP derivatives in q and
+// r, u_x = (y_r u_q - y_q u_r) / J, u_y = (x_q u_r - x_r u_q) / J, the
+// stresses (the 1/J rides on lambda / J and mu / J, which the context stores
+// in place of lambda and mu), and the four J-weighted fluxes
+//   F^q_u = y_r s_xx - x_r s_xy,  F^r_u = -y_q s_xx + x_q s_xy,
+//   F^q_v = y_r s_xy - x_r s_yy,  F^r_v = -y_q s_xy + x_q s_yy;
+// the divergence kernel forms -D_q F^q - D_r F^r + H^{-1} B F (the Cartesian
+// kernel with the fluxes in place of the stresses) times 1/(rho J h^2).
+// The metric planes are (y_r, -x_r, -y_q, x_q).
+//
+// In two kernels (see the 2D pair above), the differences divided by 12 at once.
+// Per level, stress and divergence: 1026 x 1026 nodes 21.9 -> 14.6 us in FP32 (122 MB,
+// mostly out of L2), 144 -> 131 us in FP64 (its pipe); 66 x 66 7.2 -> 3.6 us and 11.3 -> 7.1
+// us.  A fused form (u, metrics and fluxes of a tile in shared memory) took 6.9 us at
+// 66^2 and 38 us at 1026^2 in FP32.
+// ---------------------------------------------------------------------------
 template <typename T>
 __device__ __forceinline__ void curv_flux(T uq, T ur, T vq, T vr, T a0, T a1, T a2, T a3, T l, T m, T* o0, T* o1, T* o2,
                                           T* o3) {
@@ -1060,29 +933,22 @@ __device__ __forceinline__ void curv_flux(T uq, T ur, T vq, T vr, T a0, T a1, T 
   *o3 = a2 * sxy + a3 * syy;
 }
 
-// The closure taps into shared memory (frame blocks; blockDim.x >= 32)
 template <typename T>
-__device__ __forceinline__ void curv_taps(const S3Taps<T>& tp, S3Taps<T>& st) {
-  for (int i = threadIdx.x; i < 36; i += blockDim.x) st.off[i] = tp.off[i], st.w[i] = tp.w[i];
-  __syncthreads();
-}
-
-template <typename T>
-__global__ void __launch_bounds__(CURV_THREADS) curv_stress2d(Geom g, CurvPart cp, const T* __restrict__ u,
+__global__ void __launch_bounds__(P2_THREADS) curv_stress2d(Geom g, Part2d cp, const T* __restrict__ u,
                                                               const T* __restrict__ lam, const T* __restrict__ mu,
                                                               const T* __restrict__ met, T* __restrict__ sig,
                                                               const __grid_constant__ S3Taps<T> tp) {
   if (g.dim != 2) return;
   constexpr int V = 16 / sizeof(T);
   int x, y;
-  const bool frame = curv_pos(g, cp, V, x, y);
+  const bool frame = part2d_pos(g, cp, V, x, y);
   const int rhs = blockIdx.y;
   const long long pc = x < 0 ? 0 : pidx(g, 0, 0, x, y, 0);  // lam, mu: lambda / J, mu / J
   const T* const U = u + (long long)rhs * 2 * g.field + pc;
   T* const out = sig + (long long)rhs * 4 * g.field + pc;
   if (frame) {
     __shared__ S3Taps<T> taps;
-    curv_taps(tp, taps);
+    load_taps(tp, taps);
     const T l = lam[pc], m = mu[pc], a0 = met[pc], a1 = met[g.field + pc], a2 = met[2 * g.field + pc];
     const T a3 = met[3 * g.field + pc];
     pdl_wait();
@@ -1108,94 +974,26 @@ __global__ void __launch_bounds__(CURV_THREADS) curv_stress2d(Geom g, CurvPart c
   if (x < 0) return;
   const int sy = g.np[0];
   T uq[V], ur[V], vq[V], vr[V];
-  curv_dx(U, uq);
-  curv_dx(U + g.field, vq);
-  curv_dy(U, sy, ur);
-  curv_dy(U + g.field, sy, vr);
+  dx16(U, uq);
+  dx16(U + g.field, vq);
+  dy16(U, sy, ur);
+  dy16(U + g.field, sy, vr);
   alignas(16) T o[4][V];
+  const T w = T(1.0 / 12.0);
 #pragma unroll
   for (int k = 0; k < V; ++k)
-    curv_flux(uq[k], ur[k], vq[k], vr[k], a[0][k], a[1][k], a[2][k], a[3][k], l[0][k], m[0][k], &o[0][k], &o[1][k],
+    curv_flux(w * uq[k], w * ur[k], w * vq[k], w * vr[k], a[0][k], a[1][k], a[2][k], a[3][k], l[0][k], m[0][k], &o[0][k], &o[1][k],
               &o[2][k], &o[3][k]);
 #pragma unroll
   for (int k = 0; k < 4; ++k) st16(out + k * g.field, o[k]);
 }
 
+// fluxes F^q_u, F^r_u, F^q_v, F^r_v; irh2 = 1 / (rho J h^2)
 template <typename T, int MODE, bool FORCED>
-__global__ void __launch_bounds__(CURV_THREADS) curv_div2d(Geom g, CurvPart cp, WaveFields<T> f, StepScalars s,
-                                                           const __grid_constant__ S3Taps<T> tp) {
+__global__ void __launch_bounds__(P2_THREADS) curv_div2d(Geom g, Part2d cp, WaveFields<T> f, StepScalars s,
+                                                         const __grid_constant__ S3Taps<T> tp) {
   if (g.dim != 2) return;
-  constexpr int V = 16 / sizeof(T);
-  int x, y;
-  const bool frame = curv_pos(g, cp, V, x, y);
-  const int rhs = blockIdx.y;
-  const long long pc = x < 0 ? 0 : pidx(g, 0, 0, x, y, 0);
-  const long long p0 = (long long)rhs * 2 * g.field + pc;
-  const T* const fqu = f.sigma + (long long)rhs * 4 * g.field + pc;
-  const T* const fru = fqu + g.field;
-  const T* const fqv = fqu + 2 * g.field;
-  const T* const frv = fqu + 3 * g.field;
-  if (frame) {
-    __shared__ S3Taps<T> taps;
-    curv_taps(tp, taps);
-    const bool unk = x >= 0 && is_unknown(g, x, y, 0);
-    const T irh = f.irh2[pc];  // 1 / (rho J h^2)
-    const T fr0 = FORCED ? f.frho[p0] : T(0), fr1 = FORCED ? f.frho[p0 + g.field] : T(0);
-    pdl_wait();
-    pdl_trigger();
-    if (!unk) return;
-    constexpr bool RD = MODE == STEP_MID || MODE == STEP_LAST;
-    const T u0 = f.u_cur[p0], u1 = f.u_cur[p0 + g.field];
-    const T d0 = RD ? f.delta[p0] : T(0), d1 = RD ? f.delta[p0 + g.field] : T(0);
-    const T a0 = RD ? f.acc[p0] : T(0), a1 = RD ? f.acc[p0 + g.field] : T(0);
-    const int sy = g.np[0], cx = s3_class(x, g.n[0]), cy = s3_class(y, g.n[1]);
-    const T w = T(-1.0 / 12.0), ih = T(48.0 / 17.0);
-    const T bx = x == 0 ? -ih : (x == g.n[0] - 1 ? ih : T(0)), by = y == 0 ? -ih : (y == g.n[1] - 1 ? ih : T(0));
-    const T ku = w * (s3_taps12(fqu, 1, cx, taps) + s3_taps12(fru, sy, cy, taps)) + bx * fqu[0] + by * fru[0];
-    const T kv = w * (s3_taps12(fqv, 1, cx, taps) + s3_taps12(frv, sy, cy, taps)) + bx * fqv[0] + by * frv[0];
-    leapfrog_update_pre<T, MODE, FORCED>(f, p0, u0, ku * irh, s, d0, a0, fr0);
-    leapfrog_update_pre<T, MODE, FORCED>(f, p0 + g.field, u1, kv * irh, s, d1, a1, fr1);
-    return;
-  }
-  alignas(16) T irh[1][V], fr[2][V];
-  if (x >= 0) {
-    ld16<T, 1>(f.irh2 + pc, irh);
-    if (FORCED) ld16<T, 1>(f.frho + p0, fr), ld16<T, 1>(f.frho + p0 + g.field, fr + 1);
-  }
-  pdl_wait();
-  pdl_trigger();
-  if (x < 0) return;
-  const int sy = g.np[0];
-  alignas(16) T uv[2][V], dl[2][V], ac[2][V], dq[2][V], dr[2][V];
-#pragma unroll
-  for (int c = 0; c < 2; ++c) {  // all loads before the first store
-    const long long p = p0 + c * g.field;
-    ld16<T, 1>(f.u_cur + p, uv + c);
-    if (MODE == STEP_MID || MODE == STEP_LAST) ld16<T, 1>(f.delta + p, dl + c), ld16<T, 1>(f.acc + p, ac + c);
-    curv_dx(c ? fqv : fqu, dq[c]);
-    curv_dy(c ? frv : fru, sy, dr[c]);
-  }
-#pragma unroll
-  for (int c = 0; c < 2; ++c) {
-    const long long p = p0 + c * g.field;
-    alignas(16) T un[V];
-#pragma unroll
-    for (int k = 0; k < V; ++k) {
-      T a = (-dq[c][k] - dr[c][k]) * irh[0][k];
-      if (MODE == 3) {  // operator only
-        un[k] = a;
-        continue;
-      }
-      if (FORCED) a += fr[c][k] * T(s.cosn);
-      const T d = MODE == STEP_FIRST ? T(-0.5) * T(s.kt) * a : dl[c][k] - T(s.kt) * a;
-      un[k] = uv[c][k] + d;
-      ac[c][k] = MODE == STEP_FIRST ? T(s.w0) * uv[c][k] + T(s.wnew) * un[k] : ac[c][k] + T(s.wnew) * un[k];
-      dl[c][k] = d;
-    }
-    if (MODE != STEP_LAST) st16(f.u_next + p, un);
-    if (MODE == STEP_FIRST || MODE == STEP_MID) st16(f.delta + p, dl[c]);
-    if (MODE != 3) st16(f.acc + p, ac[c]);
-  }
+  div2d_part<T, MODE, FORCED>(g, cp, f, s, tp, 4, 0, 1, 2, 3, T(1.0 / 12.0), T(12));
 }
 
 // Metric terms of a mapped grid (FP64, dense C-order planes, x fastest):
@@ -1246,13 +1044,23 @@ static const S3Taps<T>& s3_taps() {
   return t;
 }
 
-template <typename T, int MODE, bool FORCED, int TX, int TY>
-static cudaError_t launch_split_o4(const Geom& g, const WaveFields<T>& f, const StepScalars& s, cudaStream_t st) {
-  dim3 tgrd((g.n[0] + TX - 1) / TX, (g.n[1] + TY - 1) / TY, g.nrhs);
-  cudaError_t e = launch_k(sbp_stress2d_tl<T, TX, TY>, tgrd, dim3(TX, TY), st, g, (const T*)f.u_cur, f.lam, f.mu,
-                           f.sigma);
-  if (e != cudaSuccess) return e;
-  return launch_k(sbp_div2d_tl<T, MODE, FORCED, TX, TY>, tgrd, dim3(TX, TY), st, g, f, s);
+// Rectangle and frame of the 2D pair, and its launch shape.
+template <typename T>
+static Part2d part2d(const Geom& g, dim3* grd, dim3* blk) {
+  constexpr int V = 16 / sizeof(T);
+  Part2d cp;
+  cp.xa = 4 + (V - (4 + g.padx) % V) % V;
+  cp.nr = g.n[1] - 8;
+  cp.ngx = cp.nr > 0 ? std::max(0, (g.n[0] - 4 - cp.xa) / V) : 0;
+  cp.nfc = g.n[0] - V * cp.ngx;
+  cp.frame = 8 * g.n[0] + cp.nfc * cp.nr;
+  // blocks of 64 threads (mapped, 1026^2 FP32: 14.6 us a level, with 256 14.9, with 32 19.0), of
+  // one warp where those would leave SMs short (202^2 FP64: 8.9 us, with 64 12.0)
+  const int nt = (long long)(cp.frame + cp.ngx * cp.nr) * g.nrhs < 4LL * 152 * P2_THREADS ? 32 : P2_THREADS;
+  cp.nbf = (cp.frame + nt - 1) / nt;
+  *blk = dim3(nt);
+  *grd = dim3(cp.nbf + (cp.ngx * cp.nr + nt - 1) / nt, g.nrhs);
+  return cp;
 }
 
 template <typename T, int MODE, bool FORCED>
@@ -1278,18 +1086,8 @@ static cudaError_t launch_mode(const Geom& g, int order, const WaveFields<T>& f,
     return cudaGetLastError();
   }
   if (g.mapped) {  // curvilinear 2D order 4: stress + divergence
-    constexpr int V = 16 / sizeof(T);
-    CurvPart cp;
-    cp.xa = 4 + (V - (4 + g.padx) % V) % V;
-    cp.nr = g.n[1] - 8;
-    cp.ngx = cp.nr > 0 ? std::max(0, (g.n[0] - 4 - cp.xa) / V) : 0;
-    cp.nfc = g.n[0] - V * cp.ngx;
-    cp.frame = 8 * g.n[0] + cp.nfc * cp.nr;
-    // blocks of 64 threads (1026^2 FP32: 14.6 us a level, with 256 14.9, with 32 19.0), of one
-    // warp where those would leave SMs short (202^2 FP64: 8.9 us, with 64 12.0)
-    const int nt = (long long)(cp.frame + cp.ngx * cp.nr) * g.nrhs < 4LL * 152 * CURV_THREADS ? 32 : CURV_THREADS;
-    cp.nbf = (cp.frame + nt - 1) / nt;
-    dim3 blk(nt), grd(cp.nbf + (cp.ngx * cp.nr + nt - 1) / nt, g.nrhs);
+    dim3 grd, blk;
+    const Part2d cp = part2d<T>(g, &grd, &blk);
     cudaError_t e = launch_k(curv_stress2d<T>, grd, blk, st, g, cp, (const T*)f.u_cur, f.lam, f.mu, f.met, f.sigma,
                              s3_taps<T>());
     if (e != cudaSuccess) return e;
@@ -1321,25 +1119,12 @@ static cudaError_t launch_mode(const Geom& g, int order, const WaveFields<T>& f,
       return cudaGetLastError();
     }
   }
-  if (g.dim == 2 && step2d_o4_variant(g) == 1) {
-    constexpr int TY = o4_tile_y<T>();
-    dim3 blk(32, TY), grd((g.n[0] + 31) / 32, (g.n[1] + TY - 1) / TY, g.nrhs);
-    cudaError_t e = launch_k(step2d_o4_fused<T, MODE, FORCED>, grd, blk, st, g, f, s);
-    if (e != cudaSuccess) return e;
-    if (nl) *nl += 1;
-    return cudaGetLastError();
-  }
   if (g.dim == 2) {
-    cudaError_t e;
-    if constexpr (sizeof(T) == 8) {
-      e = launch_split_o4<T, MODE, FORCED, 32, 8>(g, f, s, st);
-    } else {
-      const int tv = step2d_o4_tile(g);
-      e = tv == 1   ? launch_split_o4<T, MODE, FORCED, 32, 16>(g, f, s, st)
-          : tv == 2 ? launch_split_o4<T, MODE, FORCED, 64, 8>(g, f, s, st)
-          : tv == 3 ? launch_split_o4<T, MODE, FORCED, 64, 4>(g, f, s, st)
-                    : launch_split_o4<T, MODE, FORCED, 32, 8>(g, f, s, st);
-    }
+    dim3 grd, blk;
+    const Part2d cp = part2d<T>(g, &grd, &blk);
+    cudaError_t e = launch_k(sbp_stress2d<T>, grd, blk, st, g, cp, (const T*)f.u_cur, f.lam, f.mu, f.sigma, s3_taps<T>());
+    if (e != cudaSuccess) return e;
+    e = launch_k(sbp_div2d<T, MODE, FORCED>, grd, blk, st, g, cp, f, s, s3_taps<T>());
     if (e != cudaSuccess) return e;
   } else {
     if constexpr (sizeof(T) == 4 && MODE != 3) {
