@@ -2548,9 +2548,8 @@ ewh_status ewh_batch_apply_S(ewh_batch* b, const double* const* v_in, double* co
   // Each member's own step graph, captured once, between its pack and unpack: the
   // members side by side, or one after another when one of them runs on chip (see
   // capture_branches).  A graph that has to be built is built while the members before
-  // it run.  Capturing all levels of all members anew for every call took 2.2 ms of 33.6 with
-  // per-level launches
-  // (258, 386 and 514 nodes a side, 22 right-hand sides each, FP32).
+  // it run.  Capturing all levels of all members anew for every call took 2.2 ms of 33.6
+  // with per-level launches (258, 386 and 514 nodes a side, 22 right-hand sides each, FP32).
   bool serial = false;
   for (ewh_ctx* c : b->p) {  // variants first: the members' timings must not overlap
     if (f64 && c->w64.variant < 0 && !c->w64.graph_S) autotune<double>(c, c->w64);
