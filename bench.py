@@ -825,14 +825,9 @@ def main():
     it = [i.iters for i in infos]
     peaks_fma = fma_peaks() if rank == 0 else None
     if peaks_fma and st.steps[0]:
-        if int(L.ewh_get_info(wh.ctx).kernel_variant[0]) in (1, 2):  # block fixed point: no FP64-FMA roofline
-            roofline["fp64_alu"] = {"kernel": "step2d_o4_fx (block fixed point), Pi 0 and the residual replacements",
-                                    "bound": "integer and FP64 pipes", "frac": None,
-                                    "gpt_updates_s": nodes * st.steps[0] / (st.wave_ms[0] * 1e-3) / 1e9}
-        else:
-            roofline["fp64_alu"] = alu_roofline(FLOPS_PER_NODE_LEVEL[2], nodes, st.wave_ms[0] / st.steps[0],
-                                                peaks_fma["fp64"], "FP64 per-level order-4 kernels (Pi 0 and the "
-                                                "residual replacements of the step)")
+        roofline["fp64_alu"] = alu_roofline(FLOPS_PER_NODE_LEVEL[2], nodes, st.wave_ms[0] / st.steps[0],
+                                            peaks_fma["fp64"], "FP64 per-level order-4 kernels (Pi 0 and the "
+                                            "residual replacements of the step)")
 
     extra = {}
     # the same step with CG windows under device control (the library's default)

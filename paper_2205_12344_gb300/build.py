@@ -17,10 +17,9 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "libewh.so")
-SOURCES = ["ewh_stencil.cu", "ewh_zmarch.cu", "ewh_ymarch.cu", "ewh_krylov.cu", "ewh_api.cu", "ewh_fx2d.cu", "ewh_small2d.cu",
+SOURCES = ["ewh_stencil.cu", "ewh_zmarch.cu", "ewh_ymarch.cu", "ewh_krylov.cu", "ewh_api.cu", "ewh_small2d.cu",
            "ewh_net.cu", "ewh_conv.cu", "ewh_peak.cu"]
-HEADERS = [os.path.join(CSRC, h) for h in ("ewh_internal.cuh", "ewh_march.cuh", "ewh_conv.cuh", "ewh_fixed.cuh",
-                                                  "ewh_order2.cuh")]
+HEADERS = [os.path.join(CSRC, h) for h in ("ewh_internal.cuh", "ewh_march.cuh", "ewh_conv.cuh", "ewh_order2.cuh")]
 HEADERS.append(os.path.join(ROOT, "include", "ewh.h"))
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-O2"]

@@ -17,7 +17,6 @@
 #include <vector>
 
 #include "../../include/ewh.h"
-#include "ewh_fixed.cuh"
 #include "ewh_internal.cuh"
 
 using namespace ewh;
@@ -191,34 +190,6 @@ __global__ void to_padded_kernel(Geom g, const double* __restrict__ src, const d
   }
 }
 
-// Count the blocks of 32 x 8 nodes (x 8 planes in 3D, each with the 2 nodes
-// around it) whose moduli differ by more than 2^FX_CONTRAST.
-__global__ void __launch_bounds__(256) steep_blocks_kernel(Geom g, const double* __restrict__ lam,
-                                                           const double* __restrict__ mu, int* __restrict__ count) {
-  const int x0 = blockIdx.x * 32 - 2, y0 = blockIdx.y * 8 - 2, z0 = g.dim == 3 ? blockIdx.z * 8 - 2 : 0;
-  const int nz = g.dim == 3 ? 12 : 1;
-  double hi = 0.0, lo = INFINITY;
-  for (int i = threadIdx.x; i < 36 * 12 * nz; i += 256) {
-    const int x = x0 + i % 36, y = y0 + i / 36 % 12, z = z0 + i / (36 * 12);
-    if (x < 0 || x >= g.n[0] || y < 0 || y >= g.n[1] || z < 0 || z >= g.n[2]) continue;
-    const long long o = ((long long)z * g.n[1] + y) * g.n[0] + x;
-    const double m = mu[o];
-    hi = fmax(hi, fmax(fabs(lam[o]), m));
-    lo = fmin(lo, m);
-  }
-  __shared__ double s_hi[8], s_lo[8];
-  for (int o = 16; o > 0; o >>= 1) {
-    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-  }
-  if (threadIdx.x % 32 == 0) s_hi[threadIdx.x / 32] = hi, s_lo[threadIdx.x / 32] = lo;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < 8; ++w) hi = fmax(hi, s_hi[w]), lo = fmin(lo, s_lo[w]);
-    if (hi > lo * (double)(1 << FX_CONTRAST)) atomicAdd(count, 1);
-  }
-}
-
 template <typename T>
 ewh_status build_wave(ewh_ctx* ctx, Wave<T>& w, const double* d_rho, const double* d_lam, const double* d_mu,
                       const double* d_f, const double* d_met) {
@@ -322,7 +293,7 @@ Wave<float>& wave_of<float>(ewh_ctx* c) { return c->w32; }
 // ---------------------------------------------------------------------------
 // Autotuner: pick the step-kernel variant of a context by timing.
 //
-// The candidates (order-4 pair, fixed-point, marching and on-chip forms; tile
+// The candidates (order-4 pair, marching and on-chip forms; tile
 // height of the order-2 2D kernel or its on-chip form) are timed on the context's own buffers with 2 warm-up and
 // 8 timed leapfrog levels each; the fastest wins.  Results are kept in a JSON
 // file ($EWH_TUNE_CACHE, else $HOME/.cache/ewh/tune.json) keyed by the GPU and
@@ -398,7 +369,7 @@ std::string tune_key(const ewh_ctx* ctx) {
       restricted = restricted || (ctx->w32.rplan[k].ok && (long long)ctx->w32.rplan[k].bx * ctx->w32.rplan[k].by <
                                                               RS_BATCH_MIN_BLOCK);
   if (ctx->batch_member && (sizeof(T) == 4 ? ctx->w32.splan.ok : ctx->w64.splan.ok)) restricted = true;  // small2d_ok
-  return name + "|v6" + (restricted ? "b" : "") + (g.mapped ? "|map" : "") + (g.contrast ? "|c" : "") + "|d" + std::to_string(g.dim) +
+  return name + "|v6" + (restricted ? "b" : "") + (g.mapped ? "|map" : "") + "|d" + std::to_string(g.dim) +
          "|o" + std::to_string(ctx->order) + "|" +
          (sizeof(T) == 8 ? "f64" : "f32") + "|" + std::to_string(g.n[0]) + "x" + std::to_string(g.n[1]) + "x" +
          std::to_string(g.n[2]) + "|r" + std::to_string(g.nrhs);
@@ -480,7 +451,7 @@ bool ymarch_ok(const ewh_ctx* ctx, const Wave<T>& w) {
 
 template <typename T>
 void autotune(ewh_ctx* ctx, Wave<T>& w) {
-  const int nbase = ctx->g.mapped ? 1 : step_variant_count(ctx->g.dim, ctx->order, sizeof(T));
+  const int nbase = ctx->g.mapped ? 1 : step_variant_count(ctx->g.dim, ctx->order);
   const char* force = getenv("EWH_STEP2D_O4");
   // a launcher named by the environment (the y-march exists in FP32 only)
   const bool forced_launcher = force && (force[0] == 's' || force[0] == 'f' || (force[0] == 'y' && sizeof(T) == 4));
@@ -2149,7 +2120,6 @@ ewh_status create_impl(const ewh_grid_desc* desc, const double* xmap, const doub
     s = build_wave<float>(ctx, ctx->w32, d_r, d_l, d_m, d_f, d_met);
   const long long n = total_unknowns(ctx);
   ctx->nblk = dot_blocks(g);
-  const dim3 steep_grid((g.n[0] + 31) / 32, (g.n[1] + 7) / 8, dim == 3 ? (g.n[2] + 7) / 8 : 1);
   if (s == EWH_OK) {
     ok = alloc_zero(&ctx->kx, n, ctx->st) == cudaSuccess && alloc_zero(&ctx->kr, n, ctx->st) == cudaSuccess &&
          alloc_zero(&ctx->kp, n, ctx->st) == cudaSuccess && alloc_zero(&ctx->kq, n, ctx->st) == cudaSuccess &&
@@ -2189,17 +2159,7 @@ ewh_status create_impl(const ewh_grid_desc* desc, const double* xmap, const doub
       s = fail(ctx, EWH_ECUDA, "mass kernel launch failed");
     ctx->launches += 1;
   }
-  const bool steep = s == EWH_OK && ctx->order == 4 && !mapped && steep_grid.y < 65536 && steep_grid.z < 65536;
-  if (steep) {
-    *ctx->h_flag = 0;
-    steep_blocks_kernel<<<steep_grid, 256, 0, ctx->st>>>(g, d_l, d_m, ctx->flags);
-    cudaMemcpyAsync(ctx->h_flag, ctx->flags, sizeof(int), cudaMemcpyDeviceToHost, ctx->st);
-    cudaMemsetAsync(ctx->flags, 0, sizeof(int), ctx->st);
-    ctx->launches += 1;
-  }
   cudaError_t e = cudaStreamSynchronize(ctx->st);
-  // more than one block in 32: the fixed-point steps would take their plain path too often
-  if (steep) g.contrast = (long long)*ctx->h_flag * 32 > (long long)steep_grid.x * steep_grid.y * steep_grid.z;
   cudaFree(d_met);
   d_met = nullptr;
   cudaFree(d_r);

@@ -34,7 +34,6 @@ struct Geom {
   long long nodes; // unknown nodes per component
   int nrhs;
   int variant;     // step-kernel variant chosen by the autotuner (host side)
-  int contrast;    // 1: moduli differ too much within the fixed-point steps' tiles (see FX_CONTRAST): they are not used
   int mapped;      // 1: curvilinear 2D grid (order 4): fluxes through WaveFields::met
 };
 
@@ -47,9 +46,9 @@ constexpr double SBP_CLOSURE[4][6] = {{-24.0 / 17, 59.0 / 34, -4.0 / 17, -3.0 / 
                                       {4.0 / 43, -59.0 / 86, 0.0, 59.0 / 86, -4.0 / 43, 0.0},
                                       {3.0 / 98, 0.0, -59.0 / 98, 0.0, 32.0 / 49, -4.0 / 49}};
 
-// Number of step-kernel variants worth timing for a geometry/order (bytes per value: elem).
-inline int step_variant_count(int dim, int order, int elem) {
-  if (dim == 2 && order == 4) return elem == 8 ? 3 : 1;  // stress + divergence pair; FP64 also two fixed-point tiles
+// Number of step-kernel variants worth timing for a geometry/order.
+inline int step_variant_count(int dim, int order) {
+  if (dim == 2 && order == 4) return 1;  // stress + divergence pair
   if (dim == 2 && order == 2) return 3;  // tile heights 8, 4, 16
   if (dim == 3 && order == 4) return 3;  // stress + divergence pair, fused z-march 64x8 and 32x8 (FP32)
   return 1;
@@ -269,14 +268,6 @@ constexpr int YM_VARIANT = 8;
 ZmPlan plan_ymarch(const Geom& g, const float* u_a, const float* u_b, unsigned* ctl);
 cudaError_t launch_ymarch(const Geom& g, const ZmPlan& p, const WaveFields<float>& f, StepMode mode,
                           const StepScalars& s, cudaStream_t st);
-
-// ---- fused 2D order-4 FP64 step in block fixed point (ewh_fx2d.cu) ------------
-// Step-kernel variants FX_VARIANT + shape of the 2D order-4 FP64 launcher:
-// tiles of 32 x 16 and 32 x 8 nodes (0 is the pair).
-constexpr int FX_VARIANT = 1;
-constexpr int FX_SHAPES = 2;
-cudaError_t launch_fx2d(const Geom& g, int shape, const WaveFields<double>& f, StepMode mode, const StepScalars& s,
-                        cudaStream_t st);
 
 // Message for ewh_last_error(NULL) of calls that have no context.
 void set_global_error(const std::string& msg);

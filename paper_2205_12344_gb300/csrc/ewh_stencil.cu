@@ -83,37 +83,6 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;"
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---------------------------------------------------------------------------
-// Time update shared by all kernels.  a = M^{-1} K u (FP of the state).
-// ---------------------------------------------------------------------------
-// The same update with delta^n, acc and f/rho already loaded (dprev, accprev
-// are not read at the first level; fr only when FORCED).
-template <typename T, int MODE, bool FORCED>
-__device__ __forceinline__ void leapfrog_update_pre(const WaveFields<T>& f, long long p, T uval, T a,
-                                                    const StepScalars& s, T dprev, T accprev, T fr) {
-  if (MODE == 3) {
-    f.u_next[p] = a;
-    return;
-  }
-  if (FORCED) a += fr * T(s.cosn);
-  if (MODE == STEP_FIRST) {
-    const T d = T(-0.5) * T(s.kt) * a;
-    const T un = uval + d;
-    f.delta[p] = d;
-    f.u_next[p] = un;
-    f.acc[p] = T(s.w0) * uval + T(s.wnew) * un;
-  } else {
-    const T d = dprev - T(s.kt) * a;
-    const T un = uval + d;
-    if (MODE == STEP_MID) {
-      f.delta[p] = d;
-      f.u_next[p] = un;
-    }
-    f.acc[p] = accprev + T(s.wnew) * un;
-  }
-}
-
-
-// ---------------------------------------------------------------------------
 // Order 2, 2D: 32 x TYV tile, one node per thread, halo 1 in shared memory.  The
 // medium is staged before the wait for the previous level.  Warps off the free sides
 // take the row without weights; next to one, a difference takes the node itself
@@ -657,10 +626,9 @@ static cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, cud
 }
 
 // 2D order-4 kernel variants (Geom::variant, chosen per context by the
-// autotuner): 0 = stress + divergence pair, FX_VARIANT + shape = the FP64
-// block-fixed-point step (ewh_fx2d.cu), YM_VARIANT = the FP32 y-march
-// (ewh_ymarch.cu).  EWH_STEP2D_O4=split|ym|fx overrides it (read whenever
-// launches are enqueued; a context captures its step graph once, on first use).
+// autotuner): 0 = stress + divergence pair (the only one in FP64), YM_VARIANT =
+// the FP32 y-march (ewh_ymarch.cu).  EWH_STEP2D_O4=split|ym overrides it (read
+// whenever launches are enqueued; a context captures its step graph once, on first use).
 // ---------------------------------------------------------------------------
 // Order 4 (SBP), 2D, in two launches: stresses, then divergence and update.  A
 // thread takes 16 bytes' worth of nodes along x (four in FP32, two in FP64) of the
@@ -674,7 +642,7 @@ static cudaError_t launch_k(void (*kernel)(KArgs...), dim3 grid, dim3 block, cud
 //
 // Per level, against one node a thread in shared-memory tiles with six-tap closures: FP32
 // 66^2 6.4 -> 3.6 us, 258^2 6.6 -> 3.9, 514^2 9.5 -> 6.1, 1026^2 22.6 -> 12.6, 2002^2
-// 94 -> 59 us; FP64 66^2 10.1 -> 5.5, 1026^2 106 -> 90 us.  Small grids are bound by the two
+// 94 -> 59 us; FP64 66^2 10.1 -> 5.5, 1026^2 106 -> 87 us.  Small grids are bound by the two
 // launches, FP32 by L2 and HBM (88 bytes a node and level; 2002^2: 0.88 of the copy
 // rate), FP64 by its pipe.  One launch over tiles with recomputed stresses was slower
 // at every size.
@@ -816,11 +784,32 @@ __global__ void __launch_bounds__(P2_THREADS) sbp_stress2d(Geom g, Part2d cp, co
   for (int k = 0; k < 3; ++k) st16(out + k * g.field, o[k]);
 }
 
+// Leapfrog / filter update of one value, kd = -M^{-1} K u / irh in units of 1 / kts (dl, ac: delta^n and
+// the filter's sum in, the new ones out); the operator alone: un = -kd kts irh.  The value
+// meets kts, then irh: the product of these two, rounded, would change every wave's
+// frequency alike, and M^{-1} K u alone exceeds the field by 1 / (c dt^2).
+template <typename T, int MODE, bool FORCED>
+__device__ __forceinline__ void pair_update(T kd, T kts, T irh, T fc, T fr, T w0, T wnew, T uv, T& dl, T& ac, T& un) {
+  const T k = kd * kts;
+  if (MODE == 3) {
+    un = -k * irh;
+    return;
+  }
+  T d = MODE == STEP_FIRST ? k * irh : dl + k * irh;
+  if (FORCED) d -= fr * fc;
+  if (MODE == STEP_FIRST) d *= T(0.5);
+  un = uv + d;
+  ac = MODE == STEP_FIRST ? w0 * uv + wnew * un : ac + wnew * un;
+  dl = d;
+}
+
 // Divergence and update of both kinds of grid: component c from the fields at qc (along
-// x) and rc (along y), in units of 1 / scale.
+// x) and rc (along y).  kts: c dt^2 (for the operator alone: 1) over the scale that the
+// fields and the differences carry.  ktcos: c dt^2 cos(w t_n).
 template <typename T, int MODE, bool FORCED>
 __device__ __forceinline__ void div2d_part(const Geom& g, const Part2d& cp, const WaveFields<T>& f, const StepScalars& s,
-                                           const S3Taps<T>& tp, int nf, int qu, int ru, int qv, int rv, T scale, T bscale) {
+                                           const S3Taps<T>& tp, int nf, int qu, int ru, int qv, int rv, double kts,
+                                           double ktcos) {
   constexpr int V = 16 / sizeof(T);
   constexpr bool RD = MODE == STEP_MID || MODE == STEP_LAST;
   int x, y;
@@ -836,21 +825,25 @@ __device__ __forceinline__ void div2d_part(const Geom& g, const Part2d& cp, cons
     __shared__ S3Taps<T> taps;
     load_taps(tp, taps);
     const bool unk = x >= 0 && is_unknown(g, x, y, 0);
-    const T irh = f.irh2[pc] * scale;
+    const T irh = f.irh2[pc];
     const T fr0 = FORCED ? f.frho[p0] : T(0), fr1 = FORCED ? f.frho[p0 + g.field] : T(0);
     pdl_wait();
     pdl_trigger();
     if (!unk) return;
     const T u0 = f.u_cur[p0], u1 = f.u_cur[p0 + g.field];
-    const T d0 = RD ? f.delta[p0] : T(0), d1 = RD ? f.delta[p0 + g.field] : T(0);
-    const T a0 = RD ? f.acc[p0] : T(0), a1 = RD ? f.acc[p0 + g.field] : T(0);
+    T d0 = RD ? f.delta[p0] : T(0), d1 = RD ? f.delta[p0 + g.field] : T(0);
+    T a0 = RD ? f.acc[p0] : T(0), a1 = RD ? f.acc[p0 + g.field] : T(0);
     const int cx = s3_class(x, g.n[0]), cy = s3_class(y, g.n[1]);
-    const T ih = bscale * T(48.0 / 17.0);
-    const T bx = x == 0 ? -ih : (x == g.n[0] - 1 ? ih : T(0)), by = y == 0 ? -ih : (y == g.n[1] - 1 ? ih : T(0));
-    const T ku = bx * fqu[0] + by * fru[0] - (s3_taps12(fqu, 1, cx, taps) + s3_taps12(fru, sy, cy, taps));
-    const T kv = bx * fqv[0] + by * frv[0] - (s3_taps12(fqv, 1, cx, taps) + s3_taps12(frv, sy, cy, taps));
-    leapfrog_update_pre<T, MODE, FORCED>(f, p0, u0, ku * irh, s, d0, a0, fr0);
-    leapfrog_update_pre<T, MODE, FORCED>(f, p0 + g.field, u1, kv * irh, s, d1, a1, fr1);
+    const T ih = T(12.0 * 48.0 / 17.0);
+    const T bx = x == 0 ? ih : (x == g.n[0] - 1 ? -ih : T(0)), by = y == 0 ? ih : (y == g.n[1] - 1 ? -ih : T(0));
+    const T ku = s3_taps12(fqu, 1, cx, taps) + s3_taps12(fru, sy, cy, taps) + (bx * fqu[0] + by * fru[0]);
+    const T kv = s3_taps12(fqv, 1, cx, taps) + s3_taps12(frv, sy, cy, taps) + (bx * fqv[0] + by * frv[0]);
+    T n0, n1;
+    pair_update<T, MODE, FORCED>(ku, T(kts), irh, T(ktcos), fr0, T(s.w0), T(s.wnew), u0, d0, a0, n0);
+    pair_update<T, MODE, FORCED>(kv, T(kts), irh, T(ktcos), fr1, T(s.w0), T(s.wnew), u1, d1, a1, n1);
+    if (MODE != STEP_LAST) f.u_next[p0] = n0, f.u_next[p0 + g.field] = n1;
+    if (MODE == STEP_FIRST || MODE == STEP_MID) f.delta[p0] = d0, f.delta[p0 + g.field] = d1;
+    if (MODE != 3) f.acc[p0] = a0, f.acc[p0 + g.field] = a1;
     return;
   }
   alignas(16) T irh[1][V], fr[2][V];
@@ -876,16 +869,8 @@ __device__ __forceinline__ void div2d_part(const Geom& g, const Part2d& cp, cons
     alignas(16) T un[V];
 #pragma unroll
     for (int k = 0; k < V; ++k) {
-      T a = (-dq[c][k] - dr[c][k]) * (irh[0][k] * scale);
-      if (MODE == 3) {  // operator only
-        un[k] = a;
-        continue;
-      }
-      if (FORCED) a += fr[c][k] * T(s.cosn);
-      const T d = MODE == STEP_FIRST ? T(-0.5) * T(s.kt) * a : dl[c][k] - T(s.kt) * a;
-      un[k] = uv[c][k] + d;
-      ac[c][k] = MODE == STEP_FIRST ? T(s.w0) * uv[c][k] + T(s.wnew) * un[k] : ac[c][k] + T(s.wnew) * un[k];
-      dl[c][k] = d;
+      pair_update<T, MODE, FORCED>(dq[c][k] + dr[c][k], T(kts), irh[0][k], T(ktcos), FORCED ? fr[c][k] : T(0), T(s.w0),
+                                   T(s.wnew), uv[c][k], dl[c][k], ac[c][k], un[k]);
     }
     if (MODE != STEP_LAST) st16(f.u_next + p, un);
     if (MODE == STEP_FIRST || MODE == STEP_MID) st16(f.delta + p, dl[c]);
@@ -896,9 +881,10 @@ __device__ __forceinline__ void div2d_part(const Geom& g, const Part2d& cp, cons
 // stresses xx, yy, xy (12 sigma)
 template <typename T, int MODE, bool FORCED>
 __global__ void __launch_bounds__(P2_THREADS) sbp_div2d(Geom g, Part2d cp, WaveFields<T> f, StepScalars s,
+                                                        double kts, double ktcos,
                                                         const __grid_constant__ S3Taps<T> tp) {
   if (g.dim != 2) return;
-  div2d_part<T, MODE, FORCED>(g, cp, f, s, tp, 3, 0, 2, 2, 1, T(1.0 / 144.0), T(12));
+  div2d_part<T, MODE, FORCED>(g, cp, f, s, tp, 3, 0, 2, 2, 1, kts, ktcos);
 }
 
 // ---------------------------------------------------------------------------
@@ -991,9 +977,10 @@ __global__ void __launch_bounds__(P2_THREADS) curv_stress2d(Geom g, Part2d cp, c
 // fluxes F^q_u, F^r_u, F^q_v, F^r_v; irh2 = 1 / (rho J h^2)
 template <typename T, int MODE, bool FORCED>
 __global__ void __launch_bounds__(P2_THREADS) curv_div2d(Geom g, Part2d cp, WaveFields<T> f, StepScalars s,
+                                                         double kts, double ktcos,
                                                          const __grid_constant__ S3Taps<T> tp) {
   if (g.dim != 2) return;
-  div2d_part<T, MODE, FORCED>(g, cp, f, s, tp, 4, 0, 1, 2, 3, T(1.0 / 12.0), T(12));
+  div2d_part<T, MODE, FORCED>(g, cp, f, s, tp, 4, 0, 1, 2, 3, kts, ktcos);
 }
 
 // Metric terms of a mapped grid (FP64, dense C-order planes, x fastest):
@@ -1091,7 +1078,8 @@ static cudaError_t launch_mode(const Geom& g, int order, const WaveFields<T>& f,
     cudaError_t e = launch_k(curv_stress2d<T>, grd, blk, st, g, cp, (const T*)f.u_cur, f.lam, f.mu, f.met, f.sigma,
                              s3_taps<T>());
     if (e != cudaSuccess) return e;
-    e = launch_k(curv_div2d<T, MODE, FORCED>, grd, blk, st, g, cp, f, s, s3_taps<T>());
+    e = launch_k(curv_div2d<T, MODE, FORCED>, grd, blk, st, g, cp, f, s, (MODE == 3 ? 1.0 : s.kt) / 12.0, s.kt * s.cosn,
+                 s3_taps<T>());
     if (e != cudaSuccess) return e;
     if (nl) *nl += 2;
     return cudaGetLastError();
@@ -1107,24 +1095,13 @@ static cudaError_t launch_mode(const Geom& g, int order, const WaveFields<T>& f,
       return cudaGetLastError();
     }
   }
-  if constexpr (sizeof(T) == 8 && MODE != 3) {
-    // fused block-fixed-point step: autotuner variants FX_VARIANT + shape; EWH_STEP2D_O4=fx|fx1 forces one
-    const char* ev = getenv("EWH_STEP2D_O4");
-    int shape = g.variant - FX_VARIANT;
-    if (ev) shape = (ev[0] == 'f' && ev[1] == 'x') ? (ev[2] == '1' ? 1 : 0) : -1;
-    if (g.dim == 2 && !g.contrast && shape >= 0 && shape < FX_SHAPES) {
-      cudaError_t e = launch_fx2d(g, shape, f, (StepMode)MODE, s, st);
-      if (e != cudaSuccess) return e;
-      if (nl) *nl += 1;
-      return cudaGetLastError();
-    }
-  }
   if (g.dim == 2) {
     dim3 grd, blk;
     const Part2d cp = part2d<T>(g, &grd, &blk);
     cudaError_t e = launch_k(sbp_stress2d<T>, grd, blk, st, g, cp, (const T*)f.u_cur, f.lam, f.mu, f.sigma, s3_taps<T>());
     if (e != cudaSuccess) return e;
-    e = launch_k(sbp_div2d<T, MODE, FORCED>, grd, blk, st, g, cp, f, s, s3_taps<T>());
+    e = launch_k(sbp_div2d<T, MODE, FORCED>, grd, blk, st, g, cp, f, s, (MODE == 3 ? 1.0 : s.kt) / 144.0, s.kt * s.cosn,
+                 s3_taps<T>());
     if (e != cudaSuccess) return e;
   } else {
     if constexpr (sizeof(T) == 4 && MODE != 3) {
