@@ -271,14 +271,16 @@ ewh_status ewh_reset_stats(ewh_ctx* ctx);
  * counterpart in the paper): the grid barrier of the on-chip wave solve (2D,
  * every time level in one cooperative launch per group of right-hand sides,
  * CTAs meeting once per level) and the mbarrier waits of the marching kernels
- * (2D y-march, 3D z-march) for their bulk-tensor copies; the FP32 limit of the
- * on-chip solve of small order-2 grids (its FP64 waits keep the default).  Every wait is
+ * (2D y-march, 3D z-march) for their bulk-tensor copies; and of the waits of the
+ * on-chip solve of small order-2 grids, in either precision.  Every wait is
  * bounded: after ns nanoseconds (default 1e9; the grid barrier also after 2^22
  * polls) the waiting CTA gives up (the on-chip solve raises an error flag and
  * every CTA leaves at its next barrier; a marching CTA waits, bounded, for its
  * copies in flight and returns), and the launch fills its remaining
  * accumulator nodes with NaN (so ewh_apply_S returns NaN and a solve sees an
- * FP32 breakdown and continues with the FP64 operator).  ns = 0 makes every
+ * FP32 breakdown and continues with the FP64 operator).  An FP64 wave solve
+ * that gives up is redone on the device without waits and returns the same
+ * result.  ns = 0 makes every
  * wait give up at once: a way to exercise that path without a hung GPU.  The
  * count of give-ups is in ewh_stats.grid_wait_timeouts.  Takes effect for the
  * next launch (the stream is synchronised first); a no-op on contexts that

@@ -438,8 +438,8 @@ bool is_small2d(const ewh_ctx* ctx, const Wave<T>& w, int v) {
 
 template <typename T>
 cudaError_t enqueue_small2d(ewh_ctx* ctx, Wave<T>& w, bool forced, int nsteps) {
-  const Small2dIO<T> io{w.u_a,    w.acc,  w.lam,   w.mu,   w.irh2, forced ? w.frho : nullptr, w.d_cosn,
-                        w.d_wnew, ctx->kt, ctx->weights[0], nsteps, w.xbuf, w.bar};
+  const Small2dIO<T> io{w.u_a,    w.u_b,    w.delta, w.acc,           w.lam,  w.mu,   w.irh2, forced ? w.frho : nullptr,
+                        w.d_cosn, w.d_wnew, ctx->kt, ctx->weights[0], nsteps, w.xbuf, w.bar};
   return launch_small2d<T>(ctx->g, w.splan, io, ctx->st);
 }
 
@@ -593,7 +593,7 @@ cudaError_t enqueue_steps(ewh_ctx* ctx, Wave<T>& w, bool forced, long long* nl) 
     return e;
   }
   if (is_small2d<T>(ctx, w, w.variant)) {
-    if (nl) *nl += 1;
+    if (nl) *nl += sizeof(T) == 8 ? 2 : 1;  // FP64: and the redo kernel
     return enqueue_small2d<T>(ctx, w, forced, N);
   }
   Geom gv = ctx->g;
@@ -2279,11 +2279,11 @@ ewh_status ewh_get_info(const ewh_ctx* ctx, ewh_problem_info* info) {
 ewh_status ewh_set_grid_wait(ewh_ctx* ctx, long long ns) {
   if (!ctx) return EWH_EINVAL;
   if (ns < 0) return fail(ctx, EWH_EINVAL, "grid wait limit must be >= 0 ns");
-  if (!ctx->w32.bar) return EWH_OK;  // this context never runs the on-chip solve
   const unsigned long long v = (unsigned long long)ns;
-  if (cudaStreamSynchronize(ctx->st) != cudaSuccess ||
-      cudaMemcpy(ctx->w32.bar + 2, &v, sizeof(v), cudaMemcpyHostToDevice) != cudaSuccess)
-    return fail(ctx, EWH_ECUDA, "setting the grid wait limit failed");
+  for (unsigned* bar : {ctx->w32.bar, ctx->w64.bar})
+    if (bar && (cudaStreamSynchronize(ctx->st) != cudaSuccess ||
+                cudaMemcpy(bar + 2, &v, sizeof(v), cudaMemcpyHostToDevice) != cudaSuccess))
+      return fail(ctx, EWH_ECUDA, "setting the grid wait limit failed");
   return EWH_OK;
 }
 

@@ -237,8 +237,10 @@ struct Small2dPlan {
 };
 template <typename T>
 struct Small2dIO {
-  const T* u0;  // u^0 (padded, 2 components per right-hand side)
-  T* acc;       // filter accumulator, written at the end (unknowns only)
+  T* u0;     // u^0 (padded, 2 components per right-hand side)
+  T* u1;     // u0, u1, delta: the state of an FP64 solve that is redone level by level
+  T* delta;
+  T* acc;    // filter accumulator, written at the end (unknowns only)
   const T* lam;
   const T* mu;
   const T* irh2;

@@ -17,6 +17,9 @@
 // 4.9 and 1.9 -> 1.6 us.
 // Bound by the store-to-poll latency through L2 and, in FP64, its pipe (20
 // instructions a thread).  Grids that do not fit one CTA an SM keep the tiles.
+//
+// A solve whose waits give up ends with NaN.  In FP64, which right-hand sides, residuals and
+// the solves that FP32 gave up on rest upon, a second launch then redoes it (step2d_o2_redo).
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -88,6 +91,39 @@ __device__ __forceinline__ bool s2_wait(const unsigned long long* w, unsigned ta
   return false;
 }
 
+// A node's row of K for one component in the form of the per-level kernels, times 2 h^2: axis a
+// along the component, b across.  A free side takes the node itself for the neighbour that is
+// missing, over half the width: offsets a0 .. b1 to the neighbours in an array of strides sx, sy.
+template <typename T>
+struct S2Node {
+  O2Row<T> cf;
+  int a0, a1, b0, b1;
+  __device__ __forceinline__ S2Node(const Geom& g, const T* lam, const T* mu, int comp, int x, int y, int sx, int sy) {
+    const long long pc = pidx(g, 0, 0, x, y, 0);
+    const bool lox = x == 0, hix = x == g.n[0] - 1, loy = y == 0, hiy = y == g.n[1] - 1;
+    const bool loa = comp ? loy : lox, hia = comp ? hiy : hix, lob = comp ? lox : loy, hib = comp ? hix : hiy;
+    const int ga = comp ? g.np[0] : 1, gb = comp ? 1 : g.np[0];  // neighbours in the padded medium
+    const int sa = comp ? sy : sx, sb = comp ? sx : sy;
+    a0 = loa ? 0 : -sa, a1 = hia ? 0 : sa, b0 = lob ? 0 : -sb, b1 = hib ? 0 : sb;
+    const T wa = loa || hia ? T(2) : T(1), wb = lob || hib ? T(2) : T(1);
+    const T l0 = lam[pc], m0 = mu[pc], p0 = l0 + T(2) * m0;
+    const long long qa0 = pc - (loa ? 0 : ga), qa1 = pc + (hia ? 0 : ga);
+    const long long qb0 = pc - (lob ? 0 : gb), qb1 = pc + (hib ? 0 : gb);
+    cf.ca0 = wa * (p0 + (lam[qa0] + T(2) * mu[qa0]));
+    cf.ca1 = wa * (p0 + (lam[qa1] + T(2) * mu[qa1]));
+    cf.cb0 = wb * (m0 + mu[qb0]);
+    cf.cb1 = wb * (m0 + mu[qb1]);
+    cf.la0 = T(0.5) * (loa ? T(-2) : wa) * wb * lam[qa0];
+    cf.la1 = T(0.5) * (hia ? T(-2) : wa) * wb * lam[qa1];
+    cf.mb0 = T(0.5) * (lob ? T(-2) : wb) * wa * mu[qb0];
+    cf.mb1 = T(0.5) * (hib ? T(-2) : wb) * wa * mu[qb1];
+  }
+  // 2 h^2 rho M^{-1} K u; U the node's value, V that of the other component
+  __device__ __forceinline__ T row(const T* U, const T* V, T u) const {
+    return o2_row(cf, u, O2Vals<T>{U[a0], U[a1], U[b0], U[b1], V[a0 + b0], V[a0 + b1], V[a1 + b0], V[a1 + b1]});
+  }
+};
+
 // NT_MAX: most threads of the CTA (512: no spills in FP64)
 template <typename T, bool FORCED, int NT_MAX>
 __global__ void __launch_bounds__(NT_MAX) step2d_o2_resident(Geom g, Small2dShape sh, Small2dIO<T> io) {
@@ -138,9 +174,7 @@ __global__ void __launch_bounds__(NT_MAX) step2d_o2_resident(Geom g, Small2dShap
       }
     }
   }
-  // this thread's node and component (warps hold one component): axis a along the
-  // component, b across; the row of K in the form of the per-level kernels, times 2 h^2
-  // (a free side takes the node itself for the missing neighbour, over half the width)
+  // this thread's node and component (warps hold one component)
   const int comp = t >= sh.P, j = t - comp * sh.P;
   const int jx = j % sh.bx, jy = j / sh.bx;
   const bool own = jy < wy && jx < wx;
@@ -148,29 +182,8 @@ __global__ void __launch_bounds__(NT_MAX) step2d_o2_resident(Geom g, Small2dShap
   const int ps = own ? (jy + 1) * SX + jx + 1 : SX + 1;
   const int x = X0 + (own ? jx : 0) + g.off[0], y = Y0 + (own ? jy : 0) + g.off[1];
   const long long pc = pidx(g, 0, 0, x, y, 0), p = pidx(g, rhs, comp, x, y, 0);
-  const bool lox = x == 0, hix = x == g.n[0] - 1, loy = y == 0, hiy = y == g.n[1] - 1;
-  const bool loa = comp ? loy : lox, hia = comp ? hiy : hix, lob = comp ? lox : loy, hib = comp ? hix : hiy;
-  const int ga = comp ? g.np[0] : 1, gb = comp ? 1 : g.np[0];  // neighbours in the padded medium
-  const int sa = comp ? SX : 1, sc = comp ? 1 : SX;            // ... and in the tile
-  const int a0 = loa ? 0 : -sa, a1 = hia ? 0 : sa, b0 = lob ? 0 : -sc, b1 = hib ? 0 : sc;
-  O2Row<T> cf;
-  T ks, fr = T(0);
-  {
-    const T wa = loa || hia ? T(2) : T(1), wb = lob || hib ? T(2) : T(1);
-    const T l0 = io.lam[pc], m0 = io.mu[pc], p0 = l0 + T(2) * m0;
-    const long long qa0 = pc - (loa ? 0 : ga), qa1 = pc + (hia ? 0 : ga);
-    const long long qb0 = pc - (lob ? 0 : gb), qb1 = pc + (hib ? 0 : gb);
-    cf.ca0 = wa * (p0 + (io.lam[qa0] + T(2) * io.mu[qa0]));
-    cf.ca1 = wa * (p0 + (io.lam[qa1] + T(2) * io.mu[qa1]));
-    cf.cb0 = wb * (m0 + io.mu[qb0]);
-    cf.cb1 = wb * (m0 + io.mu[qb1]);
-    cf.la0 = T(0.5) * (loa ? T(-2) : wa) * wb * io.lam[qa0];
-    cf.la1 = T(0.5) * (hia ? T(-2) : wa) * wb * io.lam[qa1];
-    cf.mb0 = T(0.5) * (lob ? T(-2) : wb) * wa * io.mu[qb0];
-    cf.mb1 = T(0.5) * (hib ? T(-2) : wb) * wa * io.mu[qb1];
-    ks = T(0.5 * io.kt) * io.irh2[pc];
-    if (FORCED) fr = io.frho[p];
-  }
+  const S2Node<T> nd(g, io.lam, io.mu, comp, x, y, 1, SX);
+  const T ks = T(0.5 * io.kt) * io.irh2[pc], fr = FORCED ? io.frho[p] : T(0);
   const int oc = comp ? -TP : TP;  // to the other component
   __syncthreads();
   T uv = sb[comp * TP + ps], d = T(0), ac = o2_mul(T(io.w0), uv);
@@ -196,9 +209,7 @@ __global__ void __launch_bounds__(NT_MAX) step2d_o2_resident(Geom g, Small2dShap
     }
     if (own) {
       const T* const U = cur + comp * TP + ps;
-      const T* const V = U + oc;
-      const O2Vals<T> nv{U[a0], U[a1], U[b0], U[b1], V[a0 + b0], V[a0 + b1], V[a1 + b0], V[a1 + b1]};
-      d = o2_delta<T, FORCED>(n == 0 ? T(0.5) * ks : ks, o2_row(cf, uv, nv), kc, fr, d);
+      d = o2_delta<T, FORCED>(n == 0 ? T(0.5) * ks : ks, nd.row(U, U + oc, uv), kc, fr, d);
       const T un = o2_add(uv, d);
       if (n + 1 < io.nsteps) {
         if (rim) s2_send(xs + ((n + 1) & 1) * half, un, (unsigned)(n + 1));
@@ -209,6 +220,32 @@ __global__ void __launch_bounds__(NT_MAX) step2d_o2_resident(Geom g, Small2dShap
     }
   }
   if (own) io.acc[p] = alive ? ac : T(NAN);
+}
+
+// The solve again, level by level over the whole grid, by one CTA per right-hand side that
+// waits for no other: the same bits, if a CTA of step2d_o2_resident gave up on a wait
+// (else it returns at once; the launch costs 2.2 of 309 us at 62 x 62 nodes and 183 levels).
+template <typename T, bool FORCED>
+__global__ void __launch_bounds__(1024) step2d_o2_redo(Geom g, Small2dIO<T> io) {
+  if (g.dim != 2 || *reinterpret_cast<const unsigned*>(io.xbuf) == 0u) return;
+  const int nu0 = g.nu[0], N = nu0 * g.nu[1];
+  for (int n = 0; n < io.nsteps; ++n) {
+    const T* const cur = n & 1 ? io.u1 : io.u0;
+    T* const next = n & 1 ? io.u0 : io.u1;
+    const T wn = T(io.wnew[n]), kc = FORCED ? T((n == 0 ? 0.5 : 1.0) * io.kt * io.cosn[n]) : T(0);
+    for (int i = threadIdx.x; i < 2 * N; i += blockDim.x) {
+      const int comp = i >= N, j = i - comp * N, x = j % nu0 + g.off[0], y = j / nu0 + g.off[1];
+      const long long p = pidx(g, blockIdx.x, comp, x, y, 0);
+      const S2Node<T> nd(g, io.lam, io.mu, comp, x, y, 1, g.np[0]);
+      const T ks = T(0.5 * io.kt) * io.irh2[pidx(g, 0, 0, x, y, 0)], fr = FORCED ? io.frho[p] : T(0);
+      const T uv = cur[p], k = nd.row(cur + p, cur + p + (comp ? -g.field : g.field), uv);
+      const T d = o2_delta<T, FORCED>(n == 0 ? T(0.5) * ks : ks, k, kc, fr, n == 0 ? T(0) : io.delta[p]);
+      const T un = o2_add(uv, d);
+      if (n + 1 < io.nsteps) next[p] = un, io.delta[p] = d;
+      io.acc[p] = o2_fma(wn, un, n == 0 ? o2_mul(T(io.w0), uv) : io.acc[p]);
+    }
+    __syncthreads();
+  }
 }
 
 template <typename T>
@@ -277,7 +314,13 @@ cudaError_t launch_small2d(const Geom& g, const Small2dPlan& p, const Small2dIO<
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, small2d_kernel<T>(2 * p.P, io.frho != nullptr), g, Small2dShape{p.px, p.px * p.py, p.bx, p.by, p.P}, io);
+  e = cudaLaunchKernelEx(&cfg, small2d_kernel<T>(2 * p.P, io.frho != nullptr), g, Small2dShape{p.px, p.px * p.py, p.bx, p.by, p.P}, io);
+  if (e != cudaSuccess || sizeof(T) == 4) return e;
+  if (io.frho)
+    step2d_o2_redo<T, true><<<g.nrhs, 1024, 0, st>>>(g, io);
+  else
+    step2d_o2_redo<T, false><<<g.nrhs, 1024, 0, st>>>(g, io);
+  return cudaGetLastError();
 }
 
 template Small2dPlan plan_small2d<float>(const Geom&);
