@@ -523,6 +523,12 @@ void autotune(ewh_ctx* ctx, Wave<T>& w) {
   int best = 0, best_base = 0;
   float best_ms = 1e30f, best_base_ms = 1e30f;
   const int N = ctx->nt * ctx->periods;
+  auto give_ups = [&]() {  // launches whose wait gave up (they end early: their time says nothing)
+    unsigned n = 0;
+    if (w.bar && cudaMemcpy(&n, w.bar + 4, sizeof(n), cudaMemcpyDeviceToHost) != cudaSuccess) cudaGetLastError();
+    return n;
+  };
+  unsigned gave_up = give_ups();
   for (int v = 0; v < nv; ++v) {
     float per_level = 1e30f;
     if (is_resident_variant(v) || (sm && v == SMALL2D_VARIANT)) {
@@ -538,6 +544,7 @@ void autotune(ewh_ctx* ctx, Wave<T>& w) {
         if (ok && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess)
           per_level = ms / ns;
         cudaGetLastError();
+        if (const unsigned n = give_ups(); n != gave_up) per_level = 1e30f, gave_up = n;
       }
     } else if (v < nbase || (v == YM_VARIANT && ym)) {
       Geom g = ctx->g;
@@ -553,6 +560,7 @@ void autotune(ewh_ctx* ctx, Wave<T>& w) {
       if (ok && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess)
         per_level = ms / 8;
       cudaGetLastError();
+      if (const unsigned n = give_ups(); n != gave_up) per_level = 1e30f, gave_up = n;
       if (per_level < best_base_ms) {
         best_base_ms = per_level;
         best_base = v;
