@@ -395,18 +395,20 @@ ewh_status ewh_fma_rate(int precision, double* flops_per_second, void* cuda_stre
 /* y = conv3x3(x, w) + bias (zero padding, stride 1), BF16 tensor-core MMA with
  * FP32 accumulation.  y_pre (FP32, may be NULL) receives the pre-activation,
  * y_act (BF16, may be NULL) the activation (act = 1: leaky ReLU 0.1, 0: none).
- * Ci a multiple of 16, Co a multiple of 8; bias may be NULL. */
+ * Ci a multiple of 16, Co a multiple of 8; bias may be NULL.  x and w 16-byte
+ * aligned (else EWH_EINVAL). */
 ewh_status ewh_conv3x3_fwd(const void* x, const void* w, const float* bias, float* y_pre, void* y_act, int act,
                            int N, int H, int W, int Ci, int Co, void* stream);
 
 /* dx = gradient with respect to x of <conv3x3(x, w), dy> (FP32 out, BF16 dy).
  * w_scratch: caller buffer of 9*Ci*Co bf16 for the flipped weights.  Ci, Co
- * multiples of 16. */
+ * multiples of 16; dy and w_scratch 16-byte aligned (else EWH_EINVAL). */
 ewh_status ewh_conv3x3_dgrad(const void* dy, const void* w, void* w_scratch, float* dx, int N, int H, int W, int Ci,
                              int Co, void* stream);
 
 /* dw (FP32, overwritten) = gradient with respect to w of <conv3x3(x, w), dy>.
- * x, dy BF16.  Ci, Co multiples of 16. */
+ * x, dy BF16 (any alignment; a slower kernel unless both are 16-byte aligned).
+ * Ci, Co multiples of 16. */
 ewh_status ewh_conv3x3_wgrad(const void* x, const void* dy, float* dw, int N, int H, int W, int Ci, int Co,
                              void* stream);
 

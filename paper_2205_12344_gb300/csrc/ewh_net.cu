@@ -33,6 +33,93 @@ __global__ void flip_transpose_kernel(const bf16* __restrict__ w, bf16* __restri
 }
 
 // ---------------------------------------------------------------------------
+// Weight gradient of operands that the bulk-tensor loads of ewh_conv.cu cannot
+// address (x or dy off a 16-byte boundary): element-wise loads, mma.sync.
+// dw[co][ky][kx][ci] = sum_p dy[p][co] x[p shifted][ci].
+// CTA: 64 co x 64 ci for one (ky, kx) and one chunk of pixels (split K);
+// partial sums are added into the FP32 result with atomics.  A = dy^T (co x
+// pixels), B = shifted x (pixels x ci), K step = 16 pixels.  Bound by its scalar
+// staging: 1590 us at 8 x 256 x 256, 32 -> 32 channels (37 us aligned), 970 us at
+// 8 x 64 x 64, 256 -> 128 (43 us).
+// ---------------------------------------------------------------------------
+// D (16x8 f32) += A (16x16 bf16, row) * B (16x8 bf16, col)
+__device__ __forceinline__ void mma_bf16_16816(float* d, const unsigned* a, const unsigned* b) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
+      "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+}
+
+__device__ __forceinline__ unsigned ld32(const bf16* p) { return *reinterpret_cast<const unsigned*>(p); }
+
+constexpr int WG_PIX_CHUNK = 1024, WG_LD = 24;  // LD: padded row length (bf16)
+
+__global__ void __launch_bounds__(128) conv3x3_wgrad_unaligned(const bf16* __restrict__ x, const bf16* __restrict__ dy,
+                                                            float* __restrict__ dw, int N, int H, int W, int Ci,
+                                                            int Co) {
+  __shared__ __align__(16) bf16 sA[64][WG_LD];  // [co][pixel]
+  __shared__ __align__(16) bf16 sB[64][WG_LD];  // [ci][pixel]
+  const int k9 = blockIdx.x % 9;
+  const int ky = k9 / 3, kx = k9 % 3;
+  const int ci_tiles = (Ci + 63) / 64;
+  const int co0 = (blockIdx.x / 9 / ci_tiles) * 64;
+  const int ci0 = ((blockIdx.x / 9) % ci_tiles) * 64;
+  const long long P = (long long)N * H * W;
+  const long long p_begin = (long long)blockIdx.y * WG_PIX_CHUNK;
+  const long long p_end = p_begin + WG_PIX_CHUNK < P ? p_begin + WG_PIX_CHUNK : P;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int gid = lane >> 2, tig = lane & 3;
+  // warp tile: 16 co (rows) x 64 ci (8 n-tiles)
+  float acc[8][4];
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) acc[j][q] = 0.f;
+  for (long long pb = p_begin; pb < p_end; pb += 16) {
+    // stage dy[p][co0..co0+63] transposed into sA[co][p], and the shifted x
+    for (int i = tid; i < 16 * 64; i += 128) {
+      const int pl = i / 64, c = i % 64;
+      const long long p = pb + pl;
+      bf16 vdy = __float2bfloat16(0.f), vx = __float2bfloat16(0.f);
+      if (p < p_end) {
+        if (co0 + c < Co) vdy = dy[p * Co + co0 + c];
+        const int n = (int)(p / ((long long)H * W));
+        const int r = (int)(p - (long long)n * H * W);
+        const int yy = r / W + ky - 1, xx = r % W + kx - 1;
+        if (ci0 + c < Ci && yy >= 0 && yy < H && xx >= 0 && xx < W)
+          vx = x[(((long long)n * H + yy) * W + xx) * Ci + ci0 + c];
+      }
+      sA[c][pl] = vdy;
+      sB[c][pl] = vx;
+    }
+    __syncthreads();
+    unsigned a[4];
+    const int r0 = warp * 16 + gid;
+    a[0] = ld32(&sA[r0][tig * 2]);
+    a[1] = ld32(&sA[r0 + 8][tig * 2]);
+    a[2] = ld32(&sA[r0][tig * 2 + 8]);
+    a[3] = ld32(&sA[r0 + 8][tig * 2 + 8]);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      unsigned b[2];
+      b[0] = ld32(&sB[j * 8 + gid][tig * 2]);
+      b[1] = ld32(&sB[j * 8 + gid][tig * 2 + 8]);
+      mma_bf16_16816(acc[j], a, b);
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int co = co0 + warp * 16 + gid + (q >= 2 ? 8 : 0);
+      const int ci = ci0 + j * 8 + tig * 2 + (q & 1);
+      if (co < Co && ci < Ci) atomicAdd(&dw[(((long long)co * 3 + ky) * 3 + kx) * Ci + ci], acc[j][q]);
+    }
+}
+
+// ---------------------------------------------------------------------------
 // Element-wise layers
 // ---------------------------------------------------------------------------
 // db[c] = sum over pixels of dy[p][c].  A cluster of CTAs takes 8 channels (one
@@ -232,6 +319,8 @@ int egrid(long long n) {
   return (int)(b < 1 ? 1 : b);
 }
 
+bool aligned16(const void* p) { return (uintptr_t)p % 16 == 0; }
+
 ewh_status nfail(const char* msg) {
   ewh::set_global_error(msg);
   return EWH_EINVAL;
@@ -255,6 +344,7 @@ ewh_status ewh_conv3x3_fwd(const void* x, const void* w, const float* bias, floa
                            int H, int W, int Ci, int Co, void* stream) {
   if (!x || !w || (!y_pre && !y_act) || N < 1 || H < 1 || W < 1 || Ci < 16 || Ci % 16 || Co < 8 || Co % 8)
     return nfail("ewh_conv3x3_fwd: bad arguments (Ci multiple of 16, Co multiple of 8)");
+  if (!aligned16(x) || !aligned16(w)) return nfail("ewh_conv3x3_fwd: x and w must be 16-byte aligned");
   return launched(ewh::launch_conv3x3(x, w, bias, y_pre, y_act, act, N, H, W, Ci, Co, (cudaStream_t)stream));
 }
 
@@ -262,6 +352,7 @@ ewh_status ewh_conv3x3_dgrad(const void* dy, const void* w, void* w_scratch, flo
                              int Co, void* stream) {
   if (!dy || !w || !w_scratch || !dx || Ci % 16 || Co % 16 || Ci < 16 || Co < 16)
     return nfail("ewh_conv3x3_dgrad: bad arguments (Ci, Co multiples of 16)");
+  if (!aligned16(dy) || !aligned16(w_scratch)) return nfail("ewh_conv3x3_dgrad: dy and w_scratch must be 16-byte aligned");
   cudaStream_t st = (cudaStream_t)stream;
   flip_transpose_kernel<<<egrid(9LL * Ci * Co), 256, 0, st>>>((const bf16*)w, (bf16*)w_scratch, Ci, Co);
   return launched(ewh::launch_conv3x3(dy, w_scratch, nullptr, dx, nullptr, 0, N, H, W, Co, Ci, st));
@@ -272,7 +363,15 @@ ewh_status ewh_conv3x3_wgrad(const void* x, const void* dy, float* dw, int N, in
   if (!x || !dy || !dw || Ci % 16 || Co % 16 || Ci < 16 || Co < 16)
     return nfail("ewh_conv3x3_wgrad: bad arguments (Ci, Co multiples of 16)");
   cudaStream_t st = (cudaStream_t)stream;
-  cudaMemsetAsync(dw, 0, sizeof(float) * 9LL * Ci * Co, st);
+  const cudaError_t e = cudaMemsetAsync(dw, 0, sizeof(float) * 9LL * Ci * Co, st);
+  if (e != cudaSuccess) return launched(e);
+  if (!aligned16(x) || !aligned16(dy)) {
+    const long long P = (long long)N * H * W;
+    const int ci_t = (Ci + 63) / 64, co_t = (Co + 63) / 64;
+    const dim3 grid((unsigned)(9 * ci_t * co_t), (unsigned)((P + WG_PIX_CHUNK - 1) / WG_PIX_CHUNK));
+    conv3x3_wgrad_unaligned<<<grid, 128, 0, st>>>((const bf16*)x, (const bf16*)dy, dw, N, H, W, Ci, Co);
+    return launched();
+  }
   return launched(ewh::launch_conv3x3_wgrad(x, dy, dw, N, H, W, Ci, Co, st));
 }
 
