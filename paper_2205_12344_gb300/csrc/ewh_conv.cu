@@ -11,8 +11,8 @@
 // times, not nine), and the zero padding of the convolution is the fill of
 // the loads' out-of-range part.
 //
-// Waits on the barriers are bounded (one second); a CTA that gives up writes
-// NaN to its outputs.
+// Waits on the barriers are bounded (one second); a CTA that gives up waits,
+// bounded again, for its loads and MMAs in flight and writes NaN to its outputs.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -118,6 +118,7 @@ __device__ __forceinline__ void cv_tmem_free(unsigned t, int cols) {
 struct CvBarriers {
   uint64_t full[CV_STAGES_MAX], empty[CV_STAGES_MAX], done;
   unsigned tmem;
+  int issued, multiplied;  // K steps whose loads were requested, whose MMAs were issued
 };
 
 // Barriers, tensor memory and the stage buffers of a CTA; returns the
@@ -137,6 +138,20 @@ __device__ __forceinline__ unsigned cv_begin(CvBarriers& b, unsigned char* raw, 
   __syncthreads();
   cv_fence_after();
   return (smem_u32(raw) + 1023u) & ~1023u;
+}
+// The end of the K loop: true when every MMA has completed, else after the
+// (bounded) waits of cv_drain.
+__device__ __forceinline__ bool cv_finish(CvBarriers& b, int steps, int stages) {
+  const bool ok = __syncthreads_and(cv_wait(&b.done, 0));  // issued, multiplied are written
+  if (!ok) {
+    if (threadIdx.x == 0)
+      cv_drain(b.issued, b.multiplied, steps, stages, [&](CvBar kind, int stage, unsigned parity) {
+        cv_wait(kind == CV_FULL ? b.full + stage : (kind == CV_EMPTY ? b.empty + stage : &b.done), parity);
+      });
+    __syncthreads();
+  }
+  cv_fence_after();
+  return ok;
 }
 __device__ __forceinline__ void cv_end(CvBarriers& b, int cols) {
   cv_fence_before();
@@ -180,7 +195,8 @@ __global__ void __launch_bounds__(CV_NT) conv3x3_tc(const __grid_constant__ CUte
   const int steps = 3 * (p.Ci / p.KC);
   const unsigned tmem = bars.tmem;
   if (t == 0) {  // loads: step = (channel block, horizontal tap)
-    for (int s = 0; s < steps; ++s) {
+    int s = 0;
+    for (; s < steps; ++s) {
       const int st = s % p.stages, c = (s / 3) * p.KC, kx = s % 3;
       if (s >= p.stages && !cv_wait(bars.empty + st, ((s / p.stages) - 1) & 1)) break;
       const unsigned a = base + st * p.stage_bytes, b = a + p.a_bytes;
@@ -189,9 +205,11 @@ __global__ void __launch_bounds__(CV_NT) conv3x3_tc(const __grid_constant__ CUte
       for (int ky = 0; ky < 3; ++ky)
         cv_load2(&mw, b + ky * p.b_bytes, bars.full + st, (3 * ky + kx) * p.Ci + c, co0);
     }
+    bars.issued = s;
   } else if (t == 32) {  // one thread issues the MMAs
     const unsigned idesc = cv_idesc(p.BN, false);
-    for (int s = 0; s < steps; ++s) {
+    int s = 0;
+    for (; s < steps; ++s) {
       const int st = s % p.stages;
       if (!cv_wait(bars.full + st, (s / p.stages) & 1)) break;
       cv_fence_after();
@@ -204,14 +222,13 @@ __global__ void __launch_bounds__(CV_NT) conv3x3_tc(const __grid_constant__ CUte
         }
       cv_commit(s + 1 < steps ? bars.empty + st : &bars.done);
     }
+    bars.multiplied = s;
   }
   __syncwarp();
   // epilogue: row = pixel; 16 columns at a time through a transpose in shared
   // memory (the stage buffers are free once the last MMA is done), so that
   // stores run along the channels of a pixel
-  const bool ok = cv_wait(&bars.done, 0);
-  cv_fence_after();
-  __syncthreads();
+  const bool ok = cv_finish(bars, steps, p.stages);
   float* const tr = reinterpret_cast<float*>(cv_raw + (base - smem_u32(cv_raw))) + warp * CV_EPI;
   const float nanv = __int_as_float(0x7fc00000);
   for (int cb = 0; cb < p.BN && co0 + cb < p.Co; cb += 16) {
@@ -308,7 +325,8 @@ __global__ void __launch_bounds__(CV_NT) conv3x3_wgrad_tc(const __grid_constant_
   const int q0 = blockIdx.x * WG_PER, steps = min(WG_PER, p.patches - q0);
   const unsigned tmem = bars.tmem;
   if (t == 0) {
-    for (int s = 0; s < steps; ++s) {
+    int s = 0;
+    for (; s < steps; ++s) {
       const int st = s % p.stages;
       if (s >= p.stages && !cv_wait(bars.empty + st, ((s / p.stages) - 1) & 1)) break;
       const int q = q0 + s, n = q / (p.tx * p.ty), rem = q - n * p.tx * p.ty;
@@ -324,11 +342,13 @@ __global__ void __launch_bounds__(CV_NT) conv3x3_wgrad_tc(const __grid_constant_
         for (int kx = 0; kx < 3; ++kx) cv_load4(&mx, x + kx * p.x_copy, bars.full + st, ci0, x0 + kx - 1, y0 - 1, n);
       }
     }
+    bars.issued = s;
   } else if (t == 32) {
     const unsigned idesc = cv_idesc(p.NB, true);
     const unsigned lbo = wide ? p.x_copy : 8 * p.rowx;       // between the blocks of M rows
     const unsigned off = wide ? 8 * p.rowx : p.x_copy;       // between the three MMAs of a K step
-    for (int s = 0; s < steps; ++s) {
+    int s = 0;
+    for (; s < steps; ++s) {
       const int st = s % p.stages;
       if (!cv_wait(bars.full + st, (s / p.stages) & 1)) break;
       cv_fence_after();
@@ -342,10 +362,10 @@ __global__ void __launch_bounds__(CV_NT) conv3x3_wgrad_tc(const __grid_constant_
       }
       cv_commit(s + 1 < steps ? bars.empty + st : &bars.done);
     }
+    bars.multiplied = s;
   }
   __syncwarp();
-  const bool ok = cv_wait(&bars.done, 0);
-  cv_fence_after();
+  const bool ok = cv_finish(bars, steps, p.stages);
   // row m, column j NB + co: consecutive lanes are consecutive ci
   const int m = warp * 32 + lane;
   const int ci = ci0 + (wide ? m : m % p.KC), kyr = m / p.KC;
