@@ -461,12 +461,13 @@ cudaError_t launch_conv3x3(const void* x, const void* w, const float* bias, floa
   p.pre = pre;
   p.out = (bf16*)out;
   p.vec = ((uintptr_t)pre % 16 == 0 && (uintptr_t)out % 8 == 0) ? 1 : 0;
+  // ahead of the tensor maps: a runtime call, which binds a context to a thread that has none
+  cudaError_t e = cudaFuncSetAttribute(conv3x3_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, CV_SMEM_CTA);
+  if (e != cudaSuccess) return e;
   CUtensorMap mx, mw;
   if (!map_pixels(&mx, x, N, H, W, Ci, p.KC, CV_PY + 2) || !map_weights(&mw, w, Ci, Co, p.KC, p.BN))
     return launch_err(false);
   const int bytes = shared_bytes(p.stage_bytes, std::min(3 * (Ci / p.KC), p.KC == 64 ? 2 : 3), p.cols, &p.stages);
-  cudaError_t e = cudaFuncSetAttribute(conv3x3_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, CV_SMEM_CTA);
-  if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)((long long)N * p.tx * p.ty), (unsigned)((Co + p.BN - 1) / p.BN));
   conv3x3_tc<<<grid, CV_NT, bytes, st>>>(mx, mw, p);
   return launch_err(true);
@@ -501,11 +502,11 @@ cudaError_t launch_conv3x3_wgrad(const void* x, const void* dy, float* dw, int N
   const int blocks = p.cob * (wide ? 3 * ((Ci + 127) / 128) : Ci / p.KC);
   const int bytes = shared_bytes(p.stage_bytes, 2, p.cols, &p.stages);
   p.dw = dw;
+  cudaError_t e = cudaFuncSetAttribute(conv3x3_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, CV_SMEM_CTA);
+  if (e != cudaSuccess) return e;  // before the maps, as above
   CUtensorMap mx, mo;
   if (!map_pixels(&mx, x, N, H, W, Ci, p.KC, CV_PY + 2) || !map_pixels(&mo, dy, N, H, W, Co, p.KO, CV_PY))
     return launch_err(false);
-  cudaError_t e = cudaFuncSetAttribute(conv3x3_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, CV_SMEM_CTA);
-  if (e != cudaSuccess) return e;
   const dim3 grid((unsigned)((p.patches + WG_PER - 1) / WG_PER), (unsigned)blocks);
   conv3x3_wgrad_tc<<<grid, CV_NT, bytes, st>>>(mx, mo, p);
   return launch_err(true);
