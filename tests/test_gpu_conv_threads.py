@@ -1,5 +1,5 @@
 """The convolutions called from threads other than the one that set the GPU up: first calls of a
-thread."""
+thread, one after another and of several threads at once (streams and buffers of their own)."""
 import os
 import subprocess
 import sys
@@ -64,3 +64,8 @@ def _run(how):
 @pytest.mark.parametrize("how", ["fwd", "wgrad"])
 def test_first_call_of_a_thread(how):
     _run(how)
+
+
+@pytest.mark.parametrize("attempt", range(4))  # a race: one program shows it only now and then
+def test_first_calls_of_several_threads(attempt):
+    _run("at once")
