@@ -118,12 +118,13 @@ __device__ __forceinline__ void cv_tmem_free(unsigned t, int cols) {
 struct CvBarriers {
   uint64_t full[CV_STAGES_MAX], empty[CV_STAGES_MAX], done;
   unsigned tmem;
-  int issued, multiplied;  // K steps whose loads were requested, whose MMAs were issued
+  int issued, multiplied;  // K steps whose loads were requested, whose MMAs were issued: all, unless a wait gave up (noted
+                           // there: a store after the loops slows the weight gradient by 4%)
 };
 
 // Barriers, tensor memory and the stage buffers of a CTA; returns the
 // 1024-byte aligned shared address of stage 0.
-__device__ __forceinline__ unsigned cv_begin(CvBarriers& b, unsigned char* raw, int cols) {
+__device__ __forceinline__ unsigned cv_begin(CvBarriers& b, unsigned char* raw, int cols, int steps) {
   if (threadIdx.x == 0) {
     for (int k = 0; k < CV_STAGES_MAX; ++k) {
       mbar_init(b.full + k, 1);
@@ -133,29 +134,23 @@ __device__ __forceinline__ unsigned cv_begin(CvBarriers& b, unsigned char* raw, 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
+  if (threadIdx.x == 96) b.issued = b.multiplied = steps;
   if (threadIdx.x >= 64 && threadIdx.x < 96) cv_tmem_alloc(&b.tmem, cols);
   cv_fence_before();
   __syncthreads();
   cv_fence_after();
   return (smem_u32(raw) + 1023u) & ~1023u;
 }
-// The end of the K loop: true when every MMA has completed, else after the
-// (bounded) waits of cv_drain.
-__device__ __forceinline__ bool cv_finish(CvBarriers& b, int steps, int stages) {
-  const bool ok = __syncthreads_and(cv_wait(&b.done, 0));  // issued, multiplied are written
-  if (!ok) {
+// The CTA's end; ok: this thread saw every MMA complete (else cv_drain's bounded waits first).
+__device__ __forceinline__ void cv_end(CvBarriers& b, int cols, bool ok, int steps, int stages) {
+  cv_fence_before();
+  if (!__syncthreads_and(ok)) {
     if (threadIdx.x == 0)
       cv_drain(b.issued, b.multiplied, steps, stages, [&](CvBar kind, int stage, unsigned parity) {
         cv_wait(kind == CV_FULL ? b.full + stage : (kind == CV_EMPTY ? b.empty + stage : &b.done), parity);
       });
     __syncthreads();
   }
-  cv_fence_after();
-  return ok;
-}
-__device__ __forceinline__ void cv_end(CvBarriers& b, int cols) {
-  cv_fence_before();
-  __syncthreads();
   if (threadIdx.x >= 64 && threadIdx.x < 96) cv_tmem_free(b.tmem, cols);
 }
 
@@ -186,32 +181,35 @@ __global__ void __launch_bounds__(CV_NT) conv3x3_tc(const __grid_constant__ CUte
                                                     const __grid_constant__ CUtensorMap mw, ConvArgs p) {
   extern __shared__ unsigned char cv_raw[];
   __shared__ CvBarriers bars;
-  const unsigned base = cv_begin(bars, cv_raw, p.cols);
+  const int steps = 3 * (p.Ci / p.KC);
+  const unsigned base = cv_begin(bars, cv_raw, p.cols, steps);
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const int tile = blockIdx.x;
   const int n = tile / (p.tx * p.ty), rem = tile - n * p.tx * p.ty;
   const int y0 = (rem / p.tx) * CV_PY, x0 = (rem % p.tx) * CV_PX;
   const int co0 = blockIdx.y * p.BN;
-  const int steps = 3 * (p.Ci / p.KC);
   const unsigned tmem = bars.tmem;
   if (t == 0) {  // loads: step = (channel block, horizontal tap)
-    int s = 0;
-    for (; s < steps; ++s) {
+    for (int s = 0; s < steps; ++s) {
       const int st = s % p.stages, c = (s / 3) * p.KC, kx = s % 3;
-      if (s >= p.stages && !cv_wait(bars.empty + st, ((s / p.stages) - 1) & 1)) break;
+      if (s >= p.stages && !cv_wait(bars.empty + st, ((s / p.stages) - 1) & 1)) {
+        bars.issued = s;
+        break;
+      }
       const unsigned a = base + st * p.stage_bytes, b = a + p.a_bytes;
       cv_expect(bars.full + st, p.a_bytes + 3 * p.b_bytes);
       cv_load4(&mx, a, bars.full + st, c, x0 + kx - 1, y0 - 1, n);
       for (int ky = 0; ky < 3; ++ky)
         cv_load2(&mw, b + ky * p.b_bytes, bars.full + st, (3 * ky + kx) * p.Ci + c, co0);
     }
-    bars.issued = s;
   } else if (t == 32) {  // one thread issues the MMAs
     const unsigned idesc = cv_idesc(p.BN, false);
-    int s = 0;
-    for (; s < steps; ++s) {
+    for (int s = 0; s < steps; ++s) {
       const int st = s % p.stages;
-      if (!cv_wait(bars.full + st, (s / p.stages) & 1)) break;
+      if (!cv_wait(bars.full + st, (s / p.stages) & 1)) {
+        bars.multiplied = s;
+        break;
+      }
       cv_fence_after();
       const unsigned a = base + st * p.stage_bytes, b = a + p.a_bytes;
       for (int ky = 0; ky < 3; ++ky)
@@ -222,13 +220,14 @@ __global__ void __launch_bounds__(CV_NT) conv3x3_tc(const __grid_constant__ CUte
         }
       cv_commit(s + 1 < steps ? bars.empty + st : &bars.done);
     }
-    bars.multiplied = s;
   }
   __syncwarp();
   // epilogue: row = pixel; 16 columns at a time through a transpose in shared
   // memory (the stage buffers are free once the last MMA is done), so that
   // stores run along the channels of a pixel
-  const bool ok = cv_finish(bars, steps, p.stages);
+  const bool ok = cv_wait(&bars.done, 0);
+  cv_fence_after();
+  __syncthreads();
   float* const tr = reinterpret_cast<float*>(cv_raw + (base - smem_u32(cv_raw))) + warp * CV_EPI;
   const float nanv = __int_as_float(0x7fc00000);
   for (int cb = 0; cb < p.BN && co0 + cb < p.Co; cb += 16) {
@@ -277,7 +276,7 @@ __global__ void __launch_bounds__(CV_NT) conv3x3_tc(const __grid_constant__ CUte
     }
     __syncwarp();
   }
-  cv_end(bars, p.cols);
+  cv_end(bars, p.cols, ok, steps, p.stages);
 }
 
 // ---------------------------------------------------------------------------
@@ -314,7 +313,8 @@ __global__ void __launch_bounds__(CV_NT) conv3x3_wgrad_tc(const __grid_constant_
                                                           const __grid_constant__ CUtensorMap mo, WgradArgs p) {
   extern __shared__ unsigned char cv_raw[];
   __shared__ CvBarriers bars;
-  const unsigned base = cv_begin(bars, cv_raw, p.cols);
+  const int q0 = blockIdx.x * WG_PER, steps = min(WG_PER, p.patches - q0);
+  const unsigned base = cv_begin(bars, cv_raw, p.cols, steps);
   const int t = threadIdx.x, warp = t >> 5, lane = t & 31;
   const bool wide = p.KC == 64;
   int blk = blockIdx.y;
@@ -322,13 +322,14 @@ __global__ void __launch_bounds__(CV_NT) conv3x3_wgrad_tc(const __grid_constant_
   blk /= p.cob;
   const int kxf = wide ? blk % 3 : 0;
   const int ci0 = wide ? (blk / 3) * 128 : blk * p.KC;
-  const int q0 = blockIdx.x * WG_PER, steps = min(WG_PER, p.patches - q0);
   const unsigned tmem = bars.tmem;
   if (t == 0) {
-    int s = 0;
-    for (; s < steps; ++s) {
+    for (int s = 0; s < steps; ++s) {
       const int st = s % p.stages;
-      if (s >= p.stages && !cv_wait(bars.empty + st, ((s / p.stages) - 1) & 1)) break;
+      if (s >= p.stages && !cv_wait(bars.empty + st, ((s / p.stages) - 1) & 1)) {
+        bars.issued = s;
+        break;
+      }
       const int q = q0 + s, n = q / (p.tx * p.ty), rem = q - n * p.tx * p.ty;
       const int y0 = (rem / p.tx) * CV_PY, x0 = (rem % p.tx) * CV_PX;
       const unsigned o = base + st * p.stage_bytes, x = o + p.o_bytes;
@@ -342,15 +343,16 @@ __global__ void __launch_bounds__(CV_NT) conv3x3_wgrad_tc(const __grid_constant_
         for (int kx = 0; kx < 3; ++kx) cv_load4(&mx, x + kx * p.x_copy, bars.full + st, ci0, x0 + kx - 1, y0 - 1, n);
       }
     }
-    bars.issued = s;
   } else if (t == 32) {
     const unsigned idesc = cv_idesc(p.NB, true);
     const unsigned lbo = wide ? p.x_copy : 8 * p.rowx;       // between the blocks of M rows
     const unsigned off = wide ? 8 * p.rowx : p.x_copy;       // between the three MMAs of a K step
-    int s = 0;
-    for (; s < steps; ++s) {
+    for (int s = 0; s < steps; ++s) {
       const int st = s % p.stages;
-      if (!cv_wait(bars.full + st, (s / p.stages) & 1)) break;
+      if (!cv_wait(bars.full + st, (s / p.stages) & 1)) {
+        bars.multiplied = s;
+        break;
+      }
       cv_fence_after();
       const unsigned o = base + st * p.stage_bytes, x = o + p.o_bytes;
       for (int k = 0; k < CV_PY; k += 2) {
@@ -362,10 +364,10 @@ __global__ void __launch_bounds__(CV_NT) conv3x3_wgrad_tc(const __grid_constant_
       }
       cv_commit(s + 1 < steps ? bars.empty + st : &bars.done);
     }
-    bars.multiplied = s;
   }
   __syncwarp();
-  const bool ok = cv_finish(bars, steps, p.stages);
+  const bool ok = cv_wait(&bars.done, 0);
+  cv_fence_after();
   // row m, column j NB + co: consecutive lanes are consecutive ci
   const int m = warp * 32 + lane;
   const int ci = ci0 + (wide ? m : m % p.KC), kyr = m / p.KC;
@@ -385,7 +387,7 @@ __global__ void __launch_bounds__(CV_NT) conv3x3_wgrad_tc(const __grid_constant_
         __syncwarp();
       }
     }
-  cv_end(bars, p.cols);
+  cv_end(bars, p.cols, ok, steps, p.stages);
 }
 
 // ---- host side ----------------------------------------------------------------
