@@ -227,6 +227,7 @@ ewh_status build_wave(ewh_ctx* ctx, Wave<T>& w, const double* d_rho, const doubl
       }
   }
   EWH_CU(cudaGetLastError());
+  // (not in a batch: its members' launches run side by side, and this one wants the GPU)
   if (g.dim == 2 && ctx->order == 2 && !g.mapped && !ctx->implicit && !ctx->batch_member) {
     w.splan = plan_small2d<T>(g);
     if (w.splan.ok) EWH_CU(cudaMalloc(&w.xbuf, small2d_words(g, sizeof(T)) * sizeof(unsigned long long)));
@@ -368,7 +369,7 @@ std::string tune_key(const ewh_ctx* ctx) {
     for (int k = 0; k < RS_SHAPES; ++k)
       restricted = restricted || (ctx->w32.rplan[k].ok && (long long)ctx->w32.rplan[k].bx * ctx->w32.rplan[k].by <
                                                               RS_BATCH_MIN_BLOCK);
-  if (ctx->batch_member && (sizeof(T) == 4 ? ctx->w32.splan.ok : ctx->w64.splan.ok)) restricted = true;  // small2d_ok
+  if (ctx->batch_member && g.dim == 2 && ctx->order == 2) restricted = true;  // no on-chip solve (build_wave)
   return name + "|v6" + (restricted ? "b" : "") + (g.mapped ? "|map" : "") + "|d" + std::to_string(g.dim) +
          "|o" + std::to_string(ctx->order) + "|" +
          (sizeof(T) == 8 ? "f64" : "f32") + "|" + std::to_string(g.n[0]) + "x" + std::to_string(g.n[1]) + "x" +
@@ -422,12 +423,11 @@ cudaError_t enqueue_resident(ewh_ctx* ctx, Wave<T>& w, int v, bool forced, int n
   }
 }
 
-// The on-chip solve of small order-2 2D grids usable by this context?  (Not in a batch:
-// its members' launches run side by side, and this one wants the GPU.)
+// The on-chip solve of small order-2 2D grids usable by this context?
 template <typename T>
-bool small2d_ok(const ewh_ctx* ctx, const Wave<T>& w) {
+bool small2d_ok(const Wave<T>& w) {
   const char* e = getenv("EWH_RESIDENT");
-  return w.splan.ok && !ctx->batch_member && !(e && e[0] == '0');
+  return w.splan.ok && !(e && e[0] == '0');
 }
 
 // The variant runs all levels of a wave solve in one launch?
@@ -460,7 +460,7 @@ void autotune(ewh_ctx* ctx, Wave<T>& w) {
   const bool ym = ymarch_ok<T>(ctx, w) && !forced_launcher;
   // candidates: the launcher's own variants [0, nbase), the resident shapes,
   // the y-march (only the launcher's own when the environment names one)
-  const bool sm = small2d_ok<T>(ctx, w);
+  const bool sm = small2d_ok<T>(w);
   const int nv = ym ? YM_VARIANT + 1 : (any_res ? VARIANT_RESIDENT + RS_SHAPES : (sm ? SMALL2D_VARIANT + 1 : nbase));
   w.fallback = 0;
   if (force && force[0] == 'r') {  // EWH_STEP2D_O4=r, r0, r1, r2: resident solve of that CTA shape
@@ -1911,7 +1911,7 @@ namespace {
 // Context creation; xmap/ymap (node coordinates of a mapped 2D grid) may be null.
 ewh_status create_impl(const ewh_grid_desc* desc, const double* xmap, const double* ymap, const double* rho,
                        const double* lambda, const double* mu, double omega, const double* forcing, int nrhs,
-                       void* cuda_stream, ewh_ctx** out) {
+                       void* cuda_stream, ewh_ctx** out, bool batch_member = false) {
   if (!out) return fail(nullptr, EWH_EINVAL, "out is NULL");
   *out = nullptr;
   ewh_status vs = validate_desc(desc, nrhs);
@@ -2017,6 +2017,7 @@ ewh_status create_impl(const ewh_grid_desc* desc, const double* xmap, const doub
   }
 
   ewh_ctx* ctx = new ewh_ctx();
+  ctx->batch_member = batch_member;
   ctx->order = desc->order;
   ctx->precision = desc->precision;
   ctx->periods = desc->periods;
@@ -2470,15 +2471,14 @@ ewh_status ewh_batch_create(const ewh_problem* probs, int nprob, void* cuda_stre
     if (probs[k].desc.implicit) return fail(nullptr, EWH_EINVAL, "batch members must use the explicit scheme");
   for (int k = 0; k < nprob; ++k) {
     ewh_ctx* c = nullptr;
-    ewh_status s = ewh_create(&probs[k].desc, probs[k].rho, probs[k].lambda, probs[k].mu, probs[k].omega,
-                              probs[k].forcing, probs[k].nrhs, cuda_stream, &c);
+    ewh_status s = create_impl(&probs[k].desc, nullptr, nullptr, probs[k].rho, probs[k].lambda, probs[k].mu,
+                               probs[k].omega, probs[k].forcing, probs[k].nrhs, cuda_stream, &c, true);
     if (s != EWH_OK) {
       const std::string m = "member " + std::to_string(k) + ": " + g_create_error;
       ewh_batch_destroy(b);
       g_create_error = m;
       return s;
     }
-    c->batch_member = true;
     b->p.push_back(c);
   }
   b->joins.resize(nprob, nullptr);
