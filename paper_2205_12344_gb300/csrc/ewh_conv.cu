@@ -306,11 +306,50 @@ struct WgradArgs {
   int NB, cols, cob;        // output channels per CTA, tensor-memory columns, blocks of output channels
   int x_copy;               // bytes of one staged x patch (one horizontal tap or channel block)
   int stages, o_bytes, stage_bytes, tx_bytes;
+  int ragged;               // the patches cover more than the images
+  const bf16 *x, *dy;
   float* dw;
 };
 
+// A pixel of a patch beyond the image is zero in dy, but it meets values inside the image in x: an
+// infinity or a NaN there makes NaN of sums that the pixel does not belong to.  So
+// sums that came out as NaN in images that the patches do not divide are formed again, one by
+// one, over the pixels of the images.
+__device__ float wgrad_plain(const WgradArgs& p, int q0, int steps, int co, int tap, int ci) {
+  float s = 0.f;
+  for (int q = q0; q < q0 + steps; ++q) {
+    const int n = q / (p.tx * p.ty), rem = q - n * p.tx * p.ty;
+    const int y0 = (rem / p.tx) * CV_PY, x0 = (rem % p.tx) * CV_PX;
+    for (int i = 0; i < CV_ROWS; ++i) {
+      const int y = y0 + i / CV_PX, x = x0 + i % CV_PX, yy = y + tap / 3 - 1, xx = x + tap % 3 - 1;
+      if (y >= p.H || x >= p.W) continue;
+      const bool in = yy >= 0 && yy < p.H && xx >= 0 && xx < p.W;  // the zero padding takes part
+      const float a = in ? __bfloat162float(p.x[(((long long)n * p.H + yy) * p.W + xx) * p.Ci + ci]) : 0.f;
+      s += __bfloat162float(p.dy[(((long long)n * p.H + y) * p.W + x) * p.Co + co]) * a;
+    }
+  }
+  return s;
+}
+// The groups of 16 columns marked in `redo` (bit j 4 + column / 16) of this warp's rows, added to dw.
+__device__ __noinline__ void wgrad_redo(const WgradArgs& p, unsigned redo, unsigned trow, int q0, int steps, int co0,
+                                        int tap0, int dtap, int ci, bool live) {
+  for (; redo; redo &= redo - 1) {
+    const int bit = __ffs(redo) - 1, j = bit / 4, cb = bit % 4 * 16;
+    float v[16];
+    cv_ld16(trow + j * p.NB + cb, v);
+    for (int i = 0; i < 16 && live; ++i) {
+      const int co = co0 + cb + i, tap = tap0 + dtap * j;
+      if (co >= p.Co) break;
+      const float a = isnan(v[i]) ? wgrad_plain(p, q0, steps, co, tap, ci) : v[i];
+      atomicAdd(p.dw + ((long long)co * 9 + tap) * p.Ci + ci, a);
+    }
+    __syncwarp();
+  }
+}
+
 __global__ void __launch_bounds__(CV_NT) conv3x3_wgrad_tc(const __grid_constant__ CUtensorMap mx,
-                                                          const __grid_constant__ CUtensorMap mo, WgradArgs p) {
+                                                          const __grid_constant__ CUtensorMap mo,
+                                                          const __grid_constant__ WgradArgs p) {
   extern __shared__ unsigned char cv_raw[];
   __shared__ CvBarriers bars;
   const int q0 = blockIdx.x * WG_PER, steps = min(WG_PER, p.patches - q0);
@@ -372,12 +411,26 @@ __global__ void __launch_bounds__(CV_NT) conv3x3_wgrad_tc(const __grid_constant_
   const int m = warp * 32 + lane;
   const int ci = ci0 + (wide ? m : m % p.KC), kyr = m / p.KC;
   const bool live = wide ? ci < p.Ci : kyr < 3;
+  const int tap0 = wide ? kxf : 3 * kyr, dtap = wide ? 3 : 1;
+  const unsigned trow = tmem + ((unsigned)(warp * 32) << 16);
+  unsigned redo = 0;  // groups of columns left to wgrad_redo
   if (wide || warp * 32 < 3 * p.KC)
     for (int j = 0; j < 3; ++j) {
-      const int tap = wide ? 3 * j + kxf : 3 * kyr + j;
+      const int tap = tap0 + dtap * j;
       for (int cb = 0; cb < p.NB && co0 + cb < p.Co; cb += 16) {
         float v[16];
-        cv_ld16(tmem + ((unsigned)(warp * 32) << 16) + j * p.NB + cb, v);
+        cv_ld16(trow + j * p.NB + cb, v);
+        if (p.ragged && ok) {
+          float s[8];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) s[i] = v[i] + v[i + 8];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) s[i] += s[i + 4];
+          if (__any_sync(0xffffffffu, live && isnan((s[0] + s[1]) + (s[2] + s[3])))) {
+            redo |= 1u << (4 * j + cb / 16);
+            continue;
+          }
+        }
         if (live)
 #pragma unroll
           for (int i = 0; i < 16; ++i)
@@ -387,6 +440,7 @@ __global__ void __launch_bounds__(CV_NT) conv3x3_wgrad_tc(const __grid_constant_
         __syncwarp();
       }
     }
+  if (redo) wgrad_redo(p, redo, trow, q0, steps, co0, tap0, dtap, ci, live);
   cv_end(bars, p.cols, ok, steps, p.stages);
 }
 
@@ -503,6 +557,9 @@ cudaError_t launch_conv3x3_wgrad(const void* x, const void* dy, float* dw, int N
   p.stage_bytes = (p.tx_bytes + (wide ? 0 : 5 * 8 * p.rowx) + 1023) / 1024 * 1024;
   const int blocks = p.cob * (wide ? 3 * ((Ci + 127) / 128) : Ci / p.KC);
   const int bytes = shared_bytes(p.stage_bytes, 2, p.cols, &p.stages);
+  p.ragged = W % CV_PX != 0 || H % CV_PY != 0;
+  p.x = (const bf16*)x;
+  p.dy = (const bf16*)dy;
   p.dw = dw;
   cudaError_t e = cudaFuncSetAttribute(conv3x3_wgrad_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, CV_SMEM_CTA);
   if (e != cudaSuccess) return e;  // before the maps, as above
