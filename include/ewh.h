@@ -389,7 +389,9 @@ ewh_status ewh_fma_rate(int precision, double* flops_per_second, void* cuda_stre
  * Conventions: activations NHWC, weights [Co][3][3][Ci]; tensors typed void*
  * hold bfloat16, float* hold FP32; all pointers are device pointers; the work
  * is enqueued on `stream` (NULL = legacy default stream) and nothing is
- * allocated.  Errors: EWH_EINVAL (bad sizes, message in ewh_last_error(NULL)),
+ * allocated.  The convolutions wait for their bulk-tensor copies on the device,
+ * each wait bounded by one second; a block whose copy does not arrive leaves NaN
+ * in its outputs (the calls do not synchronise, so no status can tell).  Errors: EWH_EINVAL (bad sizes, message in ewh_last_error(NULL)),
  * EWH_ECUDA. */
 
 /* y = conv3x3(x, w) + bias (zero padding, stride 1), BF16 tensor-core MMA with

@@ -786,8 +786,8 @@ __global__ void __launch_bounds__(P2_THREADS) sbp_stress2d(Geom g, Part2d cp, co
 
 // Leapfrog / filter update of one value, kd = -M^{-1} K u / irh in units of 1 / kts (dl, ac: delta^n and
 // the filter's sum in, the new ones out); the operator alone: un = -kd kts irh.  The value
-// meets kts, then irh: the product of these two, rounded, would change every wave's
-// frequency alike, and M^{-1} K u alone exceeds the field by 1 / (c dt^2).
+// meets kts, then irh: M^{-1} K u alone exceeds the field by 1 / (c dt^2), and the product of
+// the two constants would be one more rounding that every level of a node shares.
 template <typename T, int MODE, bool FORCED>
 __device__ __forceinline__ void pair_update(T kd, T kts, T irh, T fc, T fr, T w0, T wnew, T uv, T& dl, T& ac, T& un) {
   const T k = kd * kts;
